@@ -185,6 +185,7 @@ struct jslam_ctx {
     jslam_config cfg;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    int n_sm = 0;  // streaming multiprocessors of the device
     jslam_status status = JSLAM_OK;
 
     // constant tables
@@ -306,6 +307,54 @@ void fast_block(int c, int k, int tile_w, int tile_h, int *bx, int *by)
     *by = y;
 }
 
+// Pyramid strips of a level.
+int pyramid_strips(int W, int H, int rows) { return ((W + kPyrCols - 1) / kPyrCols) * ((H + rows - 1) / rows); }
+
+// Output rows of the strips of each level number of a launch over the images
+// `geo` describes (two each).  A strip computes six rows more than it writes,
+// so tall strips do the least work, but a launch with fewer strips than the
+// chip runs at once takes as long as one strip.  So: the fewest rows (in
+// fours, as the kernel's loop is unrolled) with which the launch's strips all
+// run at once, for launches too large for that the most.  Measured, rows 6 /
+// 10 / 18 / 34 / 58: one pair of 1241x376 (8 levels) 18.6 / 16.2 / 16.9 / 20.1
+// / 23.6 us (10 rows: 2560 strips of the 3344 that fit), one of 1920x1080 39 /
+// 32 / 30 / 27 / 30 us (34: 3330), 100 of 1241x376 720 / 537 / 426 / 360 / 337.
+// The cascaded pyramid launches each level number by itself.
+void pyramid_strip_rows(const std::vector<Geometry> &geo, bool cascade, int n_sm, int rows[kMaxLevels])
+{
+    for (int l0 = 0; l0 < kMaxLevels; l0 += cascade ? 1 : kMaxLevels) {
+        int r = kPyrMinRows;
+        for (; r < kPyrMaxRows; r += 4) {
+            long long strips = 0;
+            for (const Geometry &g : geo)
+                for (int l = l0; l < (cascade ? std::min(l0 + 1, g.levels) : g.levels); ++l)
+                    strips += 2 * pyramid_strips(g.W[l], g.H[l], r);
+            if (strips <= (long long)n_sm * kPyrWarpsPerSm) break;
+        }
+        for (int l = l0; l < (cascade ? l0 + 1 : kMaxLevels); ++l) rows[l] = r;
+    }
+}
+
+// How the pyramid kernel reads a resampled level's source columns: the taps
+// of the four columns of every word (columns past the level repeat its last)
+// within eight bytes, those of both halves of every word within eight bytes
+// each, or neither; and only where the strip's ring holds the source rows.  A window of eight bytes starts at its first tap or,
+// near the right edge, eight bytes before the row's end.
+int pyramid_mode_of(const uint32_t *tapx, int W, int src_W)
+{
+    int four = 0, two = 0;  // largest distance of a tap's second byte from the first tap
+    int range = 0;          // most source bytes of a strip
+    auto xa = [&](int x) { return (int)(tapx[std::min(std::max(x, 0), W - 1)] & 0xFFFFu); };
+    for (int x = 0; x < W; x += 4) {
+        four = std::max(four, std::min(xa(x + 3) + 1, src_W - 1) - xa(x));
+        for (int h = 0; h < 4; h += 2) two = std::max(two, std::min(xa(x + h + 1) + 1, src_W - 1) - xa(x + h));
+    }
+    for (int x0 = 0; x0 < W; x0 += kPyrCols)
+        range = std::max(range, xa(x0 + kPyrCols + 2) + 8 - std::min(xa(x0 - 4), src_W - 8));
+    const int stride = (range + 30) & ~15;
+    return four <= 7 && stride <= kPyrMaxOne ? kPyrOne : two <= 7 && stride <= kPyrMaxTwo ? kPyrTwo : kPyrBytes;
+}
+
 // Build (or reuse) the plan of a batch and upload it.
 jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
 {
@@ -407,10 +456,12 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     const size_t o_pyr = reserve(sizeof(int32_t) * (n_levels + 1));
     const size_t o_fast = reserve(sizeof(int32_t) * (n_levels + 1));
     const size_t o_seg = reserve(sizeof(int32_t) * (n_segs + 1));
+    int pyr_rows[kMaxLevels];
+    pyramid_strip_rows(geo, cfg.pyramid_mode == 1, ctx->n_sm, pyr_rows);
     size_t n_fast_tiles = 0, n_pyr_tiles = 0;
     for (int p = 0; p < n; ++p)
         for (int l = 0; l < geo[p].levels; ++l) {
-            n_pyr_tiles += 2 * (size_t)(((geo[p].W[l] + kPyrTW - 1) / kPyrTW) * ((geo[p].H[l] + kPyrTH - 1) / kPyrTH));
+            n_pyr_tiles += 2 * (size_t)pyramid_strips(geo[p].W[l], geo[p].H[l], pyr_rows[l]);
             int bx, by;
             fast_block(geo[p].c[l], k, ctx->tune.tile_w_px, ctx->tune.tile_h_px, &bx, &by);
             const int cx = (geo[p].W[l] + geo[p].c[l] - 1) / geo[p].c[l], cy = (geo[p].H[l] + geo[p].c[l] - 1) / geo[p].c[l];
@@ -530,6 +581,8 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 const double tap_s = cascade ? zeta_pow(jobs[p].scale, 1) : sc;
                 for (int x = 0; x < L.W; ++x) tx[x] = bilinear_tap(x, tap_s, L.src_W);
                 for (int y = 0; y < L.H; ++y) tx[L.W + y] = bilinear_tap(y, tap_s, L.src_H);
+                L.pyr_rows = pyr_rows[l];
+                L.pyr_mode = l == 0 ? kPyrCopy : pyramid_mode_of(tx, L.W, L.src_W);
                 t_off += align_up((size_t)(L.W + L.H) * 4, 16);
                 uint16_t *px = reinterpret_cast<uint16_t *>(host.data() + t_off);
                 L.projx = reinterpret_cast<const uint16_t *>(dplan + t_off);
@@ -561,7 +614,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 for (int r = 0; r < L.cells_y; ++r) seg_level[seg + r] = li;
                 seg += L.cells_y;
                 pyr_base[li] = pyr;
-                const int ptiles = ((L.W + kPyrTW - 1) / kPyrTW) * ((L.H + kPyrTH - 1) / kPyrTH);
+                const int ptiles = pyramid_strips(L.W, L.H, L.pyr_rows);
                 for (int q = 0; q < ptiles; ++q) ptile_level[pyr + q] = li;
                 pyr += ptiles;
                 fast_base[li] = fast;
@@ -645,8 +698,10 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
         std::copy(sorted.begin(), sorted.end(), trec);
     }
 
-    // pyramid tiles by level number (the cascaded pyramid launches level
-    // number n once level n - 1 of every image is complete)
+    // pyramid strips by level number: the cascaded pyramid launches level
+    // number n once level n - 1 of every image is complete; in one launch the
+    // strips that run together then mostly execute the same code (strips of
+    // one image's levels side by side wait for instructions)
     int pass_first[kMaxLevels + 1] = {};
     {
         auto porder = reinterpret_cast<int32_t *>(host.data() + o_porder);
@@ -828,6 +883,7 @@ jslam_status jslam_create(jslam_ctx **out, const jslam_config *cfg)
 
     jslam_status st = JSLAM_OK;
     cudaError_t e = cudaSetDevice(c.device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, c.device);
     if (e == cudaSuccess) {
         if (c.cuda_stream) {
             ctx->stream = static_cast<cudaStream_t>(c.cuda_stream);

@@ -26,8 +26,18 @@ constexpr int kPatPitch = 32;    // row pitch of the staged 27 x 27 BRIEF patch 
 constexpr int kMaxSegment = 4096;  // candidate slots per (level, cell row)
 constexpr int kMaxImages = 256;    // images per batch (two per stereo pair)
 
-// Pyramid tile (outputs per CTA) and thread count.
-constexpr int kPyrTW = 128, kPyrTH = 32, kPyrThreads = 256;
+// Pyramid strip: output columns per warp (30 lanes x 4 pixels), and how a
+// lane reads its source columns (see k_pyramid).
+constexpr int kPyrCols = 120, kPyrMinRows = 6, kPyrMaxRows = 58;
+constexpr int kPyrWarpsPerSm = 22;  // strips that run on an SM at once
+// The ring of a strip's source rows: two source rows per row, for the two
+// rows in use and the rows ahead that are being copied, and the source row
+// before them; rows of up to 16 (kPyrOne) and 32 (kPyrTwo) 16-byte units.
+constexpr int kPyrRing = 6656, kPyrAhead = 6, kPyrAheadTwo = 4;
+constexpr int kPyrMaxOne = 256, kPyrMaxTwo = 512;
+static_assert((2 * (kPyrAhead + 2) + 1) * kPyrMaxOne <= kPyrRing, "ring");
+static_assert((2 * (kPyrAheadTwo + 2) + 1) * kPyrMaxTwo <= kPyrRing, "ring");
+enum { kPyrCopy = 0, kPyrOne = 1, kPyrTwo = 2, kPyrBytes = 3 };
 // Detection tile: at most this many pixels a side (host picks cells per CTA).
 constexpr int kFastMaxTile = 128, kFastThreads = 256;
 
@@ -70,6 +80,8 @@ struct LevelDesc {
     // cascaded pyramid the raw level n - 1 (taps then use one factor zeta)
     const uint8_t *src;
     int32_t src_W, src_H, src_pitch;
+    int32_t pyr_mode;        // how the pyramid kernel reads the source columns (kPyr...)
+    int32_t pyr_rows;        // output rows of its strips
     int32_t W, H, pitch;     // pitch of raw: width rounded up to 128
     int32_t blur_pitch;
     int32_t c, cells_x, cells_y;
@@ -166,16 +178,16 @@ struct Batch {
     const LevelDesc *levels;
     const PairDesc *pairs;
     const int32_t *pyr_tile_base;   // n_levels + 1
-    const int32_t *pyr_tile_level;  // level index of each pyramid tile
-    const int32_t *pyr_order;       // pyramid tiles ordered by level number (cascaded pyramid)
+    const int32_t *pyr_tile_level;  // level index of each pyramid strip
+    const int32_t *pyr_order;       // pyramid strips ordered by level number (cascaded pyramid)
     int32_t pyr_pass_first[kMaxLevels + 1];  // first entry of pyr_order of each level number
-    int32_t pyr_pass;               // -1: one launch over every tile; n: the tiles of level number n
+    int32_t pyr_pass;               // -1: one launch over every strip; n: the strips of level number n
     const int32_t *fast_tile_base;  // n_levels + 1
     const int32_t *fast_tile_level; // level index of each detection tile
     const int32_t *seg_level;       // level index of each segment
     int32_t n_images, n_levels, n_pairs, n_segments;
     int32_t max_segment;            // largest segment (cells_x x k slots) of the batch
-    int32_t pyr_tiles, fast_tiles;
+    int32_t pyr_tiles, fast_tiles;  // pyramid strips, detection tiles
     int32_t max_capacity;           // largest keypoint capacity of any image
     int32_t fast_smem;              // dynamic shared memory of the detection kernel
     int32_t fast_max_box, fast_max_px, fast_max_cells;  // its tile layout maxima

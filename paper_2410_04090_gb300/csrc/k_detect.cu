@@ -1,11 +1,6 @@
-// Detection stage: image pyramid with Gaussian filtering, then FAST with
-// Bounded Rectification, per-cell culling and the scatter half of PFA.
+// Detection stage: FAST with Bounded Rectification, per-cell culling and the
+// scatter half of PFA.
 //
-// k_pyramid   one CTA per 128x32 output tile of any (image, level): resamples
-//             the level from level 0 (bilinear, Q8 taps from host tables),
-//             writes it (level 0: an aligned copy of the input), and writes its
-//             7-tap Gaussian (Sec. III, streamlined multiscale detection and
-//             extraction: Gaussian filtering before ORB).
 // k_fast_cull persistent CTAs over blocks of culling cells of any (image,
 //             level): stage the raw tile plus its halo in shared memory (TMA),
 //             evaluate the 16-pixel ring of every pixel (Sec. II-A, Eq. 1 labels, Eq. 3
@@ -26,256 +21,6 @@
 #include "ring_response.cuh"
 
 namespace jslam {
-
-__constant__ int32_t c_blur_w[7];
-// The same weights as bytes for the 2-way dot products of the horizontal
-// pass: {0, w0, w1, w2}, {w3, w4, w5, w6}, {w0, w1, w2, w3}, {w4, w5, w6, 0}
-// (byte 0 first; every weight is below 256).
-__constant__ uint32_t c_blur_pk[4];
-
-cudaError_t set_blur_weights(const int32_t w[7])
-{
-    cudaError_t e = cudaMemcpyToSymbol(c_blur_w, w, sizeof(int32_t) * 7);
-    if (e != cudaSuccess) return e;
-    const auto B = [](int b0, int b1, int b2, int b3) {
-        return (uint32_t)b0 | ((uint32_t)b1 << 8) | ((uint32_t)b2 << 16) | ((uint32_t)b3 << 24);
-    };
-    const uint32_t pk[4] = { B(0, w[0], w[1], w[2]), B(w[3], w[4], w[5], w[6]), B(w[0], w[1], w[2], w[3]),
-                             B(w[4], w[5], w[6], 0) };
-    return cudaMemcpyToSymbol(c_blur_pk, pk, sizeof(pk));
-}
-
-// ---------------------------------------------------------------- pyramid
-//
-// Per 128x32 output tile: the raw level over the tile plus a halo (3 rows, 4
-// columns) is built in shared memory -- level 0 is copied from the input,
-// deeper levels are resampled from level 0 separably and exactly: every
-// needed source row is interpolated horizontally once ((256-a) p0 + a p1,
-// exact in 16 bits), then pairs of those rows vertically with rounding.
-// The raw interior is written to the level buffer (level 0 included: an
-// aligned copy of the input).  The 7-tap Gaussian runs vertically first on
-// bytes in 16-bit lanes (two pixels per multiply; the symmetric taps need 3
-// adds and 4 multiplies), then horizontally on the 16-bit column sums.
-
-constexpr int kPyrCols = kPyrTW + 8;         // raw tile columns: x in [x0 - 4, x0 + 132)
-constexpr int kPyrRows = kPyrTH + 6;         // raw tile rows: y in [y0 - 3, y0 + 35)
-constexpr int kPyrSrcRows = 2 * kPyrRows;    // level-0 rows interpolated per tile, at most
-
-__device__ __forceinline__ uint32_t blur7_sym(uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t a4,
-                                              uint32_t a5, uint32_t a6)
-{
-    return c_blur_w[0] * (a0 + a6) + c_blur_w[1] * (a1 + a5) + c_blur_w[2] * (a2 + a4) + c_blur_w[3] * a3;
-}
-
-__global__ void __launch_bounds__(kPyrThreads) k_pyramid(Batch b)
-{
-    __shared__ __align__(16) uint8_t raw[kPyrRows][kPyrCols];
-    __shared__ __align__(16) uint16_t V[kPyrTH][kPyrCols];
-    __shared__ __align__(16) uint16_t Hs[kPyrSrcRows][kPyrCols];
-    __shared__ uint32_t tx[kPyrCols];
-    __shared__ int src_row[kPyrSrcRows];
-    __shared__ uint8_t ia[kPyrRows], ib[kPyrRows];
-    __shared__ uint16_t wb[kPyrRows];
-    __shared__ int s_ya[kPyrRows];
-    __shared__ int nsrc;
-
-    const int tile = b.pyr_pass < 0 ? (int)blockIdx.x : __ldg(b.pyr_order + b.pyr_pass_first[b.pyr_pass] + blockIdx.x);
-    const int li = __ldg(b.pyr_tile_level + tile);
-    const LevelDesc &L = b.levels[li];
-    const ImageDesc &I = b.images[L.image];
-    const int t = tile - b.pyr_tile_base[li];
-    const int tiles_x = (L.W + kPyrTW - 1) / kPyrTW;
-    const int x0 = (t % tiles_x) * kPyrTW, y0 = (t / tiles_x) * kPyrTH;
-    // level 0 reads the input; deeper levels resample the input, or in the
-    // cascaded pyramid the level above (complete: an earlier launch)
-    const uint8_t *L0 = L.src ? L.src : b.in.ptr[L.image];
-    const int W0 = L.src ? L.src_W : I.W0, H0 = L.src ? L.src_H : I.H0;
-    const int pitch0 = L.src ? L.src_pitch : b.in.pitch[L.image];
-    const int W = L.W, H = L.H;
-    constexpr int WPR = kPyrCols / 4;
-
-    if (L.level == 0) {
-        for (int i = threadIdx.x; i < kPyrRows * WPR; i += kPyrThreads) {
-            const int r = i / WPR, w = i - r * WPR;
-            const uint8_t *row = L0 + (size_t)min(max(y0 - 3 + r, 0), H - 1) * pitch0;
-            const int gx = x0 - 4 + 4 * w;
-            uint32_t v;
-            if (gx >= 0 && gx + 3 < W) {
-                // the two aligned words holding bytes gx .. gx + 3 (each holds
-                // at least one byte of the row, so neither leaves the buffer)
-                const uintptr_t a = reinterpret_cast<uintptr_t>(row + gx);
-                const uint32_t *p = reinterpret_cast<const uint32_t *>(a & ~static_cast<uintptr_t>(3));
-                const uint32_t sh = (uint32_t)(a & 3u) * 8u;
-                v = sh ? __funnelshift_r(__ldg(p), __ldg(p + 1), sh) : __ldg(p);
-            } else {
-                v = 0;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) v |= (uint32_t)__ldg(row + min(max(gx + q, 0), W - 1)) << (8 * q);
-            }
-            *reinterpret_cast<uint32_t *>(&raw[r][4 * w]) = v;
-        }
-    } else {
-        for (int c = threadIdx.x; c < kPyrCols; c += kPyrThreads)
-            tx[c] = __ldg(L.tapx + min(max(x0 - 4 + c, 0), W - 1));
-        if (threadIdx.x < kPyrRows) {
-            const uint32_t ty = __ldg(L.tapy + min(max(y0 - 3 + (int)threadIdx.x, 0), H - 1));
-            s_ya[threadIdx.x] = ty & 0xFFFF;
-            wb[threadIdx.x] = (uint16_t)(ty >> 16);
-        }
-        __syncthreads();
-        // level-0 rows needed by the tile's raw rows: a contiguous range when
-        // it is short enough, else two rows per raw row
-        const int first = s_ya[0], last = min(s_ya[kPyrRows - 1] + 1, H0 - 1);
-        const bool contiguous = last - first + 1 <= kPyrSrcRows;
-        if (threadIdx.x < kPyrRows) {
-            const int r = threadIdx.x, ya = s_ya[r], yb = min(ya + 1, H0 - 1);
-            ia[r] = (uint8_t)(contiguous ? ya - first : 2 * r);
-            ib[r] = (uint8_t)(contiguous ? yb - first : 2 * r + 1);
-        }
-        const int nrows = contiguous ? last - first + 1 : kPyrSrcRows;
-        for (int j = threadIdx.x; j < nrows; j += kPyrThreads)
-            src_row[j] = contiguous ? first + j : ((j & 1) ? min(s_ya[j >> 1] + 1, H0 - 1) : s_ya[j >> 1]);
-        if (threadIdx.x == 0) nsrc = nrows;
-        __syncthreads();
-        const int ns = nsrc;
-        // horizontal interpolation: a thread owns 4 adjacent columns, keeps
-        // their taps in registers and walks the source rows
-        constexpr int kQuads = kPyrCols / 4, kRowSlots = kPyrThreads / kQuads;
-        const int q = threadIdx.x % kQuads, slot = threadIdx.x / kQuads;
-        if (slot < kRowSlots) {
-            int xa[4], xb[4];
-            uint32_t wa[4], wbx[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t tp = tx[4 * q + k];
-                xa[k] = tp & 0xFFFF;
-                xb[k] = min(xa[k] + 1, W0 - 1);
-                wbx[k] = tp >> 16;
-                wa[k] = 256u - wbx[k];
-            }
-            for (int j = slot; j < ns; j += kRowSlots) {
-                // 32-bit offsets from the image's base (images are below 4 GB)
-                const uint32_t ro = (uint32_t)src_row[j] * (uint32_t)pitch0;
-                uint32_t h[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    h[k] = wa[k] * __ldg(L0 + (ro + (uint32_t)xa[k])) + wbx[k] * __ldg(L0 + (ro + (uint32_t)xb[k]));
-                *reinterpret_cast<uint2 *>(&Hs[j][4 * q]) = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
-            }
-        }
-        __syncthreads();
-        // vertical interpolation, 4 columns per thread (16-bit taps read as words)
-        for (int i = threadIdx.x; i < kPyrRows * (kPyrCols / 4); i += kPyrThreads) {
-            const int r = i / (kPyrCols / 4), q = i - r * (kPyrCols / 4);
-            const uint32_t w = wb[r], w0 = 256u - w;
-            const uint2 ha = *reinterpret_cast<const uint2 *>(&Hs[ia[r]][4 * q]);
-            const uint2 hb = *reinterpret_cast<const uint2 *>(&Hs[ib[r]][4 * q]);
-            // rounded sums below 2^24: the result is byte 2 of each, packed by byte permutes
-            const uint32_t v0 = w0 * (ha.x & 0xFFFFu) + w * (hb.x & 0xFFFFu) + 32768u;
-            const uint32_t v1 = w0 * (ha.x >> 16) + w * (hb.x >> 16) + 32768u;
-            const uint32_t v2 = w0 * (ha.y & 0xFFFFu) + w * (hb.y & 0xFFFFu) + 32768u;
-            const uint32_t v3 = w0 * (ha.y >> 16) + w * (hb.y >> 16) + 32768u;
-            *reinterpret_cast<uint32_t *>(&raw[r][4 * q]) =
-                __byte_perm(__byte_perm(v0, v1, 0x0062), __byte_perm(v2, v3, 0x0062), 0x5410);
-        }
-    }
-    __syncthreads();
-
-    // raw interior -> level buffer (whole words; the row pitch covers the tile)
-    for (int i = threadIdx.x; i < kPyrTH * (kPyrTW / 4); i += kPyrThreads) {
-        const int r = i / (kPyrTW / 4), w = i - r * (kPyrTW / 4);
-        const int gy = y0 + r, gx = x0 + 4 * w;
-        if (gy < H && gx < W)
-            *reinterpret_cast<uint32_t *>(L.raw_w + (size_t)gy * L.pitch + gx) =
-                *reinterpret_cast<const uint32_t *>(&raw[r + 3][4 * w + 4]);
-    }
-    // vertical 7-tap sums, two pixels per 32-bit lane pair: a thread owns one
-    // word column and slides a 7-row window down a run of rows
-    {
-        constexpr int kSegs = kPyrThreads / WPR, kRun = (kPyrTH + kSegs - 1) / kSegs;
-        const int w = threadIdx.x % WPR, seg = threadIdx.x / WPR;
-        if (seg < kSegs) {
-            const int r0 = seg * kRun;
-            uint32_t e[7], o[7];
-#pragma unroll
-            for (int j = 0; j < 6; ++j) {
-                const uint32_t x = *reinterpret_cast<const uint32_t *>(&raw[min(r0 + j, kPyrRows - 1)][4 * w]);
-                e[j] = x & 0x00FF00FFu;
-                o[j] = (x >> 8) & 0x00FF00FFu;
-            }
-#pragma unroll
-            for (int k = 0; k < kRun; ++k) {
-                const int r = r0 + k;
-                if (r < kPyrTH) {
-                    const uint32_t x = *reinterpret_cast<const uint32_t *>(&raw[r + 6][4 * w]);
-                    e[6] = x & 0x00FF00FFu;
-                    o[6] = (x >> 8) & 0x00FF00FFu;
-                    const uint32_t se = blur7_sym(e[0], e[1], e[2], e[3], e[4], e[5], e[6]);
-                    const uint32_t so = blur7_sym(o[0], o[1], o[2], o[3], o[4], o[5], o[6]);
-                    *reinterpret_cast<uint2 *>(&V[r][4 * w]) =
-                        make_uint2(__byte_perm(se, so, 0x5410), __byte_perm(se, so, 0x7632));
-                }
-#pragma unroll
-                for (int j = 0; j < 6; ++j) { e[j] = e[j + 1]; o[j] = o[j + 1]; }
-            }
-        }
-    }
-    __syncthreads();
-    // horizontal 7-tap on the column sums: a thread owns a row and a run of
-    // 4 quads (16 output pixels).  The 16-bit sums sit two to a word (word i:
-    // columns 2i, 2i + 1 of the run), so each output is four 2-way byte dot
-    // products over aligned words, with the weights packed for its parity
-    // (the same integer sum as the 7 products; one rounding at the end).
-    {
-        constexpr int kQuadRun = 4, kRunsPerRow = (kPyrTW / 4) / kQuadRun;
-        static_assert(kPyrTH * kRunsPerRow == kPyrThreads, "one run per thread");
-        const int r = threadIdx.x / kRunsPerRow, q0 = (threadIdx.x % kRunsPerRow) * kQuadRun;
-        const int gy = y0 + r;
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(&V[r][4 * q0]);
-        const uint32_t A = c_blur_pk[0], Bw = c_blur_pk[1], Cw = c_blur_pk[2], Dw = c_blur_pk[3];
-        uint32_t u[2 * kQuadRun + 4];
-#pragma unroll
-        for (int j = 0; j < 2 * kQuadRun + 4; ++j) u[j] = src[j];
-#pragma unroll
-        for (int k = 0; k < kQuadRun; ++k) {
-            // output m of the quad reads columns 4 k + m + 1 .. 4 k + m + 7
-            const uint32_t *w = u + 2 * k;
-            // words i .. i + 3 against the weight words P (first two) and Q (last
-            // two); the rounding term starts each sum, the sums stay below 2^24,
-            // so each result is byte 2 of its sum, packed by byte permutes
-            const auto dot7 = [&](int i, uint32_t P, uint32_t Q) {
-                const uint32_t lo = __dp2a_hi(w[i + 1], P, __dp2a_lo(w[i], P, 32768u));
-                return __dp2a_hi(w[i + 3], Q, __dp2a_lo(w[i + 2], Q, lo));
-            };
-            const uint32_t s0 = dot7(0, A, Bw), s1 = dot7(1, Cw, Dw), s2 = dot7(1, A, Bw), s3 = dot7(2, Cw, Dw);
-            const uint32_t out = __byte_perm(__byte_perm(s0, s1, 0x0062), __byte_perm(s2, s3, 0x0062), 0x5410);
-            const int gx = x0 + 4 * (q0 + k);
-            if (gy < H && gx < W) *reinterpret_cast<uint32_t *>(L.blur + (size_t)gy * L.blur_pitch + gx) = out;
-        }
-    }
-}
-
-const void *pyramid_kernel() { return reinterpret_cast<const void *>(k_pyramid); }
-
-cudaError_t launch_pyramid(const Batch &b, cudaStream_t stream)
-{
-    if (b.pyr_tiles == 0) return cudaSuccess;
-    if (b.pyr_pass < 0) {
-        k_pyramid<<<b.pyr_tiles, kPyrThreads, 0, stream>>>(b);
-        return cudaGetLastError();
-    }
-    // cascaded: level number n after n - 1, each launch over every image
-    for (int n = 0; n < kMaxLevels; ++n) {
-        const int tiles = b.pyr_pass_first[n + 1] - b.pyr_pass_first[n];
-        if (tiles == 0) continue;
-        Batch bn = b;
-        bn.pyr_pass = n;
-        k_pyramid<<<tiles, kPyrThreads, 0, stream>>>(bn);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
 
 // ---------------------------------------------------------------- FAST + FC
 //
@@ -370,6 +115,26 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// Whether the mbarrier phase `parity` is complete (waits a bounded time itself).
+__device__ __forceinline__ bool try_tile(uint64_t *bar, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    return done != 0;
+}
+
+// Wait for the mbarrier phase `parity`, giving up after about a second.
+__device__ __forceinline__ bool wait_tile(uint64_t *bar, uint32_t parity)
+{
+    if (try_tile(bar, parity)) return true;
+    const long long start = clock64();
+    while (clock64() - start <= (1ll << 31))
+        if (try_tile(bar, parity)) return true;
+    return false;
+}
+
 // Position of a detection tile: its cells, pixels and the TMA box origin.
 struct TileGeom {
     int li, ccx0, ccy0, ncx, ncy, x0, y0, tw, th, xs, ys, delta;
@@ -413,20 +178,6 @@ __device__ __forceinline__ void issue_tile(const Batch &b, int t, uint8_t *buf, 
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(smem_u32(buf)), "l"(reinterpret_cast<uint64_t>(L.tmap)), "r"(G.xs), "r"(G.ys), "r"(smem_u32(bar))
         : "memory");
-}
-
-// Wait for the mbarrier phase `parity`, giving up after about a second.
-__device__ __forceinline__ bool wait_tile(uint64_t *bar, uint32_t parity)
-{
-    const long long start = clock64();
-    for (;;) {
-        uint32_t done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-        if (done) return true;
-        if (clock64() - start > (1ll << 31)) return false;
-    }
 }
 
 // Failure-detection self-test: a tile wait on an mbarrier that nothing
