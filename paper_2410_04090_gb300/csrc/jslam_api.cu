@@ -440,11 +440,11 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
         if ((e = ctx->skipbuf.ensure(skip_bytes + 256, false, nullptr)) != cudaSuccess) return fail(ctx, e);
     }
     size_t skip_off = 0;
-    const size_t slot_words = (size_t)n_slots + 64;
+    const size_t slot_words = align_up((size_t)n_slots + 64, 4);  // slot_info holds 16-byte entries
     const size_t seg_words = (size_t)n_segs + 64;
     size_t row_words = 64;  // row index of each image's canonical list: levels x (H0 + 1)
     for (int p = 0; p < n; ++p) row_words += 2 * (size_t)geo[p].levels * (geo[p].H[0] + 1);
-    const size_t scratch_bytes = slot_words * 4 * 4 + seg_words * 4 * 2 + row_words * 4;
+    const size_t scratch_bytes = slot_words * 4 * 8 + seg_words * 4 * 2 + row_words * 4;
     if ((e = ctx->scratch.ensure(scratch_bytes, false, nullptr)) != cudaSuccess) return fail(ctx, e);
 
     // Host tables: [images][levels][pairs][pyr base][fast base][seg level][taps/proj ...]
@@ -455,7 +455,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     const size_t o_pairs = reserve(sizeof(PairDesc) * n);
     const size_t o_pyr = reserve(sizeof(int32_t) * (n_levels + 1));
     const size_t o_fast = reserve(sizeof(int32_t) * (n_levels + 1));
-    const size_t o_seg = reserve(sizeof(int32_t) * (n_segs + 1));
+    const size_t o_seg = reserve(sizeof(SegRec) * (size_t)(n_segs + 1));
     int pyr_rows[kMaxLevels];
     pyramid_strip_rows(geo, cfg.pyramid_mode == 1, ctx->n_sm, pyr_rows);
     size_t n_fast_tiles = 0, n_pyr_tiles = 0;
@@ -483,7 +483,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     auto pairs = reinterpret_cast<PairDesc *>(host.data() + o_pairs);
     auto pyr_base = reinterpret_cast<int32_t *>(host.data() + o_pyr);
     auto fast_base = reinterpret_cast<int32_t *>(host.data() + o_fast);
-    auto seg_level = reinterpret_cast<int32_t *>(host.data() + o_seg);
+    auto seg_rec = reinterpret_cast<SegRec *>(host.data() + o_seg);
     auto ftile_level = reinterpret_cast<int32_t *>(host.data() + o_ftl);
     auto ptile_level = reinterpret_cast<int32_t *>(host.data() + o_ptl);
     size_t t_off = o_tables, lvl_off = 0, map_off = 0, stage_off = 0, row_off = 0;
@@ -526,7 +526,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 skip_off += align_up((size_t)I.skip_cells_x * I.skip_cells_y, 256);
             }
             I.level_start = reinterpret_cast<int32_t *>(dplan + o_lstart) + img * (kMaxLevels + 1);
-            I.row_first = ctx->scratch.as<int32_t>(4 * (slot_words * 4 + seg_words * 2) + row_off);
+            I.row_first = ctx->scratch.as<int32_t>(4 * (slot_words * 8 + seg_words * 2) + row_off);
             row_off += 4 * (size_t)g.levels * (g.H[0] + 1);
             const SideLayout &sl = pl.side[s];
             I.out.capacity = pl.capacity;
@@ -610,8 +610,16 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 }
                 L.slot_base = slot;
                 L.seg_base = seg;
+                for (int r = 0; r < L.cells_y; ++r) {
+                    SegRec &R = seg_rec[seg + r];
+                    R.projx = L.projx; R.projy = L.projy; R.map = I.map;
+                    R.m = L.cells_x * k;
+                    R.slot = slot + r * R.m;
+                    R.c = L.c; R.y0 = r * L.c;
+                    R.cdiv = L.c == 1 ? 0u : (uint32_t)(((1ull << 32) + L.c - 1) / (uint64_t)L.c);
+                    R.W0 = I.W0; R.H0 = I.H0; R.level = l;
+                }
                 slot += L.cells_x * L.cells_y * k;
-                for (int r = 0; r < L.cells_y; ++r) seg_level[seg + r] = li;
                 seg += L.cells_y;
                 pyr_base[li] = pyr;
                 const int ptiles = pyramid_strips(L.W, L.H, L.pyr_rows);
@@ -636,7 +644,6 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     }
     pyr_base[n_levels] = pyr;
     fast_base[n_levels] = fast;
-    seg_level[n_segs] = n_levels - 1;
 
     // detection tile records (the device-side tile geometry, evaluated here)
     auto trec = reinterpret_cast<TileRec *>(host.data() + o_trec);
@@ -725,7 +732,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     b.pyr_pass = cfg.pyramid_mode == 1 ? 0 : -1;
     for (int d = 0; d <= kMaxLevels; ++d) b.pyr_pass_first[d] = pass_first[d];
     b.fast_tile_base = reinterpret_cast<const int32_t *>(dplan + o_fast);
-    b.seg_level = reinterpret_cast<const int32_t *>(dplan + o_seg);
+    b.seg_rec = reinterpret_cast<const SegRec *>(dplan + o_seg);
     b.fast_tile_level = reinterpret_cast<const int32_t *>(dplan + o_ftl);
     b.tile_rec = reinterpret_cast<const TileRec *>(dplan + o_trec);
     b.n_images = n_img; b.n_levels = n_levels; b.n_pairs = n; b.n_segments = n_segs;
@@ -742,11 +749,14 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     b.skip_max_cells = skip_max_cells;
     uint32_t *sw = ctx->scratch.as<uint32_t>();
     b.slots = sw;
-    b.slot_k = sw + slot_words;
-    b.slot_rank = reinterpret_cast<int32_t *>(sw + 2 * slot_words);
-    b.canon = reinterpret_cast<int32_t *>(sw + 3 * slot_words);
-    b.seg_count = reinterpret_cast<int32_t *>(sw + 4 * slot_words);
-    b.seg_off = reinterpret_cast<int32_t *>(sw + 4 * slot_words + seg_words);
+    b.canon_prio = sw + slot_words;
+    b.canon_pos = reinterpret_cast<uint2 *>(sw + 2 * slot_words);
+    b.slot_info = reinterpret_cast<uint4 *>(sw + 4 * slot_words);
+    b.seg_count = reinterpret_cast<int32_t *>(sw + 8 * slot_words);
+    b.seg_off = reinterpret_cast<int32_t *>(sw + 8 * slot_words + seg_words);
+    b.n_sm = ctx->n_sm;
+    b.max_slots = 0;
+    for (int i = 0; i < n_img; ++i) b.max_slots = std::max(b.max_slots, images[i].slot_count);
     b.pattern = ctx->d_pattern;
     b.pattern_off = ctx->d_pattern_off;
     b.bin_cos = ctx->d_cos;

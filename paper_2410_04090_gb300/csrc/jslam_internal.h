@@ -52,7 +52,7 @@ constexpr int kSkipC = 16;                 // channels of the learned cell-skip 
 constexpr int kSkipTileW = 26, kSkipTileH = 12;  // its logits per CTA (grid pitch 26 + 6 = 32)
 constexpr int kRefineMaxW = 10, kRefineMaxL = 7;  // correlation window half-size and search radius limits
 constexpr int kNmsThreads = 128;
-constexpr int kFinThreads = 1024;
+constexpr int kFinThreads = 512;
 
 // Device error bits (OR-ed into the context's error word).
 constexpr uint32_t kErrSegment = 1u << 0;  // a segment was larger than kMaxSegment
@@ -173,6 +173,19 @@ struct __align__(16) TileRec {
 };
 static_assert(sizeof(TileRec) % 16 == 0, "bulk copies move multiples of 16 bytes");
 
+// One segment (cell row of a level): where its candidate slots lie and what
+// turns a slot into coordinates and score-map entries.
+struct __align__(16) SegRec {
+    const uint16_t *projx, *projy;
+    uint32_t *map;
+    int32_t slot, m;         // first slot, slots (cells_x x k)
+    int32_t c, y0;           // cell size, first row
+    uint32_t cdiv;           // ceil(2^32 / c); 0 for c = 1
+    int32_t W0, H0, level;
+};
+// Rank of a slot that is no survivor (SlotInfo's w): no corner, suppressed.
+constexpr int kSlotEmpty = -2, kSlotSuppressed = -1;
+
 struct Batch {
     const ImageDesc *images;
     const LevelDesc *levels;
@@ -184,7 +197,7 @@ struct Batch {
     int32_t pyr_pass;               // -1: one launch over every strip; n: the strips of level number n
     const int32_t *fast_tile_base;  // n_levels + 1
     const int32_t *fast_tile_level; // level index of each detection tile
-    const int32_t *seg_level;       // level index of each segment
+    const SegRec *seg_rec;          // one per segment
     int32_t n_images, n_levels, n_pairs, n_segments;
     int32_t max_segment;            // largest segment (cells_x x k slots) of the batch
     int32_t pyr_tiles, fast_tiles;  // pyramid strips, detection tiles
@@ -196,11 +209,13 @@ struct Batch {
     const TileRec *tile_rec;        // one per detection tile
     const uint32_t *corner_lut;     // bit m: P_min <= longest circular run of m <= P_max
     uint32_t *slots;                // candidate keys per slot
-    uint32_t *slot_k;               // PFA scores seen by each slot
-    int32_t *slot_rank;             // rank within its segment, -1 if suppressed
+    uint4 *slot_info;               // per slot: position, X | Y << 16, cap priority, rank in its segment
     int32_t *seg_count;             // survivors per segment
     int32_t *seg_off;               // exclusive prefix of seg_count per image
-    int32_t *canon;                 // slot of each canonical position
+    uint32_t *canon_prio;           // cap priority of each canonical position
+    uint2 *canon_pos;               // its x | y << 13 | level << 26, X | Y << 16
+    int32_t max_slots;              // most candidate slots of an image
+    int32_t n_sm;                   // streaming multiprocessors of the device
     const int8_t *pattern;          // kBins x kPairs x 4
     const uint32_t *pattern_off;    // kBins x kPairs: int16 patch offsets of p | of q << 16 (pitch kPatPitch)
     const double *bin_cos, *bin_sin;

@@ -8,30 +8,45 @@
 //                 filled by the detection kernel, and is suppressed when a
 //                 neighbour dominates it (sparse NMS: only occupied pixels are
 //                 looked at).  Survivors are ranked by (y, x) inside the
-//                 segment; segments of one level are already in y order.
-// k_pfa_finalize  one CTA per image: prefix-sums the segment counts into
-//                 canonical positions (level, y, x), clears the score map
+//                 segment; segments of one level are already in y order.  A
+//                 slot's coordinates, priority and rank go to the next kernel
+//                 as one 16-byte record.
+// k_pfa_finalize  a cluster of CTAs per image: prefix-sums the segment counts
+//                 into canonical positions (level, y, x), clears the score map
 //                 entries it used, applies the keypoint cap by a radix select
 //                 on (K_l, K_r, response) with canonical order breaking ties,
-//                 and writes the compacted keypoint list.
+//                 and writes the compacted keypoint list and its row index.
 #include "jslam_internal.h"
 
 namespace jslam {
 
-struct SlotPos {
-    int x, y, r;
-};
-
-__device__ __forceinline__ SlotPos decode_slot(uint32_t key, int rel, int cells_x, int c, int k)
+// Candidate i of a segment with key `key`: its level coordinates, packed x |
+// y << 13 | level << 26, and response (the key's upper half).
+__device__ __forceinline__ uint32_t slot_pos(const SegRec &R, uint32_t key, int i, int k)
 {
-    const int cell = rel / k;
-    const int cy = cell / cells_x, cx = cell - cy * cells_x;
-    const int inidx = 0xFFFF - (int)(key & 0xFFFFu);
-    SlotPos p;
-    p.x = cx * c + inidx % c;
-    p.y = cy * c + inidx / c;
-    p.r = (int)(key >> 16);
-    return p;
+    const uint32_t inidx = 0xFFFFu - (key & 0xFFFFu);
+    const uint32_t row = R.cdiv ? __umulhi(inidx, R.cdiv) : inidx;  // inidx / c (cdiv = ceil(2^32 / c), 0 for c = 1)
+    const uint32_t x = (uint32_t)(k == 1 ? i : i / k) * (uint32_t)R.c + (inidx - row * (uint32_t)R.c);
+    return x | (((uint32_t)R.y0 + row) << 13) | ((uint32_t)R.level << 26);
+}
+__device__ __forceinline__ uint32_t pos_x(uint32_t p) { return p & 0x1FFFu; }
+__device__ __forceinline__ uint32_t pos_y(uint32_t p) { return (p >> 13) & 0x1FFFu; }
+// Order of a segment's corners by (y, x): the position without its level, rows first.
+__device__ __forceinline__ uint32_t pos_order(uint32_t p) { return (pos_y(p) << 13) | pos_x(p); }
+
+// Whether a neighbour's packed (K_l, K_r) suppresses a corner's.
+__device__ __forceinline__ bool dominates(uint32_t n, uint32_t own, int rule)
+{
+    const uint32_t ql = n >> 16, qr = n & 0xFFFFu, kl = own >> 16, kr = own & 0xFFFFu;
+    return rule == 0 ? (ql > kl && qr > kr) : (ql > kl || (ql == kl && qr > kr));
+}
+
+// The finalisation's view of a slot: packed position, X | Y << 16, the cap
+// priority K_l << 27 | K_r << 12 | response, and the rank in the segment.
+__device__ __forceinline__ uint4 slot_info(uint32_t pos, int X, int Y, uint32_t own, uint32_t key, int rank)
+{
+    return make_uint4(pos, (uint32_t)X | ((uint32_t)Y << 16), ((own >> 16) << 27) | ((own & 0xFFFFu) << 12) | (key >> 16),
+                      (uint32_t)rank);
 }
 
 __global__ void __launch_bounds__(kNmsThreads) k_pfa_nms(Batch b)
@@ -39,55 +54,51 @@ __global__ void __launch_bounds__(kNmsThreads) k_pfa_nms(Batch b)
     __shared__ uint32_t sk[kMaxSegment];
     __shared__ int alive_total;
     const int seg = blockIdx.x;
-    const LevelDesc L = b.levels[b.seg_level[seg]];
-    const ImageDesc &I = b.images[L.image];
+    const SegRec &R = b.seg_rec[seg];
     const int k = b.prm.k, rad = b.prm.nms_rad, rule = b.prm.rule;
-    const int cy = seg - L.seg_base;
-    const int m = L.cells_x * k;
+    const int m = R.m, base = R.slot, W0 = R.W0, H0 = R.H0;
     if (m > kMaxSegment) {
+        for (int i = threadIdx.x; i < m; i += kNmsThreads)
+            b.slot_info[base + i] = slot_info(0u, 0, 0, 0u, 0u, kSlotEmpty);
         if (threadIdx.x == 0) { atomicOr(b.err, kErrSegment); b.seg_count[seg] = 0; }
         return;
     }
-    const int base = L.slot_base + cy * m;
     if (threadIdx.x == 0) alive_total = 0;
     __syncthreads();
     int my_alive = 0;
     for (int i = threadIdx.x; i < m; i += kNmsThreads) {
         const uint32_t key = b.slots[base + i];
         uint32_t v = 0xFFFFFFFFu;
+        uint4 info = slot_info(0u, 0, 0, 0u, 0u, kSlotEmpty);
         if (key) {
-            const SlotPos p = decode_slot(key, cy * m + i, L.cells_x, L.c, k);
-            const int X = __ldg(L.projx + p.x), Y = __ldg(L.projy + p.y);
-            const uint32_t own = I.map[(size_t)Y * I.W0 + X];
-            const uint32_t kl = own >> 16, kr = own & 0xFFFFu;
+            const uint32_t p = slot_pos(R, key, i, k);
+            const int X = __ldg(R.projx + pos_x(p)), Y = __ldg(R.projy + pos_y(p));
+            const uint32_t own = R.map[(size_t)Y * W0 + X];
             bool dom = false;
             for (int dy = -rad; dy <= rad; ++dy) {
                 const int qy = Y + dy;
-                if (qy < 0 || qy >= I.H0) continue;
+                if (qy < 0 || qy >= H0) continue;
                 for (int dx = -rad; dx <= rad; ++dx) {
                     const int qx = X + dx;
-                    if ((dx | dy) == 0 || qx < 0 || qx >= I.W0) continue;
-                    const uint32_t w = I.map[(size_t)qy * I.W0 + qx];
-                    if (!w) continue;
-                    const uint32_t ql = w >> 16, qr = w & 0xFFFFu;
-                    dom |= rule == 0 ? (ql > kl && qr > kr) : (ql > kl || (ql == kl && qr > kr));
+                    if ((dx | dy) == 0 || qx < 0 || qx >= W0) continue;
+                    const uint32_t w = R.map[(size_t)qy * W0 + qx];
+                    if (w) dom |= dominates(w, own, rule);
                 }
             }
-            b.slot_k[base + i] = own;
-            if (!dom) { v = ((uint32_t)p.y << 16) | (uint32_t)p.x; ++my_alive; }
+            info = slot_info(p, X, Y, own, key, kSlotSuppressed);
+            if (!dom) { v = pos_order(p); ++my_alive; }
         }
+        b.slot_info[base + i] = info;
         sk[i] = v;
     }
     if (my_alive) atomicAdd(&alive_total, my_alive);
     __syncthreads();
     for (int i = threadIdx.x; i < m; i += kNmsThreads) {
         const uint32_t v = sk[i];
-        int rank = -1;
-        if (v != 0xFFFFFFFFu) {
-            rank = 0;
-            for (int j = 0; j < m; ++j) rank += sk[j] < v;
-        }
-        b.slot_rank[base + i] = rank;
+        if (v == 0xFFFFFFFFu) continue;
+        int rank = 0;
+        for (int j = 0; j < m; ++j) rank += sk[j] < v;
+        b.slot_info[base + i].w = (uint32_t)rank;
     }
     if (threadIdx.x == 0) b.seg_count[seg] = alive_total;
 }
@@ -95,333 +106,480 @@ __global__ void __launch_bounds__(kNmsThreads) k_pfa_nms(Batch b)
 // The same per segment with one warp, for batches whose segments (cell rows:
 // cells_x x k slots) all have at most 32 S slots: lane l takes slots l,
 // l + 32, ..., and every step of their chains of dependent loads (slot ->
-// projection -> own score -> neighbours) is issued for all S slots before
+// projection -> own score and neighbours) is issued for all S slots before
 // the next, so the chains overlap; a CTA of four warps takes four segments.
-template <int S>
+template <int S, int RAD>
 __global__ void __launch_bounds__(kNmsThreads) k_pfa_nms_warp(Batch b)
 {
-    __shared__ uint32_t sk[kNmsThreads / 32][32 * S];
+    __shared__ __align__(16) uint32_t sk[kNmsThreads / 32][32 * S];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int seg = blockIdx.x * (kNmsThreads / 32) + warp;
     if (seg >= b.n_segments) return;  // whole warps only
-    const LevelDesc &L = b.levels[b.seg_level[seg]];
-    const ImageDesc &I = b.images[L.image];
-    const int k = b.prm.k, rad = b.prm.nms_rad, rule = b.prm.rule;
-    const int cy = seg - L.seg_base;
-    const int m = L.cells_x * k;
+    const SegRec R = b.seg_rec[seg];
+    const int k = b.prm.k, rule = b.prm.rule;
+    const int m = R.m, base = R.slot, W0 = R.W0, H0 = R.H0;
     if (m > 32 * S) {  // the host launches this kernel only when no segment is wider
+        for (int i = lane; i < m; i += 32) b.slot_info[base + i] = slot_info(0u, 0, 0, 0u, 0u, kSlotEmpty);
         if (lane == 0) { atomicOr(b.err, kErrSegment); b.seg_count[seg] = 0; }
         return;
     }
-    const int base = L.slot_base + cy * m;
-    const int W0 = I.W0, H0 = I.H0;
-    uint32_t key[S], own[S];
-    int X[S], Y[S], px[S], py[S];
+    uint32_t key[S], own[S], pos[S];
+    int X[S], Y[S];
     bool dom[S];
 #pragma unroll
     for (int q = 0; q < S; ++q) key[q] = lane + 32 * q < m ? b.slots[base + lane + 32 * q] : 0u;
 #pragma unroll
     for (int q = 0; q < S; ++q) {
-        X[q] = Y[q] = px[q] = py[q] = 0;
+        X[q] = Y[q] = 0;
+        pos[q] = 0u;
         if (key[q]) {
-            const SlotPos p = decode_slot(key[q], cy * m + lane + 32 * q, L.cells_x, L.c, k);
-            px[q] = p.x; py[q] = p.y;
-            X[q] = __ldg(L.projx + p.x);
-            Y[q] = __ldg(L.projy + p.y);
+            pos[q] = slot_pos(R, key[q], lane + 32 * q, k);
+            X[q] = __ldg(R.projx + pos_x(pos[q]));
+            Y[q] = __ldg(R.projy + pos_y(pos[q]));
         }
     }
 #pragma unroll
     for (int q = 0; q < S; ++q) {
-        own[q] = key[q] ? I.map[(size_t)Y[q] * W0 + X[q]] : 0u;
+        own[q] = key[q] ? R.map[(size_t)Y[q] * W0 + X[q]] : 0u;
         dom[q] = false;
     }
-    for (int dy = -rad; dy <= rad; ++dy)
-        for (int dx = -rad; dx <= rad; ++dx) {
-            if ((dx | dy) == 0) continue;
-            uint32_t w[S];
+    // a window row's loads (of all slots) are in flight together, for the
+    // 3 x 3 window all eight neighbours'
+    constexpr int kSide = 2 * RAD + 1, kRows = RAD == 1 ? 3 : 1;
 #pragma unroll
-            for (int q = 0; q < S; ++q) {
-                const int qx = X[q] + dx, qy = Y[q] + dy;
-                w[q] = key[q] && qx >= 0 && qx < W0 && qy >= 0 && qy < H0 ? I.map[(size_t)qy * W0 + qx] : 0u;
-            }
+    for (int dy0 = -RAD; dy0 <= RAD; dy0 += kRows) {
+        uint32_t w[kRows][kSide][S];
 #pragma unroll
-            for (int q = 0; q < S; ++q)
-                if (w[q]) {
-                    const uint32_t ql = w[q] >> 16, qr = w[q] & 0xFFFFu, kl = own[q] >> 16, kr = own[q] & 0xFFFFu;
-                    dom[q] |= rule == 0 ? (ql > kl && qr > kr) : (ql > kl || (ql == kl && qr > kr));
+        for (int r = 0; r < kRows; ++r)
+#pragma unroll
+            for (int c = 0; c < kSide; ++c)
+#pragma unroll
+                for (int q = 0; q < S; ++q) {
+                    const int dx = c - RAD, dy = dy0 + r, qx = X[q] + dx, qy = Y[q] + dy;
+                    w[r][c][q] = (dx | dy) != 0 && key[q] && qx >= 0 && qx < W0 && qy >= 0 && qy < H0
+                                     ? R.map[(size_t)qy * W0 + qx] : 0u;
                 }
-        }
+#pragma unroll
+        for (int r = 0; r < kRows; ++r)
+#pragma unroll
+            for (int c = 0; c < kSide; ++c)
+#pragma unroll
+                for (int q = 0; q < S; ++q)
+                    if (w[r][c][q]) dom[q] |= dominates(w[r][c][q], own[q], rule);
+    }
     uint32_t v[S];
-    int alive = 0;
+    int rank[S], alive = 0;
 #pragma unroll
     for (int q = 0; q < S; ++q) {
         v[q] = 0xFFFFFFFFu;
-        if (key[q]) {
-            b.slot_k[base + lane + 32 * q] = own[q];
-            if (!dom[q]) { v[q] = ((uint32_t)py[q] << 16) | (uint32_t)px[q]; ++alive; }
-        }
+        rank[q] = key[q] ? kSlotSuppressed : kSlotEmpty;
+        if (key[q] && !dom[q]) { v[q] = pos_order(pos[q]); rank[q] = 0; ++alive; }
         sk[warp][lane + 32 * q] = v[q];
     }
     __syncwarp();
+    // entries past the segment are never below a corner
+    for (int j = 0; j < m; j += 4) {
+        const uint4 o = *reinterpret_cast<const uint4 *>(&sk[warp][j]);
+#pragma unroll
+        for (int q = 0; q < S; ++q)
+            if (rank[q] >= 0) rank[q] += (o.x < v[q]) + (o.y < v[q]) + (o.z < v[q]) + (o.w < v[q]);
+    }
 #pragma unroll
     for (int q = 0; q < S; ++q)
-        if (lane + 32 * q < m) {
-            int rank = -1;
-            if (v[q] != 0xFFFFFFFFu) {
-                rank = 0;
-                for (int j = 0; j < m; ++j) rank += sk[warp][j] < v[q];
-            }
-            b.slot_rank[base + lane + 32 * q] = rank;
-        }
+        if (lane + 32 * q < m)
+            b.slot_info[base + lane + 32 * q] = slot_info(pos[q], X[q], Y[q], own[q], key[q], rank[q]);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) alive += __shfl_xor_sync(0xFFFFFFFFu, alive, off);
     if (lane == 0) b.seg_count[seg] = alive;
 }
 
+template <int RAD>
+static void launch_nms_warp(const Batch &b, cudaStream_t stream)
+{
+    constexpr int per = kNmsThreads / 32;
+    const int grid = (b.n_segments + per - 1) / per;
+    if (b.max_segment <= 32) k_pfa_nms_warp<1, RAD><<<grid, kNmsThreads, 0, stream>>>(b);
+    else if (b.max_segment <= 64) k_pfa_nms_warp<2, RAD><<<grid, kNmsThreads, 0, stream>>>(b);
+    else k_pfa_nms_warp<3, RAD><<<grid, kNmsThreads, 0, stream>>>(b);
+}
+
 cudaError_t launch_pfa_nms(const Batch &b, cudaStream_t stream)
 {
     if (b.n_segments == 0) return cudaSuccess;
-    constexpr int per = kNmsThreads / 32;
-    if (b.nms_kernel == 1) {
+    if (b.nms_kernel == 1 || b.max_segment > 96) {
         k_pfa_nms<<<b.n_segments, kNmsThreads, 0, stream>>>(b);
-    } else if (b.max_segment <= 32) {
-        k_pfa_nms_warp<1><<<(b.n_segments + per - 1) / per, kNmsThreads, 0, stream>>>(b);
-    } else if (b.max_segment <= 64) {
-        k_pfa_nms_warp<2><<<(b.n_segments + per - 1) / per, kNmsThreads, 0, stream>>>(b);
-    } else if (b.max_segment <= 96) {
-        k_pfa_nms_warp<3><<<(b.n_segments + per - 1) / per, kNmsThreads, 0, stream>>>(b);
     } else {
-        k_pfa_nms<<<b.n_segments, kNmsThreads, 0, stream>>>(b);
+        switch (b.prm.nms_rad) {
+        case 0: launch_nms_warp<0>(b, stream); break;
+        case 1: launch_nms_warp<1>(b, stream); break;
+        case 2: launch_nms_warp<2>(b, stream); break;
+        default: launch_nms_warp<3>(b, stream); break;
+        }
     }
     return cudaGetLastError();
 }
 
-// Exclusive block-wide prefix sum of v; *total receives the block sum.
+// Exclusive block-wide prefix sum of v; *total receives the block sum.  `ws`
+// (a word a warp) may be used again once every thread has passed another
+// barrier.
 template <int NT>
-__device__ __forceinline__ int block_excl_scan(int v, int *ws, int *total)
+__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *ws, uint32_t *total)
 {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int x = v;
+    uint32_t x = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
         if (lane >= o) x += y;
     }
     if (lane == 31) ws[w] = x;
     __syncthreads();
-    if (w == 0) {
-        int s = lane < NT / 32 ? ws[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, s, o);
-            if (lane >= o) s += y;
-        }
-        if (lane < NT / 32) ws[lane] = s;
-    }
-    __syncthreads();
-    const int pre = w > 0 ? ws[w - 1] : 0;
-    *total = ws[NT / 32 - 1];
-    __syncthreads();
-    return pre + x - v;
+    // every warp sums the warps' totals for itself: those before it, and all
+    const uint32_t t = lane < NT / 32 ? ws[lane] : 0u;
+    *total = __reduce_add_sync(0xFFFFFFFFu, t);
+    return __reduce_add_sync(0xFFFFFFFFu, lane < w ? t : 0u) + x - v;
 }
 
-// Cap priorities of the first kFinPrioCache canonical survivors, kept in
-// shared memory for the four radix passes and the compaction (32 KB; two
-// CTAs still fit an SM).  Images with more survivors read the rest through
-// their slots.
-constexpr int kFinPrioCache = 8192;
+// The finalisation of one image by a cluster of CTAs (one to eight, see
+// launch_pfa_finalize): the candidate slots and then the canonical positions
+// are shared out over its CTAs, the histograms of the cap's radix select are
+// summed through distributed shared memory, and a cluster barrier ends each
+// phase.
+//
+// What bounds it: latency -- a chain of barriers and dependent reads whose
+// data lie in L2; the bytes are few.  One CTA of 1024 threads an image left
+// the chip idle for small batches.  Stage times, before and now (us): one
+// 1920x1080 pair (16 000 slots an image) 96 and 29, one 1241x376 pair 31 and
+// 22, 16 mixed pairs 98 and 33, 100 pairs of 1241x376 47 and 37.
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_size()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+// Barrier over the cluster; global and shared writes before it are seen after it.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// 16 bytes at the address of `p` (a shared object of this CTA) in CTA `rank` of the cluster.
+__device__ __forceinline__ uint4 ld_cluster(const void *p, uint32_t rank)
+{
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(r) : "memory");
+    return v;
+}
 
 // Row index of an image's canonical list, for the stereo matching (all
-// threads of the finalisation's CTA, after its barrier: the keypoints'
-// levels and Y and the level starts in lstart, kMaxLevels + 1 entries whose
-// last is the count, are complete).  Entry v of level l's table is the
-// first index of the level whose Y is >= v, else the level's end: keypoint
-// j owns the entries (Y[j - 1], Y[j]] when it is not the level's first;
-// the entries up to the first keypoint's Y (the level's start) and after
-// the last one's (its end) are spread over the CTA.  Every level with
-// keypoints gets all H0 + 1 entries.  Not inlined: its registers stay out
-// of the finalisation's allocation.
-__device__ __noinline__ void fill_row_index(const ImageDesc &I, const int *lstart)
+// threads of the cluster, after the barrier that completes the keypoints'
+// levels and Y; level starts in lstart, kMaxLevels + 1 entries whose last is
+// the count).  Entry v of level l's table is the first index of the level
+// whose Y is >= v, else the level's end: keypoint j owns the entries
+// (Y[j - 1], Y[j]] when it is not the level's first; the entries up to the
+// first keypoint's Y (the level's start) and after the last one's (its end)
+// are spread over the threads.  Every level with keypoints gets all H0 + 1
+// entries.
+__device__ __forceinline__ void fill_row_index(const ImageDesc &I, const int *lstart, int thread, int threads)
 {
     const int rows = I.H0 + 1, keep = lstart[kMaxLevels];
     const KpOut &o = I.out;
-    for (int j = threadIdx.x; j < keep; j += kFinThreads) {
-        const int l = o.level[j];
+    for (int j = thread; j < keep; j += threads) {
+        const int l = o.level[j], Yj = o.Y[j], Yp = j > 0 ? (int)o.Y[j - 1] : 0;
         if (j == lstart[l]) continue;
-        const int Yj = o.Y[j];
         int32_t *rf = I.row_first + (size_t)l * rows;
-        for (int v = (int)o.Y[j - 1] + 1; v <= Yj; ++v) rf[v] = j;
+        for (int v = Yp + 1; v <= Yj; ++v) rf[v] = j;
     }
-    for (int t = threadIdx.x; t < I.levels * rows; t += kFinThreads) {
-        const int l = t / rows, v = t - l * rows;
+    for (int l = 0; l < I.levels; ++l) {
         const int s = lstart[l], e = lstart[l + 1];
         if (s == e) continue;
-        if (v <= (int)o.Y[s]) I.row_first[t] = s;
-        else if (v > (int)o.Y[e - 1]) I.row_first[t] = e;
+        const int ys = o.Y[s], ye = o.Y[e - 1];
+        int32_t *rf = I.row_first + (size_t)l * rows;
+        for (int v = thread; v < rows; v += threads) {
+            if (v <= ys) rf[v] = s;
+            else if (v > ye) rf[v] = e;
+        }
     }
 }
 
+// Digits of the radix select over the cap priorities K_l << 27 | K_r << 12 |
+// r (31 bits: K_l <= 8, K_r <= 8 x 4080, r <= 4080), high to low, of 11, 11
+// and 9 bits: the first one reaches into K_r, since almost every K_l is 1 or 2.
+constexpr int kSelPasses = 3, kSelBins = 2048;
+constexpr int kFinSegs = 1024;   // segment offsets kept in shared memory (the rest in b.seg_off)
+constexpr int kFinKeep = 4;      // positions of a thread in a round
+constexpr int kFinCluster = 8;   // most CTAs of an image
+
 __global__ void __launch_bounds__(kFinThreads, 2) k_pfa_finalize(Batch b)
 {
-    __shared__ uint32_t s_prio[kFinPrioCache];
-    __shared__ int ws[32];
-    __shared__ int hist[256];
-    __shared__ int sh_digit, sh_need;
-    __shared__ int lstart[kMaxLevels + 1];
-    __shared__ LevelDesc levs[kMaxLevels];
-    const int img = blockIdx.x;
+    __shared__ __align__(16) uint32_t hist[kSelPasses][kSelBins];
+    __shared__ uint32_t ws[2][kFinThreads / 32];
+    __shared__ __align__(16) uint32_t s_above[4];  // of this CTA's positions: above the threshold, at it
+    __shared__ uint32_t sh_digit[kSelPasses], sh_need[kSelPasses];
+    __shared__ int lfirst[kMaxLevels + 1], lstart[kMaxLevels + 1];
+    __shared__ int s_off[kFinSegs];
+    const int C = (int)cluster_size(), rank = (int)cluster_rank();
+    const int lg = 31 - __clz(C);  // a power of two
+    const int img = blockIdx.x >> lg;
     const ImageDesc &I = b.images[img];
-    const int k = b.prm.k;
-    const int nl = I.levels;
-    if (threadIdx.x < nl) levs[threadIdx.x] = b.levels[I.level_base + threadIdx.x];
-    __syncthreads();
+    const int nl = I.levels, cap = I.max_feats, slot_base = I.slot_base;
+    const int seg_base = I.seg_base, seg_count = I.seg_count;
+    for (int i = threadIdx.x; i < kSelPasses * kSelBins; i += kFinThreads) (&hist[0][0])[i] = 0;
 
-    // Canonical offsets of the segments (level-major, then cell row).
-    int carry = 0;
-    for (int base = 0; base < I.seg_count; base += kFinThreads) {
+    // Canonical offsets of the segments (level-major, then cell row), by
+    // every CTA for itself (the same values).
+    int S = 0;
+    for (int base = 0, t = 0; base < seg_count; base += kFinThreads, t ^= 1) {
         const int i = base + threadIdx.x;
-        const int v = i < I.seg_count ? b.seg_count[I.seg_base + i] : 0;
-        int tot;
-        const int ex = block_excl_scan<kFinThreads>(v, ws, &tot);
-        if (i < I.seg_count) b.seg_off[I.seg_base + i] = carry + ex;
-        carry += tot;
+        const uint32_t v = i < seg_count ? (uint32_t)b.seg_count[seg_base + i] : 0u;
+        uint32_t tot;
+        const int ex = (int)block_excl_scan<kFinThreads>(v, ws[t], &tot);
+        if (i < kFinSegs) s_off[i] = S + ex;
+        else if (i < seg_count) b.seg_off[seg_base + i] = S + ex;
+        S += (int)tot;
     }
-    const int S = carry;
     __syncthreads();
+    // first canonical position of each level
+    if (threadIdx.x <= kMaxLevels) {
+        int first = S;
+        if (threadIdx.x < nl) {
+            const int i = b.levels[I.level_base + threadIdx.x].seg_base - seg_base;
+            first = i < kFinSegs ? s_off[i] : b.seg_off[seg_base + i];
+        }
+        lfirst[threadIdx.x] = first;
+    }
 
-    // Canonical position of every survivor; clear the map entries.
-    for (int s = threadIdx.x; s < I.slot_count; s += kFinThreads) {
-        const int gs = I.slot_base + s;
-        const uint32_t key = b.slots[gs];
-        if (!key) continue;
-        int l = nl - 1;
-        while (l > 0 && levs[l].slot_base > gs) --l;
-        const LevelDesc &L = levs[l];
-        const int rel = gs - L.slot_base;
-        const SlotPos p = decode_slot(key, rel, L.cells_x, L.c, k);
-        I.map[(size_t)__ldg(L.projy + p.y) * I.W0 + __ldg(L.projx + p.x)] = 0;
-        const int rank = b.slot_rank[gs];
-        if (rank >= 0) {
-            const int cy = rel / (L.cells_x * k);
-            b.canon[I.slot_base + b.seg_off[L.seg_base + cy] + rank] = gs;
+    // Canonical position of every survivor of this CTA's segments (a warp
+    // each), its priority and coordinates written there; the map entries
+    // cleared.
+    uint32_t *const map = I.map;
+    const int W0 = I.W0;
+    for (int i = rank * (kFinThreads / 32) + ((int)threadIdx.x >> 5); i < seg_count; i += C * (kFinThreads / 32)) {
+        const SegRec &R = b.seg_rec[seg_base + i];
+        const int m = R.m, slot = R.slot, at = slot_base + (i < kFinSegs ? s_off[i] : b.seg_off[seg_base + i]);
+        for (int j0 = threadIdx.x & 31; j0 < m; j0 += 96) {
+            uint4 v[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                v[q] = j0 + 32 * q < m ? b.slot_info[slot + j0 + 32 * q] : make_uint4(0u, 0u, 0u, (uint32_t)kSlotEmpty);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const int r = (int)v[q].w;
+                if (r == kSlotEmpty) continue;
+                map[(size_t)(v[q].y >> 16) * W0 + (v[q].y & 0xFFFFu)] = 0;
+                if (r >= 0) {
+                    b.canon_prio[at + r] = v[q].z;
+                    b.canon_pos[at + r] = make_uint2(v[q].x, v[q].y);
+                }
+            }
         }
     }
-    __syncthreads();
+    cluster_sync();
 
-    // Cap: keep the max_feats largest priorities P = K_l << 27 | K_r << 12 | r,
-    // ties at the threshold resolved in canonical order.
-    auto prio = [&](int g) -> uint32_t {
-        const int gs = b.canon[I.slot_base + g];
-        const uint32_t K = b.slot_k[gs];
-        return ((K >> 16) << 27) | ((K & 0xFFFFu) << 12) | (b.slots[gs] >> 16);
+    // This CTA's positions: [g0, g1), in rounds of kRound; a thread has
+    // kFinKeep neighbouring ones of a round, those of the first round in
+    // registers.
+    constexpr int kRound = kFinKeep * kFinThreads;
+    const uint32_t *prio = b.canon_prio + slot_base;
+    const int g0 = (int)(((uint32_t)S * (uint32_t)rank) >> lg), g1 = (int)(((uint32_t)S * (uint32_t)(rank + 1)) >> lg);
+    const int t0 = kFinKeep * (int)threadIdx.x;
+    uint32_t mine[kFinKeep];
+    const auto load = [&](int base) {
+#pragma unroll
+        for (int i = 0; i < kFinKeep; ++i) mine[i] = base + t0 + i < g1 ? prio[base + t0 + i] : 0u;
     };
-    for (int g = threadIdx.x; g < min(S, kFinPrioCache); g += kFinThreads) s_prio[g] = prio(g);
-    __syncthreads();
-    auto prio_c = [&](int g) -> uint32_t { return g < kFinPrioCache ? s_prio[g] : prio(g); };
-    const bool capped = S > I.max_feats;
-    uint32_t T = 0;
+    load(g0);
+
+    // Cap: keep the max_feats largest priorities, ties at the threshold T
+    // resolved in canonical order.
+    const bool capped = S > cap;
+    uint32_t T = 0, mask = 0;
     int quota = 0;
-    if (capped) {
-        int need = I.max_feats;
-        uint32_t prefix = 0, mask = 0;
-        for (int sh = 24; sh >= 0; sh -= 8) {
-            for (int i = threadIdx.x; i < 256; i += kFinThreads) hist[i] = 0;
-            __syncthreads();
-            for (int g = threadIdx.x; g < S; g += kFinThreads) {
-                const uint32_t P = prio_c(g);
-                if ((P & mask) == prefix) atomicAdd(&hist[(P >> sh) & 255u], 1);
-            }
-            __syncthreads();
-            // the largest digit d whose count, added to the counts of the
-            // larger digits, reaches `need` (which never exceeds the total):
-            // lane l holds digits 255 - 8 l down to 248 - 8 l, a warp scan
-            // gives the counts above each lane, and the one lane where the
-            // running count crosses `need` walks its eight digits
-            if (threadIdx.x < 32) {
-                const int lane = threadIdx.x;
-                int cnt8[8], s8 = 0;
+    // f(priority) of every position of this thread
+    const auto each = [&](auto f) {
+        for (int base = g0; base < g1; base += kRound) {
+            if (base != g0) load(base);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    cnt8[j] = hist[255 - 8 * lane - j];
-                    s8 += cnt8[j];
-                }
-                int incl = s8;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                    if (lane >= o) incl += y;
-                }
-                int cum = incl - s8;
-                if (cum < need && incl >= need) {
-                    int j = 0;
-                    for (; j < 7; ++j) {
-                        if (cum + cnt8[j] >= need) break;
-                        cum += cnt8[j];
-                    }
-                    sh_digit = 255 - 8 * lane - j;
-                    sh_need = need - cum;
-                }
-            }
-            __syncthreads();
-            prefix |= (uint32_t)sh_digit << sh;
-            mask |= 255u << sh;
-            need = sh_need;
-            __syncthreads();
+            for (int i = 0; i < kFinKeep; ++i)
+                if (base + t0 + i < g1) f(mine[i]);
         }
-        T = prefix;
+        if (g1 - g0 > kRound) load(g0);
+    };
+    if (capped) {
+        int need = cap;
+#pragma unroll
+        for (int pass = 0; pass < kSelPasses; ++pass) {
+            const int sh = pass == 0 ? 20 : pass == 1 ? 9 : 0;
+            each([&](uint32_t P) {
+                if ((P & mask) == T) atomicAdd(&hist[pass][(P & ~mask) >> sh], 1u);
+            });
+            cluster_sync();
+            // the largest digit whose count, added to the counts of the larger
+            // digits, reaches `need` (which never exceeds the total): a thread
+            // has four digits, from the largest down
+            static_assert(kSelBins == 4 * kFinThreads, "four digits a thread");
+            const int d0 = kSelBins - 4 - 4 * (int)threadIdx.x;
+            uint4 n4 = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int c = 0; c < kFinCluster; ++c)
+                if (c < C) {
+                    const uint4 h = ld_cluster(&hist[pass][d0], (uint32_t)c);
+                    n4.x += h.x; n4.y += h.y; n4.z += h.z; n4.w += h.w;
+                }
+            const int n[4] = { (int)n4.w, (int)n4.z, (int)n4.y, (int)n4.x };
+            uint32_t tot;
+            int cum = (int)block_excl_scan<kFinThreads>((uint32_t)(n[0] + n[1] + n[2] + n[3]), ws[pass & 1], &tot);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (cum < need && cum + n[j] >= need) {
+                    sh_digit[pass] = (uint32_t)(d0 + 3 - j);
+                    sh_need[pass] = (uint32_t)(need - cum);
+                }
+                cum += n[j];
+            }
+            __syncthreads();
+            T |= sh_digit[pass] << sh;
+            mask = ~((1u << sh) - 1u);
+            need = (int)sh_need[pass];
+        }
         quota = need;
     }
-    const int keep = capped ? I.max_feats : S;
-    if (threadIdx.x <= kMaxLevels) lstart[threadIdx.x] = keep;
-    __syncthreads();
+    const int keep = capped ? cap : S;
 
-    int carry_tie = 0, carry_out = 0;
+    // Positions before this CTA's that are above the threshold and at it (not
+    // capped: all are above)
+    int carry_up = g0, carry_tie = 0;
+    const auto counts = [&]() {  // of this thread's positions in the round in registers: above | at << 16
+        uint32_t c = 0;
+#pragma unroll
+        for (int i = 0; i < kFinKeep; ++i) c += (mine[i] > T ? 1u : 0u) + (mine[i] == T ? 1u << 16 : 0u);
+        return c;
+    };
+    static_assert(kRound < 65536, "a round's counts fit 16 bits");
+    if (capped) {  // T >= 1: the positions past g1 (priority 0) count for nothing
+        uint32_t up = 0, tie = 0;
+        for (int base = g0; base < g1; base += kRound) {
+            if (base != g0) load(base);
+            const uint32_t c = counts();
+            up += c & 0xFFFFu;
+            tie += c >> 16;
+        }
+        if (g1 - g0 > kRound) load(g0);
+        if (threadIdx.x < 2) s_above[threadIdx.x] = 0u;
+        __syncthreads();
+        up = __reduce_add_sync(0xFFFFFFFFu, up);
+        tie = __reduce_add_sync(0xFFFFFFFFu, tie);
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&s_above[0], up);
+            atomicAdd(&s_above[1], tie);
+        }
+        cluster_sync();
+        carry_up = 0;
+#pragma unroll
+        for (int c = 0; c < kFinCluster - 1; ++c)
+            if (c < rank) {
+                const uint4 v = ld_cluster(s_above, (uint32_t)c);
+                carry_up += (int)v.x;
+                carry_tie += (int)v.y;
+            }
+    }
+
+    // the kept positions in order; position g is preceded by up + min(tie, quota) kept ones
     const KpOut &o = I.out;
-    for (int base = 0; base < S; base += kFinThreads) {
-        const int g = base + threadIdx.x;
-        const bool valid = g < S;
-        const uint32_t P = valid ? prio_c(g) : 0u;
-        int tot;
-        const int tie_rank = carry_tie + block_excl_scan<kFinThreads>(valid && capped && P == T, ws, &tot);
-        carry_tie += tot;
-        const bool kept = valid && (!capped || P > T || (P == T && tie_rank < quota));
-        const int oi = carry_out + block_excl_scan<kFinThreads>(kept, ws, &tot);
-        carry_out += tot;
-        if (kept) {
-            const int gs = b.canon[I.slot_base + g];
-            int l = nl - 1;
-            while (l > 0 && levs[l].slot_base > gs) --l;
-            const LevelDesc &L = levs[l];
-            const uint32_t key = b.slots[gs];
-            const SlotPos p = decode_slot(key, gs - L.slot_base, L.cells_x, L.c, k);
-            const uint32_t K = b.slot_k[gs];
-            o.x[oi] = (uint16_t)p.x;
-            o.y[oi] = (uint16_t)p.y;
-            o.X[oi] = __ldg(L.projx + p.x);
-            o.Y[oi] = __ldg(L.projy + p.y);
-            o.level[oi] = (uint8_t)l;
-            o.response[oi] = (uint16_t)p.r;
-            o.k_levels[oi] = (uint8_t)(K >> 16);
-            o.k_resp[oi] = K & 0xFFFFu;
-            atomicMin(&lstart[l], oi);
+    for (int base = g0, t = 0; base < g1; base += kRound, t ^= 1) {
+        if (base != g0) load(base);
+        uint2 at[kFinKeep];
+#pragma unroll
+        for (int i = 0; i < kFinKeep; ++i)
+            at[i] = base + t0 + i < g1 ? b.canon_pos[slot_base + base + t0 + i] : make_uint2(0u, 0u);
+        int up = carry_up + t0, tie = 0;
+        uint32_t tot = kRound;
+        if (capped) {
+            const uint32_t ex = block_excl_scan<kFinThreads>(counts(), ws[t], &tot);
+            up = carry_up + (int)(ex & 0xFFFFu);
+            tie = carry_tie + (int)(ex >> 16);
+        }
+#pragma unroll
+        for (int i = 0; i < kFinKeep; ++i) {
+            const int g = base + t0 + i;
+            if (g >= g1) break;
+            const uint32_t P = mine[i];
+            const int oi = up + min(tie, quota);
+            const bool is_up = !capped || P > T, is_tie = capped && P == T;
+            const int l = (int)(at[i].x >> 26);
+            // level starts: of this level and of the empty ones before it
+            for (int m = l; m >= 0 && lfirst[m] == g; --m) I.level_start[m] = oi;
+            if (is_up || (is_tie && tie < quota)) {
+                o.x[oi] = (uint16_t)pos_x(at[i].x);
+                o.y[oi] = (uint16_t)pos_y(at[i].x);
+                o.X[oi] = (uint16_t)(at[i].y & 0xFFFFu);
+                o.Y[oi] = (uint16_t)(at[i].y >> 16);
+                o.level[oi] = (uint8_t)l;
+                o.response[oi] = (uint16_t)(P & 0xFFFu);
+                o.k_levels[oi] = (uint8_t)(P >> 27);
+                o.k_resp[oi] = (P >> 12) & 0x7FFFu;
+            }
+            up += is_up;
+            tie += is_tie;
+        }
+        carry_up += (int)(tot & 0xFFFFu);
+        carry_tie += (int)(tot >> 16);
+    }
+    if (rank == 0 && threadIdx.x <= kMaxLevels) {
+        if (lfirst[threadIdx.x] == S) I.level_start[threadIdx.x] = keep;  // no position of this level or a later one
+        if (threadIdx.x == 0) {
+            *I.count = keep;
+            *I.count_hdr = keep;
         }
     }
+    cluster_sync();
+    if (threadIdx.x <= kMaxLevels) lstart[threadIdx.x] = I.level_start[threadIdx.x];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int l = kMaxLevels - 1; l >= 0; --l) lstart[l] = min(lstart[l], lstart[l + 1]);
-        for (int l = 0; l <= kMaxLevels; ++l) I.level_start[l] = lstart[l];
-        *I.count = keep;
-        *I.count_hdr = keep;
-    }
-    __syncthreads();
-    fill_row_index(b.images[img], lstart);
+    fill_row_index(I, lstart, rank * kFinThreads + (int)threadIdx.x, C * kFinThreads);
+}
+
+// CTAs per image.  More of them shorten the chains of a small batch, each
+// costs the cluster's barriers, and in a large batch the images fill the
+// chip: at least 700 slots a CTA, and no more CTAs than SMs -- two an image
+// also when all of them run at once (three CTAs fit an SM).  Measured with 1 /
+// 2 / 4 / 8 (us, finalisation stage before the last rounds of tuning): one
+// 1920x1080 pair (16 000 slots an image) 84 / 51 / 37 / 31, one 1241x376 pair
+// (3 900) 34 / 24 / 23 / 24, 16 mixed pairs (to 16 000) 86 / 53 / 39 / 41, 12
+// of 752x480 (2 900) 29 / 23 / 21 / 35, 25 of 1241x376 35 / 27 / 27 / 45, 100 of
+// 1241x376 45 / 37 / 61 / 158.
+static int finalize_ctas(const Batch &b)
+{
+    int c = 1;
+    while (c < kFinCluster && b.max_slots / (2 * c) >= 700 &&
+           (b.n_images * 2 * c <= b.n_sm || (c == 1 && b.n_images * 2 <= 3 * b.n_sm)))
+        c *= 2;
+    return c;
 }
 
 cudaError_t launch_pfa_finalize(const Batch &b, cudaStream_t stream)
 {
     if (b.n_images == 0) return cudaSuccess;
-    k_pfa_finalize<<<b.n_images, kFinThreads, 0, stream>>>(b);
-    return cudaGetLastError();
+    const int C = finalize_ctas(b);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(b.n_images * C);
+    cfg.blockDim = dim3(kFinThreads);
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_pfa_finalize, b);
 }
 
 }  // namespace jslam
