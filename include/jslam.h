@@ -387,10 +387,11 @@ jslam_status jslam_enable_stage_timing(jslam_ctx *ctx, int32_t enable);
 jslam_status jslam_stage_times(jslam_ctx *ctx, float *ms /* JSLAM_NUM_STAGES entries */);
 
 /* Launch-shape tuning.  None of these changes a result: detection tiles hold
- * whole culling cells, and every kernel variant computes the same outputs. */
+ * whole culling cells, and every kernel variant computes the same outputs.
+ * Until a tuning is set (or tuned), tile heights and order follow the batch. */
 typedef struct {
-    int32_t tile_w_px;           /* detection tile width: 32..128, multiple of 4 (default 128) */
-    int32_t tile_h_px;           /* detection tile height: 8..128 (default 64) */
+    int32_t tile_w_px;           /* detection tile width, at most: 32..128, multiple of 4 (default 128) */
+    int32_t tile_h_px;           /* detection tile height, about: 8..128 (default 64) */
     int32_t nms_kernel;          /* PFA NMS: 0 one warp per segment when every segment of the batch has at most
                                   * 96 candidate slots, else one CTA per segment (default); 1 one CTA per
                                   * segment always */

@@ -1,6 +1,7 @@
 // C ABI of libjslam: context, grow-only device buffers, batch plans and the
 // launch sequence of the stereo frontend.
 #include <algorithm>
+#include <array>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -57,12 +58,13 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
     return fn;
 }
 
-// Detection tile box of a level: rows of box_w bytes (a multiple of 16 that
-// covers the tile, its 4-pixel halo on both sides and up to 12 bytes of
-// alignment slack on the left) and box_h rows (3-row halo above and below).
+// Detection tile box of a level: rows of box_w bytes -- the tile's 32-byte
+// chunks and one more, which covers its 4-pixel halo on both sides and up to
+// 15 bytes of alignment slack on the left -- and box_h rows (3-row halo above
+// and below).
 void detect_box(int tw, int th, int *box_w, int *box_h)
 {
-    *box_w = (int)align_up((size_t)(tw + 8 + 12), 16);
+    *box_w = 32 * ((tw + 31) / 32 + 1);
     *box_h = th + 6;
 }
 
@@ -233,6 +235,8 @@ struct jslam_ctx {
 
     // launch-shape tuning and the captured graph
     jslam_tuning tune{128, 64, 0, 0, 0};
+    bool tune_chosen = false;               // by jslam_set_tuning or the autotuner
+    bool plan_chosen = false;
     jslam_tuning plan_tune{0, 0, 0, 0, 0};  // tuning the current plan was built with (tile fields)
     cudaGraphExec_t graph = nullptr;
     cudaGraph_t graph_src = nullptr;    // the captured graph (its node handles address `graph`)
@@ -291,10 +295,10 @@ jslam_status check_job(const jslam_ctx *ctx, const jslam_stereo_job &j)
     return JSLAM_OK;
 }
 
-// Cells per detection tile: about tile_w x tile_h pixels (128 x 64 by
-// default), capped in cells x k; the tile width is kept a multiple of 4
-// pixels where possible so that tiles start on word boundaries.
-void fast_block(int c, int k, int tile_w, int tile_h, int *bx, int *by)
+// Cells per tile of the per-pixel detection kernel: about tile_w x tile_h
+// pixels, capped in cells x k; the tile width is kept a multiple of 4 pixels
+// where possible so that tiles start on word boundaries.
+void cull_block(int c, int k, int tile_w, int tile_h, int *bx, int *by)
 {
     int x = tile_w / c > 1 ? tile_w / c : 1;
     for (int cand = x; cand >= 1; --cand)
@@ -305,6 +309,117 @@ void fast_block(int c, int k, int tile_w, int tile_h, int *bx, int *by)
     }
     *bx = x;
     *by = y;
+}
+
+// Shared memory of a bit-sliced tile's two boxes and planes.
+int bits_tile_bytes(int tw, int th)
+{
+    int bw, bh;
+    detect_box(tw, th, &bw, &bh);
+    return bh * (2 * bw + 16 * bs_row_units((tw + 31) / 32));
+}
+
+// Issue slots of a tile of the bit-sliced kernel with `rows` evaluated rows of
+// nch 32-pixel chunks: measured on the 1241x376 sequence, about 1000 a warp's
+// round of ring tests and responses, 115 a round of transposed chunks, 300 a
+// tile.
+double bits_tile_cost(int rows, int nch)
+{
+    const int rounds = (rows * nch + kFastThreads - 1) / kFastThreads;
+    const int chunks = rows ? ((rows + 6) * (nch + 1) + kFastThreads - 1) / kFastThreads : 0;
+    return 1000.0 * rounds + 115.0 * chunks + 300.0;
+}
+
+struct BitsBlock {
+    int bx, by;
+    double cost, tile;  // of the level's tiles, of its dearest one
+};
+
+// Cells per tile of the bit-sliced kernel on a level.  A tile's evaluated
+// rows x 32-pixel chunks are items, a lane each, so cells whose size divides
+// neither 32 nor the CTA leave lanes and warps idle: with about 128 x 64
+// pixels, 22-pixel cells made 132 items for 128 threads.  Of the blocks at
+// most max_w x max_h pixels (one cell at least) whose two boxes and planes
+// take at most `budget` bytes of shared memory, the one whose tiles over the
+// level cost least.
+BitsBlock bits_block(int W, int H, int c, int k, int border, int max_w, int max_h, int budget)
+{
+    const int cells_x = (W + c - 1) / c, cells_y = (H + c - 1) / c;
+    BitsBlock best{ 1, 1, -1.0, 0.0 };
+    for (int x = 1; x <= cells_x && (x == 1 || x * c <= max_w); ++x)
+        for (int y = 1; y <= cells_y && (y == 1 || y * c <= max_h); ++y) {
+            if (x * y > 1 && (x * y * k > kFastMaxCellsPerCta ||
+                              bits_tile_bytes(std::min(x * c, W), std::min(y * c, H)) > budget))
+                break;
+            double cost = 0.0, tile = 0.0;
+            for (int ty = 0; ty < cells_y; ty += y) {
+                const int y0 = ty * c, th = std::min(y * c, H - y0);
+                const int rows = std::max(std::min(H - border - y0, th) - std::max(border - y0, 0), 0);
+                for (int tx = 0; tx < cells_x; tx += x) {
+                    const double one = bits_tile_cost(rows, (std::min(x * c, W - tx * c) + 31) / 32);
+                    cost += one;
+                    tile = std::max(tile, one);
+                }
+            }
+            if (best.cost < 0.0 || cost < best.cost) best = { x, y, cost, tile };
+        }
+    return best;
+}
+
+// Detection tiles of every level of a batch (pairs of one shape share them).
+// A chosen tile size is about what the tiles get (up to half as tall again
+// where that fits).  By default the tallest tiles whose launch takes least
+// time: large tiles waste less on their halo, but a launch of few tiles ends
+// with most CTAs idle, so the estimate adds the dearest tile to the tiles'
+// cost shared out over the CTAs that run at once (five an SM fit the budget
+// of a 128 x 74 tile).  Detection of 100 pairs of 1241x376: 0.729 ms with the
+// largest blocks of 128 x 64 pixels whose width is a multiple of 4, 0.692 with
+// these.  Heights up to 96 / 64 / 48 / 32 / 24 (us): those 100 pairs 585 / 596 /
+// 680 / 748 / 783 (default 585), 24 pairs of 647x363 with three keypoints a
+// cell 210 / 201 / 201 / 223 / 238 (202), one pair of 320x240 14.2 / 14.2 / 14.2
+// / 13.0 / 12.3 (12.6).
+void detect_blocks(const std::vector<Geometry> &geo, bool bits, int k, int border, int tile_w, int tile_h, bool chosen,
+                   int n_sm, std::vector<std::array<std::pair<int, int>, kMaxLevels>> &blocks)
+{
+    const int n = (int)geo.size();
+    blocks.resize(n);
+    auto same = [&](int p, int q) {
+        bool eq = geo[p].levels == geo[q].levels;
+        for (int l = 0; eq && l < geo[p].levels; ++l)
+            eq = geo[p].W[l] == geo[q].W[l] && geo[p].H[l] == geo[q].H[l] && geo[p].c[l] == geo[q].c[l];
+        return eq;
+    };
+    if (!bits) {
+        for (int p = 0; p < n; ++p)
+            for (int l = 0; l < geo[p].levels; ++l)
+                cull_block(geo[p].c[l], k, tile_w, tile_h, &blocks[p][l].first, &blocks[p][l].second);
+        return;
+    }
+    static const int heights[] = { 96, 64, 48, 32, 24, 16 };
+    std::vector<std::array<std::pair<int, int>, kMaxLevels>> cand(n);
+    double best = -1.0;
+    for (int h : heights) {
+        const int max_h = chosen ? std::min(tile_h * 3 / 2, kFastMaxTile) : h;
+        const int budget = bits_tile_bytes(tile_w, tile_h * 23 / 20);
+        double sum = 0.0, tile = 0.0, of_pair = 0.0;
+        for (int p = 0; p < n; ++p) {
+            if (p > 0 && same(p, p - 1)) {
+                cand[p] = cand[p - 1];
+            } else {
+                of_pair = 0.0;
+                for (int l = 0; l < geo[p].levels; ++l) {
+                    const BitsBlock B = bits_block(geo[p].W[l], geo[p].H[l], geo[p].c[l], k, border, tile_w, max_h, budget);
+                    cand[p][l] = { B.bx, B.by };
+                    of_pair += 2.0 * B.cost;
+                    tile = std::max(tile, B.tile);
+                }
+            }
+            sum += of_pair;
+        }
+        const double time = sum / (5.0 * n_sm) + tile;
+        if (best < 0.0 || time < best) { best = time; blocks = cand; }
+        if (chosen) break;
+    }
 }
 
 // Pyramid strips of a level.
@@ -371,13 +486,15 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     }
     if (keys == ctx->keys && ctx->plan_tune.tile_w_px == ctx->tune.tile_w_px &&
         ctx->plan_tune.tile_h_px == ctx->tune.tile_h_px && ctx->plan_tune.tile_order == ctx->tune.tile_order &&
-        ctx->plan_skip == ctx->skip_on)
+        ctx->plan_chosen == ctx->tune_chosen && ctx->plan_skip == ctx->skip_on)
         return JSLAM_OK;
     ++ctx->plan_gen;
 
     const int n_img = 2 * n;
     const int k = cfg.k_per_cell;
+    const bool bits = ctx->prm.p_min == 9 && ctx->prm.p_max == 13;  // the bit-sliced detection kernel
     std::vector<Geometry> geo(n);
+    std::vector<std::array<std::pair<int, int>, kMaxLevels>> blocks;  // cells per detection tile of each level
     std::vector<PairLayout> layouts(n);
     std::vector<size_t> result_off(n);
     size_t result_bytes = 0, level_bytes = 0, map_bytes = 0, staging_bytes = 0, table_bytes = 0;
@@ -385,6 +502,9 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     int max_box = 0, max_px = 0, max_cells = 0, max_planes = 0;
     for (int p = 0; p < n; ++p) {
         geo[p] = level_geometry(jobs[p].left.width, jobs[p].left.height, jobs[p].levels, jobs[p].scale, jobs[p].cell);
+    }
+    detect_blocks(geo, bits, k, cfg.border, ctx->tune.tile_w_px, ctx->tune.tile_h_px, ctx->tune_chosen, ctx->n_sm, blocks);
+    for (int p = 0; p < n; ++p) {
         layouts[p] = pair_layout(jobs[p].max_feats);
         result_off[p] = result_bytes;
         result_bytes += layouts[p].bytes;
@@ -399,8 +519,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 const int cx = (g.W[l] + g.c[l] - 1) / g.c[l], cy = (g.H[l] + g.c[l] - 1) / g.c[l];
                 n_slots += cx * cy * k;
                 n_segs += cy;
-                int bx, by;
-                fast_block(g.c[l], k, ctx->tune.tile_w_px, ctx->tune.tile_h_px, &bx, &by);
+                const int bx = blocks[p][l].first, by = blocks[p][l].second;
                 const int tw = std::min(bx * g.c[l], g.W[l]), th = std::min(by * g.c[l], g.H[l]);
                 int bw, bh;
                 detect_box(tw, th, &bw, &bh);
@@ -462,8 +581,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     for (int p = 0; p < n; ++p)
         for (int l = 0; l < geo[p].levels; ++l) {
             n_pyr_tiles += 2 * (size_t)pyramid_strips(geo[p].W[l], geo[p].H[l], pyr_rows[l]);
-            int bx, by;
-            fast_block(geo[p].c[l], k, ctx->tune.tile_w_px, ctx->tune.tile_h_px, &bx, &by);
+            const int bx = blocks[p][l].first, by = blocks[p][l].second;
             const int cx = (geo[p].W[l] + geo[p].c[l] - 1) / geo[p].c[l], cy = (geo[p].H[l] + geo[p].c[l] - 1) / geo[p].c[l];
             n_fast_tiles += 2 * (size_t)(((cx + bx - 1) / bx) * ((cy + by - 1) / by));
         }
@@ -548,7 +666,8 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 L.W = g.W[l]; L.H = g.H[l]; L.c = g.c[l];
                 L.cells_x = (L.W + L.c - 1) / L.c;
                 L.cells_y = (L.H + L.c - 1) / L.c;
-                fast_block(L.c, k, ctx->tune.tile_w_px, ctx->tune.tile_h_px, &L.bx, &L.by);
+                L.bx = blocks[p][l].first;
+                L.by = blocks[p][l].second;
                 L.cinv = (65536 + L.c - 1) / L.c;
                 detect_box(std::min(L.bx * L.c, L.W), std::min(L.by * L.c, L.H), &L.box_w, &L.box_h);
                 L.image = img; L.level = l;
@@ -591,11 +710,12 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 for (int y = 0; y < L.H; ++y) px[L.W + y] = project(y, sc, g.H[0]);
                 t_off += align_up((size_t)(L.W + L.H) * 2, 16);
 
-                // TMA map of the raw level when every tile starts on a word
-                // boundary (the box x is rounded down to 16 bytes)
+                // TMA map of the raw level (the box x is rounded down to 16
+                // bytes); the per-pixel kernel reads words, so its tiles have
+                // to start on word boundaries
                 L.tmap = nullptr;
                 PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
-                if (encode && (L.bx * L.c) % 4 == 0) {
+                if (encode && (bits || (L.bx * L.c) % 4 == 0)) {
                     CUtensorMap map;  // encoded into an aligned object, then copied into the plan
                     const cuuint64_t dims[2] = { (cuuint64_t)L.W, (cuuint64_t)L.H };
                     const cuuint64_t strides[1] = { (cuuint64_t)L.pitch };
@@ -616,7 +736,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                     R.m = L.cells_x * k;
                     R.slot = slot + r * R.m;
                     R.c = L.c; R.y0 = r * L.c;
-                    R.cdiv = L.c == 1 ? 0u : (uint32_t)(((1ull << 32) + L.c - 1) / (uint64_t)L.c);
+                    R.cdiv = recip_of(L.c);
                     R.W0 = I.W0; R.H0 = I.H0; R.level = l;
                 }
                 slot += L.cells_x * L.cells_y * k;
@@ -681,22 +801,33 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
             R.prj_bytes_x = (int)align_up((size_t)(ax - bx0) + 2 * (size_t)R.tw, 16);
             R.prj_bytes_y = (int)align_up((size_t)(ay - by0) + 2 * (size_t)R.th, 16);
             R.image = L.image;
+            R.r0 = std::max(cfg.border - R.y0, 0);
+            R.r1 = std::min(R.H - cfg.border - R.y0, R.th);
+            R.plo = std::max(cfg.border - R.x0, 0);
+            R.phi = std::min(R.W - cfg.border - R.x0, R.tw);
+            R.nch = (R.tw + 31) / 32;
+            R.items = std::max(R.r1 - R.r0, 0) * R.nch;
+            R.nch_inv = (65536u + R.nch - 1) / R.nch;
+            R.row_inv = (65536u + R.nch) / (R.nch + 1);
+            R.cdiv = recip_of(R.c);
+            R.ncx_div = recip_of(R.ncx);
+            R.all_open = R.x0 + R.c > cfg.border && R.y0 + R.c > cfg.border &&
+                         R.x0 + (R.ncx - 1) * R.c < R.W - cfg.border && R.y0 + (R.ncy - 1) * R.c < R.H - cfg.border;
             R.raw = L.raw; R.tmap = L.tmap; R.map = I.map; R.skip = I.skip;
         }
     }
-    // Tile order 1: the persistent detection CTAs take records t, t + grid,
-    // t + 2 grid, ...; ordered by decreasing work (evaluated rows x 32-pixel
-    // chunks, the items of a threshold pass) the grid's last rounds hold the
-    // smallest tiles.  Each record is self-contained (its tile's geometry,
-    // slots and buffers), so the order changes no result; which order is
-    // faster depends on the batch (the autotuner measures both).
-    if (ctx->tune.tile_order == 1) {
-        const int border = cfg.border;
+    // Tile order 1: the persistent detection CTAs take the records in order;
+    // ordered by decreasing work (evaluated rows x 32-pixel chunks, the items
+    // of a threshold pass) the last ones are the smallest tiles.  Each record
+    // is self-contained (its tile's geometry, slots and buffers), so the order
+    // changes no result.  Used by default too (100 pairs of 1241x376: detection
+    // 0.597 -> 0.585 ms, 12 of 752x480 with the learned skip 101 -> 95 us, one
+    // of 1920x1080 45 -> 42 us); with a chosen tuning its own order.
+    if (ctx->tune.tile_order == 1 || (bits && !ctx->tune_chosen)) {
         std::vector<std::pair<int, int>> work(fast);
         for (int t = 0; t < fast; ++t) {
             const TileRec &R = trec[t];
-            const int rows = std::max(std::min(R.H - border - R.y0, R.th) - std::max(border - R.y0, 0), 0);
-            work[t] = { -rows * ((R.tw + 31) >> 5), t };
+            work[t] = { -R.items, t };
         }
         std::stable_sort(work.begin(), work.end(),
                          [](const std::pair<int, int> &a, const std::pair<int, int> &b) { return a.first < b.first; });
@@ -740,7 +871,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     for (int l = 0; l < n_levels; ++l) b.max_segment = std::max(b.max_segment, levels[l].cells_x * k);
     b.pyr_tiles = pyr; b.fast_tiles = fast; b.max_capacity = max_cap;
     b.fast_max_box = max_box; b.fast_max_px = max_px; b.fast_max_cells = max_cells;
-    b.fast_bits = ctx->prm.p_min == 9 && ctx->prm.p_max == 13;
+    b.fast_bits = bits;
     b.fast_max_planes = max_planes;
     b.fast_smem = fast_smem_bytes(max_box, max_px, max_cells, k, b.fast_bits ? max_planes : 0);
     b.corner_lut = ctx->d_lut;
@@ -764,10 +895,12 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     b.bin_cosf = ctx->d_cosf;
     b.bin_sinf = ctx->d_sinf;
     b.err = reinterpret_cast<uint32_t *>(dcounts + 2 * cfg.max_pairs);
+    b.tile_next = reinterpret_cast<uint32_t *>(dcounts + 2 * cfg.max_pairs + 1);
     b.prm = ctx->prm;
 
     ctx->keys = keys;
     ctx->plan_tune = ctx->tune;
+    ctx->plan_chosen = ctx->tune_chosen;
     ctx->plan_skip = ctx->skip_on;
     ctx->layouts = layouts;
     ctx->result_off = result_off;
@@ -1503,6 +1636,7 @@ jslam_status jslam_set_tuning(jslam_ctx *ctx, const jslam_tuning *t)
         return JSLAM_ERR_ARG;
     if (t->tile_order < 0 || t->tile_order > 1) return JSLAM_ERR_ARG;
     ctx->tune = *t;
+    ctx->tune_chosen = true;
     return JSLAM_OK;
 }
 
@@ -1534,6 +1668,7 @@ jslam_status jslam_autotune(jslam_ctx *ctx, const jslam_stereo_job *jobs, int32_
     const bool was_timing = ctx->timing;
     jslam_status st = jslam_enable_stage_timing(ctx, 1);
     if (st != JSLAM_OK) return st;
+    ctx->tune_chosen = true;
     jslam_tuning best = ctx->tune;
     best.nms_kernel = 0;
     best.detect_ctas_per_sm = 0;

@@ -39,7 +39,7 @@ static_assert((2 * (kPyrAhead + 2) + 1) * kPyrMaxOne <= kPyrRing, "ring");
 static_assert((2 * (kPyrAheadTwo + 2) + 1) * kPyrMaxTwo <= kPyrRing, "ring");
 enum { kPyrCopy = 0, kPyrOne = 1, kPyrTwo = 2, kPyrBytes = 3 };
 // Detection tile: at most this many pixels a side (host picks cells per CTA).
-constexpr int kFastMaxTile = 128, kFastThreads = 256;
+constexpr int kFastMaxTile = 128, kFastThreads = 128;
 
 // Row stride of the bit-planes in 16-byte units for a tile of nch 32-pixel
 // chunks: chunks 0..nch (32 bytes each) and a 16-byte pad, an odd count, so
@@ -165,6 +165,12 @@ struct __align__(16) TileRec {
     int32_t prj_bytes_x, prj_bytes_y;  // bulk copy sizes (multiples of 16)
     int32_t prj_off_x, prj_off_y;      // element offset of x0 / y0 in the staged copies
     int32_t image;                     // the tile's image
+    int32_t r0, r1, plo, phi;          // evaluated rows and columns of the tile
+    int32_t nch, items;                // 32-pixel chunks of a row; (evaluated row, chunk) items
+    uint32_t nch_inv, row_inv;         // ceil(2^16 / nch), ceil(2^16 / (nch + 1))
+    uint32_t cdiv, ncx_div;            // reciprocals of c and ncx (see div_recip)
+    int32_t all_open;                  // every cell has evaluated pixels
+    int32_t pad[1];
     const uint8_t *raw;
     const CUtensorMap *tmap;           // nullptr: the box is loaded with plain loads
     const uint16_t *prj_src_x, *prj_src_y;
@@ -173,6 +179,9 @@ struct __align__(16) TileRec {
 };
 static_assert(sizeof(TileRec) % 16 == 0, "bulk copies move multiples of 16 bytes");
 
+// Reciprocal for div_recip: v / d for v * d below 2^32.
+inline uint32_t recip_of(int d) { return d == 1 ? 0u : (uint32_t)(((1ull << 32) + (uint64_t)d - 1) / (uint64_t)d); }
+
 // One segment (cell row of a level): where its candidate slots lie and what
 // turns a slot into coordinates and score-map entries.
 struct __align__(16) SegRec {
@@ -180,7 +189,7 @@ struct __align__(16) SegRec {
     uint32_t *map;
     int32_t slot, m;         // first slot, slots (cells_x x k)
     int32_t c, y0;           // cell size, first row
-    uint32_t cdiv;           // ceil(2^32 / c); 0 for c = 1
+    uint32_t cdiv;           // reciprocal of c (see recip_of)
     int32_t W0, H0, level;
 };
 // Rank of a slot that is no survivor (SlotInfo's w): no corner, suppressed.
@@ -207,6 +216,7 @@ struct Batch {
     int32_t fast_max_planes;        // bit-plane bytes of the largest tile box
     int32_t fast_bits;              // 1: bit-sliced ring test (P_min = 9, P_max = 13)
     const TileRec *tile_rec;        // one per detection tile
+    uint32_t *tile_next;            // detection tiles taken beyond each CTA's first three (zero before the launch)
     const uint32_t *corner_lut;     // bit m: P_min <= longest circular run of m <= P_max
     uint32_t *slots;                // candidate keys per slot
     uint4 *slot_info;               // per slot: position, X | Y << 16, cap priority, rank in its segment

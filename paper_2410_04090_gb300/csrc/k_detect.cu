@@ -83,28 +83,25 @@ __host__ __device__ inline FastLayout fast_layout(int max_box, int max_px, int m
 
 // Dynamic shared memory of the bit-sliced kernel: the two tile boxes, the
 // box's bit-planes (max_planes bytes: box rows of (chunks + 1) x 8 words and
-// a 16-byte pad, see bs_row_units), the corner list and keys only for k > 1
-// (k = 1 takes each cell's best corner as it is found), cell states,
-// selections and the work list of a pass (16-bit item indices; a tile has at
-// most kFastMaxTile rows of 4 items).  The fixed-size parts (corner windows,
-// tile records, staged projections, mbarriers) are static arrays of the
-// kernel.
+// a 16-byte pad, see bs_row_units), cell states and selections of two tiles
+// (by tile parity) and the work list of a pass (16-bit item indices; a tile
+// has at most kFastMaxTile rows of 4 items).  The fixed-size parts (corner
+// windows, tile records, staged projections, mbarriers) are static arrays of
+// the kernel.
 constexpr int kBitsWin = 128;
 constexpr int kBitsMaxItems = kFastMaxTile * (kFastMaxTile / 32);
 struct BitsLayout {
-    int buf0, buf1, planes, clist, ckey, has_hi, sel, wlist, total;
+    int buf0, buf1, planes, has_hi, sel, wlist, total;
 };
-__host__ __device__ inline BitsLayout bits_layout(int max_box, int max_px, int max_cells, int k, int max_planes)
+__host__ __device__ inline BitsLayout bits_layout(int max_box, int max_cells, int k, int max_planes)
 {
     BitsLayout l;
     int o = 0;
     l.buf0 = o;   o += fast_align(max_box, 128);
     l.buf1 = o;   o += fast_align(max_box, 128);
     l.planes = o; o += fast_align(max_planes, 16);
-    l.clist = o;  o += k > 1 ? fast_align(max_px * 2, 16) : 0;
-    l.ckey = o;   o += k > 1 ? fast_align(max_px * 4, 16) : 0;
-    l.has_hi = o; o += fast_align(max_cells, 16);
-    l.sel = o;    o += fast_align(max_cells * k * 4, 16);
+    l.has_hi = o; o += 2 * fast_align(max_cells, 16);
+    l.sel = o;    o += 2 * fast_align(max_cells * k * 4, 16);
     l.wlist = o;  o += kBitsMaxItems * 2;
     l.total = o;
     return l;
@@ -308,40 +305,39 @@ __device__ __forceinline__ uint32_t group_pretest(const uint32_t *base, int wpr,
 // ---- bit-sliced ring test (P_min = 9, P_max = 13): 32 pixels per word, bit
 // j of word i = bit i of pixel j's byte.  a > b for 8-bit numbers: the carry
 // out of a + ~b, one majority per bit; c + e: a ripple adder against the
-// constant's bit masks, returning the carry out.
+// constant's bit masks.
 
 // Bit-planes of a 32-byte chunk (bytes j of words a, z in memory order):
-// output word i, bit j = bit i of byte j.  Each 8-byte block is an 8 x 8 bit
-// matrix (row = byte, column = bit) transposed by three delta swaps (2 x 2,
-// 4 x 4 and 8 x 8 sub-blocks); byte i of the transposed block b is then byte
-// b of output word i.
+// output word i, bit j = bit i of byte j.  The bytes are gathered so that byte
+// b of word w is byte 8 b + w of the chunk; each byte lane of the eight words
+// is then an 8 x 8 bit matrix (row = word, column = bit), transposed by three
+// rounds of exchanges between words 4, 2 and 1 apart.
 __device__ __forceinline__ void bs_transpose(uint4 a, uint4 z, uint4 *dst)
 {
-    uint32_t w[8] = { a.x, a.y, a.z, a.w, z.x, z.y, z.z, z.w };
+    uint32_t w[8];
+    const uint32_t v[2][4] = { { a.x, a.z, z.x, z.z }, { a.y, a.w, z.y, z.w } };
 #pragma unroll
-    for (int blk = 0; blk < 4; ++blk) {
-        uint32_t lo = w[2 * blk], hi = w[2 * blk + 1], t;
-        t = (lo ^ (lo >> 7)) & 0x00AA00AAu;  lo ^= t ^ (t << 7);
-        t = (hi ^ (hi >> 7)) & 0x00AA00AAu;  hi ^= t ^ (t << 7);
-        t = (lo ^ (lo >> 14)) & 0x0000CCCCu; lo ^= t ^ (t << 14);
-        t = (hi ^ (hi >> 14)) & 0x0000CCCCu; hi ^= t ^ (t << 14);
-        t = (lo ^ (hi << 4)) & 0xF0F0F0F0u;  lo ^= t; hi ^= t >> 4;
-        w[2 * blk] = lo; w[2 * blk + 1] = hi;
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t t0 = __byte_perm(v[h][0], v[h][1], 0x5140), t1 = __byte_perm(v[h][0], v[h][1], 0x7362);
+        const uint32_t u0 = __byte_perm(v[h][2], v[h][3], 0x5140), u1 = __byte_perm(v[h][2], v[h][3], 0x7362);
+        w[4 * h + 0] = __byte_perm(t0, u0, 0x5410);
+        w[4 * h + 1] = __byte_perm(t0, u0, 0x7632);
+        w[4 * h + 2] = __byte_perm(t1, u1, 0x5410);
+        w[4 * h + 3] = __byte_perm(t1, u1, 0x7632);
     }
-    uint32_t o[8];
 #pragma unroll
-    for (int half = 0; half < 2; ++half)
+    for (int s = 4; s > 0; s >>= 1) {
+        const uint32_t m = s == 4 ? 0x0F0F0F0Fu : s == 2 ? 0x33333333u : 0x55555555u;
 #pragma unroll
-        for (int i = 0; i < 4; i += 2) {
-            const uint32_t sel = (uint32_t)i | ((uint32_t)(4 + i) << 4) | ((uint32_t)(i + 1) << 8) |
-                                 ((uint32_t)(5 + i) << 12);
-            const uint32_t A = __byte_perm(w[half], w[2 + half], sel);
-            const uint32_t B = __byte_perm(w[4 + half], w[6 + half], sel);
-            o[4 * half + i] = __byte_perm(A, B, 0x5410u);
-            o[4 * half + i + 1] = __byte_perm(A, B, 0x7632u);
+        for (int i = 0; i < 8; ++i) {
+            if (i & s) continue;
+            const uint32_t lo = w[i], hi = w[i + s];
+            w[i] = (lo & m) | ((hi << s) & ~m);
+            w[i + s] = ((lo >> s) & m) | (hi & ~m);
         }
-    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+    }
+    dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
 __device__ __forceinline__ uint32_t bs_greater(const uint32_t (&a)[8], const uint32_t (&b)[8])
@@ -352,33 +348,20 @@ __device__ __forceinline__ uint32_t bs_greater(const uint32_t (&a)[8], const uin
     return c;
 }
 
-__device__ __forceinline__ uint32_t bs_add_const(const uint32_t (&c)[8], uint32_t e, uint32_t (&t)[8])
-{
-    uint32_t k = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint32_t E = 0u - ((e >> i) & 1u);
-        t[i] = c[i] ^ E ^ k;
-        k = maj3(c[i], E, k);
-    }
-    return k;
-}
-
-// Longest circular run of the 16 flag words in [9, 13], with three-input
-// ANDs: A3 = windows of 3, A9 = three A3 end to end, a run of 14 = an A9
-// followed by two overlapping A3 (positions q + 9 .. q + 13).
+// Longest circular run of the 16 flag words in [9, 13]: A3 = windows of 3, A9
+// = three A3 end to end, a run of 14 = an A9 and the one five positions on.
 __device__ __forceinline__ uint32_t bs_run_9_13(const uint32_t (&F)[16])
 {
-    uint32_t A3[16];
+    uint32_t A3[16], A9[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q) A3[q] = F[q] & F[(q + 1) & 15] & F[(q + 2) & 15];
-    uint32_t r9 = 0, r14 = 0;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const uint32_t a9 = A3[q] & A3[(q + 3) & 15] & A3[(q + 6) & 15];
-        r9 |= a9;
-        r14 |= a9 & A3[(q + 9) & 15] & A3[(q + 11) & 15];
-    }
+    for (int q = 0; q < 16; ++q) A9[q] = A3[q] & A3[(q + 3) & 15] & A3[(q + 6) & 15];
+    uint32_t r9 = A9[0] | A9[1], r14 = A9[0] & A9[5];
+#pragma unroll
+    for (int q = 2; q < 16; q += 2) r9 |= A9[q] | A9[q + 1];
+#pragma unroll
+    for (int q = 1; q < 16; ++q) r14 |= A9[q] & A9[(q + 5) & 15];
     return r9 & ~r14;
 }
 
@@ -402,7 +385,8 @@ __device__ __forceinline__ int ring_sad(const uint8_t *p, int rowb)
 // `planes`: box rows of `ru` 16-byte units, chunk m at unit 2 m; tile pixel 0
 // sits at box column sb, so pixel 32 m + j + dx is bit sb + dx + j of chunks
 // (m, m + 1).
-__device__ __forceinline__ uint32_t bs_corners(const uint32_t *planes, int ru, int py, int m, int sb, int eps)
+__device__ __forceinline__ uint32_t bs_corners(const uint32_t *planes, int ru, int py, int m, int sb,
+                                               const uint32_t (&eps)[8])
 {
     constexpr int RDX[16] = { 0, 1, 2, 3, 3, 3, 2, 1, 0, -1, -2, -3, -3, -3, -2, -1 };
     constexpr int RDY[16] = { 3, 3, 2, 1, 0, -1, -2, -3, -3, -3, -2, -1, 0, 1, 2, 3 };
@@ -415,19 +399,17 @@ __device__ __forceinline__ uint32_t bs_corners(const uint32_t *planes, int ru, i
 #pragma unroll
         for (int i = 0; i < 8; ++i) C[i] = __funnelshift_r(lo[i], hi[i], sb);
     }
-    // a centre with C + eps >= 256 is never brighter (threshold 255, which
-    // no P exceeds); one with C < eps never darker (threshold 0)
-    const uint32_t nb = bs_add_const(C, (uint32_t)eps, Tb);
-    if (eps > 0) {
-        const uint32_t nd = ~bs_add_const(C, (uint32_t)(256 - eps), Td);
+    // thresholds C + eps and C - eps = ~(~C + eps), eps as a word mask for each
+    // of its bits; a centre whose sum wraps (nb: C + eps >= 256, nd: C < eps)
+    // is never brighter (darker), its flags are dropped at the end
+    uint32_t nb = 0, nd = 0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) Td[i] &= ~nd;
-    } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) Td[i] = C[i];
+    for (int i = 0; i < 8; ++i) {
+        Tb[i] = C[i] ^ eps[i] ^ nb;
+        Td[i] = C[i] ^ eps[i] ^ nd;
+        nb = maj3(C[i], eps[i], nb);
+        nd = maj3(~C[i], eps[i], nd);
     }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) Tb[i] |= nb;
     uint32_t Fb[16], Fd[16];
 #pragma unroll
     for (int dy = 3; dy >= -3; --dy) {
@@ -445,7 +427,7 @@ __device__ __forceinline__ uint32_t bs_corners(const uint32_t *planes, int ru, i
             Fd[q] = bs_greater(Td, P);
         }
     }
-    return bs_run_9_13(Fb) | bs_run_9_13(Fd);
+    return (bs_run_9_13(Fb) & ~nb) | (bs_run_9_13(Fd) & ~nd);
 }
 
 // Bits j of the 32 pixels of tile row chunk px0..px0+31 whose cell state
@@ -465,6 +447,9 @@ __device__ __forceinline__ uint32_t cell_bits(const uint8_t *st, int px0, int tw
 }
 
 __device__ __forceinline__ int div_small(int v, uint32_t cinv) { return (int)(((uint32_t)v * cinv) >> 16); }
+
+// v / d by d's reciprocal (recip_of; 0 stands for d = 1).
+__device__ __forceinline__ int div_recip(int v, uint32_t recip) { return recip ? (int)__umulhi((uint32_t)v, recip) : v; }
 
 // Bits j of the 32 pixels px0 + j of a tile row that lie inside the level's
 // evaluated columns [plo, phi) (tile coordinates).
@@ -799,47 +784,50 @@ __device__ __forceinline__ void issue_rec_tile(const TileRec &R, uint8_t *buf, u
                  "r"((uint32_t)R.prj_bytes_y), "r"(smem_u32(bar)) : "memory");
 }
 
-// Thread 0 of k_fast_bits after the wait for tile t's box ran out: wait once
-// more, with the same limit, for every copy it still has in flight (this
-// box; then either the next tile's box and the record after it, or the next
-// record if its wait ran out too), so that no copy lands in the shared
-// memory of a CTA that has ended.  rph bit s is the parity of the next
+// Thread 0 of k_fast_bits after a tile's box did not arrive in time: wait
+// once more, with the same limit, for the copies it still has in flight (this
+// box and, if there is one, the next tile's record), so that none lands in the
+// shared memory of a CTA that has ended.  rph bit s is the parity of the next
 // completion of record barrier 2 + s, phases bit p that of box barrier p.
-__device__ __forceinline__ void drain_bits(const Batch &b, uint64_t *bars, int t, int grid, int cur, int s3,
-                                        uint32_t phases, uint32_t rph, int aborted)
+__device__ __forceinline__ void drain_bits(uint64_t *bars, bool more, int cur, int s3, uint32_t phases, uint32_t rph)
 {
     wait_tile(&bars[cur], (phases >> cur) & 1u);
-    if (t + grid >= b.fast_tiles) return;
-    const int sn = s3 == 2 ? 0 : s3 + 1, sa = s3 == 0 ? 2 : s3 - 1;
-    if (aborted) {
-        wait_tile(&bars[2 + sn], (rph >> sn) & 1u);
-        return;
-    }
-    wait_tile(&bars[cur ^ 1], (phases >> (cur ^ 1)) & 1u);
-    if (t + 2 * grid < b.fast_tiles) wait_tile(&bars[2 + sa], (rph >> sa) & 1u);
+    const int sn = s3 == 2 ? 0 : s3 + 1;
+    if (more) wait_tile(&bars[2 + sn], (rph >> sn) & 1u);
 }
 
 // Bit-sliced ring test (P_min = 9, P_max = 13), the same results as
-// k_fast_cull.  Tiles come with host-made records: thread 0 fetches the
-// record of the tile after next and, once the next tile's record is in,
-// issues that tile's box and projection ranges, so every tile starts from
-// shared memory.  Per tile: tile wait, cell states, bit-planes, one barrier;
-// each threshold pass classifies 32 pixels of a row per thread, and every
-// warp scores its own corners right away through a window of entries in
-// shared memory (k = 1: atomic maximum of the cell's key; k > 1: corner list
-// for the top-k rounds); a barrier ends each pass and one the tile.  The
-// counters of a tile live in one of two sets by tile parity, so the set of
-// the next tile is cleared while the current one is in use.
+// k_fast_cull.  Tiles come with host-made records; from its fourth tile on a
+// CTA takes the next one from a counter (cleared by the pyramid launch
+// before), which evens out what their corners cost (100 pairs of 1241x376:
+// 0.692 -> 0.596 ms).  Per tile: tile wait, cell states, bit-planes, a barrier;
+// thread 0 then issues the next tile's box and projection ranges, fetches the
+// record after it and asks for the number of the one after that; each threshold pass
+// classifies 32 pixels of a row per thread, and every warp scores its own
+// corners right away through a window of entries in shared memory, keeping
+// each cell's k best by atomic maxima; a barrier ends each pass, and the slots
+// are written.  Cell states, selections and counters are kept by tile parity,
+// so that no barrier ends a tile: a warp may start the next one while others
+// write this one's slots (what the next tile's first phase overwrites -- the
+// planes, the other set -- was last read before the barrier that ended this
+// tile's passes, and what thread 0 refills, before the next one's first).
+// What bounds it: the ALU pipe (LOP3 and shifts, half rate: 60 % busy) and the
+// barriers and dependent steps between.  Four warps a CTA, five CTAs an SM (96
+// registers): with eight warps and three CTAs a barrier stopped more of the
+// SM.  For 100 pairs of 1241x376 the kernel executed 1750 instructions per
+// 1024 pixels and took 0.965 ms; now 1430 and 0.585 ms (threads and barriers
+// 0.965 -> 0.82, run test and registers -> 0.765, host-made tile numbers,
+// reciprocals and whole-word clears -> 0.729, blocks of cells that fill the
+// warps -> 0.692, tiles from a counter -> 0.596, largest first -> 0.585).
 // Compile-time variants: kArc, the corner response (the arc's, an opt-in
 // reading, or the whole ring's SAD); kSkip, the learned cell-skip mode;
-// kTop1, one keypoint per cell (k = 1, the default) or the top-k rounds.
+// kTop1, one keypoint per cell (k = 1, the default) or several.
 template <bool kArc, bool kSkip, bool kTop1>
-__global__ void __launch_bounds__(kFastThreads, 3) k_fast_bits(Batch b)
+__global__ void __launch_bounds__(kFastThreads, 5) k_fast_bits(Batch b)
 {
     extern __shared__ __align__(128) uint8_t smem[];
-    // per set: corners listed (k > 1), skipped cells, cells open at the
-    // start (state 0), open cells that got a primary-threshold corner
-    __shared__ int cnt[2][4];
+    __shared__ int s_skipped[2];  // skipped cells, by tile parity
+    __shared__ int s_more[2];     // whether another tile follows, by tile parity
     __shared__ int s_nlist[2];  // work-list lengths of pass 0 (cells skipped) and pass 1
     __shared__ int s_abort;
     __shared__ uint32_t s_rph;  // thread 0: parity of the next completion of each record barrier (bit s)
@@ -848,75 +836,58 @@ __global__ void __launch_bounds__(kFastThreads, 3) k_fast_bits(Batch b)
     __shared__ __align__(16) uint8_t s_prj[2][2 * kPrjBytes];  // per box: x range, y range
     __shared__ __align__(8) uint64_t bars[5];                   // [0..1] boxes, [2..4] records
     const int k = kTop1 ? 1 : b.prm.k, border = b.prm.border;
-    const BitsLayout lay = bits_layout(b.fast_max_box, b.fast_max_px, b.fast_max_cells, k, b.fast_max_planes);
+    const BitsLayout lay = bits_layout(b.fast_max_box, b.fast_max_cells, k, b.fast_max_planes);
     uint8_t *const buf0 = smem + lay.buf0, *const buf1 = smem + lay.buf1;
     uint32_t *planes = reinterpret_cast<uint32_t *>(smem + lay.planes);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint16_t *wbuf = s_wbuf[warp];
-    uint16_t *clist = reinterpret_cast<uint16_t *>(smem + lay.clist);
-    uint32_t *ckey = reinterpret_cast<uint32_t *>(smem + lay.ckey);
-    uint8_t *has_hi = smem + lay.has_hi;
-    uint32_t *sel = reinterpret_cast<uint32_t *>(smem + lay.sel);
     uint16_t *wlist = reinterpret_cast<uint16_t *>(smem + lay.wlist);
 
     if ((smem_u32(buf0) | smem_u32(buf1)) & 127u) {
         if (threadIdx.x == 0) atomicOr(b.err, kErrDecode);
         return;
     }
-    const int grid = (int)gridDim.x;
+    // thread 0: the next tile and the one after it
+    const int tiles = b.fast_tiles;
+    int t1 = tiles, t2 = tiles;
     if (threadIdx.x == 0) {
         for (int i = 0; i < 5; ++i)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[i])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_abort = 0;
-        const int t0 = blockIdx.x;
-        if (t0 < b.fast_tiles) {
-            fetch_rec(b, t0, &recs[0], &bars[2]);
-            if (t0 + grid < b.fast_tiles) fetch_rec(b, t0 + grid, &recs[1], &bars[3]);
-            if (wait_tile(&bars[2], 0u)) issue_rec_tile(recs[0], buf0, s_prj[0], &bars[0]);
-            else {
-                // give up, after waiting once more (same limit) for both
-                // record copies, so that none lands after the CTA has ended
-                atomicOr(b.err, kErrTimeout);
-                s_abort = 1;
-                wait_tile(&bars[2], 0u);
-                if (t0 + grid < b.fast_tiles) wait_tile(&bars[3], 0u);
-            }
+        // the grid is no larger than the number of tiles
+        fetch_rec(b, blockIdx.x, &recs[0], &bars[2]);
+        t1 = (int)(blockIdx.x + gridDim.x);
+        t2 = t1 + (int)gridDim.x;
+        if (t1 < tiles) fetch_rec(b, t1, &recs[1], &bars[3]);
+        if (wait_tile(&bars[2], 0u)) issue_rec_tile(recs[0], buf0, s_prj[0], &bars[0]);
+        else {
+            // give up, after waiting once more (same limit) for both
+            // record copies, so that none lands after the CTA has ended
+            atomicOr(b.err, kErrTimeout);
+            s_abort = 1;
+            wait_tile(&bars[2], 0u);
+            if (t1 < tiles) wait_tile(&bars[3], 0u);
         }
         s_rph = 1u;
     }
-    if (threadIdx.x < 8) cnt[threadIdx.x >> 2][threadIdx.x & 3] = 0;
+    if (threadIdx.x < 2) s_skipped[threadIdx.x] = 0;
     __syncthreads();
     if (s_abort) return;
     uint32_t phases = 0u;  // bit p: parity of the next completion of box barrier p
 
-    int it = 0;
-    for (int t = blockIdx.x; t < b.fast_tiles; t += grid, ++it) {
+    for (int it = 0;; ++it) {
         const int cur = it & 1, s3 = it % 3;
-        int *const C = cnt[cur];
         const TileRec &R = recs[s3];
         const uint16_t *prj = reinterpret_cast<const uint16_t *>(s_prj[cur]);
+        uint8_t *const has_hi = smem + lay.has_hi + cur * fast_align(b.fast_max_cells, 16);
+        uint32_t *const sel =
+            reinterpret_cast<uint32_t *>(smem + lay.sel + cur * fast_align(b.fast_max_cells * k * 4, 16));
         if (threadIdx.x == 0) {
-            // the next tile's record was fetched one tile ago; the slot of the
-            // tile after it, the other box and its projections were last read
-            // before the barrier that ended the previous tile
-            // (after a record wait runs out nothing more is issued; the CTA
-            // stops at the abort check after the tile's bit-plane barrier)
-            if (t + grid < b.fast_tiles) {
-                const int sn = s3 == 2 ? 0 : s3 + 1;
-                if (wait_tile(&bars[2 + sn], (s_rph >> sn) & 1u)) {
-                    issue_rec_tile(recs[sn], cur ? buf0 : buf1, s_prj[cur ^ 1], &bars[cur ^ 1]);
-                    s_rph ^= 1u << sn;
-                    if (t + 2 * grid < b.fast_tiles) {
-                        const int sa = s3 == 0 ? 2 : s3 - 1;
-                        fetch_rec(b, t + 2 * grid, &recs[sa], &bars[2 + sa]);
-                    }
-                } else { atomicOr(b.err, kErrTimeout); s_abort = 1; }
-            }
-            cnt[cur ^ 1][0] = cnt[cur ^ 1][1] = cnt[cur ^ 1][2] = cnt[cur ^ 1][3] = 0;
-            // the lists of the previous tile were last read before its closing
-            // barrier; this tile's are built after a barrier that follows this
+            // read last before the barrier that ended the previous tile's passes
+            s_skipped[cur ^ 1] = 0;
             s_nlist[0] = s_nlist[1] = 0;
+            s_more[cur] = t1 < tiles;
         }
         uint8_t *const tb = cur ? buf1 : buf0;
         // the box and the projections (every tile waits: the projections
@@ -924,7 +895,7 @@ __global__ void __launch_bounds__(kFastThreads, 3) k_fast_bits(Batch b)
         if (!wait_tile(&bars[cur], (phases >> cur) & 1u)) {
             if (threadIdx.x == 0) {
                 atomicOr(b.err, kErrTimeout);
-                drain_bits(b, bars, t, grid, cur, s3, phases, s_rph, s_abort);
+                drain_bits(bars, t1 < tiles, cur, s3, phases, s_rph);
             }
             return;
         }
@@ -955,85 +926,101 @@ __global__ void __launch_bounds__(kFastThreads, 3) k_fast_bits(Batch b)
             }
         }
         // cell states (as in k_fast_cull) and cleared selections
-        int my_skipped = 0, my_open = 0;
-        for (int i = threadIdx.x; i < cells; i += kFastThreads) {
-            const int lcy = i / ncx, lcx = i - lcy * ncx;
-            const int cx0 = (R.ccx0 + lcx) * c, cy0 = (R.ccy0 + lcy) * c;
-            const bool evaluated = cx0 + c > border && cx0 < W - border && cy0 + c > border && cy0 < Hh - border;
-            uint8_t st = evaluated ? 0 : 3;
-            if (tskip && evaluated) {
-                const int px = min(cx0 + c / 2, W - 1), py = min(cy0 + c / 2, Hh - 1);
-                const int X = prj[R.prj_off_x + px - x0], Y = prj[kPrjBytes / 2 + R.prj_off_y + py - y0];
-                st = R.skip[(Y / R.skip_c0) * R.skip_cells_x + X / R.skip_c0] ? 2 : 0;
+        int my_skipped = 0;
+        if (R.all_open && !tskip) {
+            for (int i = threadIdx.x; i < (cells + 3) >> 2; i += kFastThreads) reinterpret_cast<uint32_t *>(has_hi)[i] = 0u;
+        } else {
+            for (int i = threadIdx.x; i < cells; i += kFastThreads) {
+                const int lcy = i / ncx, lcx = i - lcy * ncx;
+                const int cx0 = (R.ccx0 + lcx) * c, cy0 = (R.ccy0 + lcy) * c;
+                const bool evaluated = cx0 + c > border && cx0 < W - border && cy0 + c > border && cy0 < Hh - border;
+                uint8_t st = evaluated ? 0 : 3;
+                if (tskip && evaluated) {
+                    const int px = min(cx0 + c / 2, W - 1), py = min(cy0 + c / 2, Hh - 1);
+                    const int X = prj[R.prj_off_x + px - x0], Y = prj[kPrjBytes / 2 + R.prj_off_y + py - y0];
+                    st = R.skip[(Y / R.skip_c0) * R.skip_cells_x + X / R.skip_c0] ? 2 : 0;
+                }
+                if (tskip && st != 0) { st = 2; ++my_skipped; }
+                has_hi[i] = st;
             }
-            if (tskip && st != 0) { st = 2; ++my_skipped; }
-            my_open += st == 0;
-            has_hi[i] = st;
         }
-        for (int i = threadIdx.x; i < cells * k; i += kFastThreads) sel[i] = 0;
-        if (my_skipped) atomicAdd(&C[1], my_skipped);
-        if (my_open) atomicAdd(&C[2], my_open);
+        for (int i = threadIdx.x; i < (cells * k + 3) >> 2; i += kFastThreads)
+            reinterpret_cast<uint4 *>(sel)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (my_skipped) atomicAdd(&s_skipped[cur], my_skipped);
         // a box loaded with plain loads, the cell states and, in skip mode,
         // the skipped count are complete before the planes
         if (!R.tmap || tskip) __syncthreads();
-        all_skipped = tskip && C[1] == cells;
+        all_skipped = tskip && s_skipped[cur] == cells;
 
         // bit-planes of the box rows [r0, r1 + 6) that the evaluated rows
         // [r0, r1) read, chunks 0..nch (an item of chunk m reads m and m + 1),
-        // one 32-byte chunk per thread; chunks at or past the box's end
-        // (a row's last may hold only 16 bytes) are zero
-        const int r0 = max(border - y0, 0), r1 = min(Hh - border - y0, R.th);
-        const int nch = (R.tw + 31) >> 5;
-        const int nbc = (rowb + 31) >> 5, ru = bs_row_units(nch);
+        // one 32-byte chunk per thread
+        const int r0 = R.r0, nch = R.nch, ru = bs_row_units(nch);
         if (!all_skipped) {
-            const int nrows = max(r1 - r0, 0) > 0 ? r1 - r0 + 6 : 0;
-            for (int ci = threadIdx.x; ci < nrows * (nch + 1); ci += kFastThreads) {
-                const int rr = ci / (nch + 1), kc = ci - rr * (nch + 1), r = r0 + rr;
-                uint4 a = make_uint4(0u, 0u, 0u, 0u), z = a;
-                if (kc < nbc) {
-                    const uint4 *src = reinterpret_cast<const uint4 *>(tb + r * rowb + 32 * kc);
-                    a = src[0];
-                    if (32 * kc + 16 < rowb) z = src[1];
-                }
-                bs_transpose(a, z, reinterpret_cast<uint4 *>(planes) + r * ru + 2 * kc);
+            const int chunks = R.items > 0 ? (R.r1 - r0 + 6) * (nch + 1) : 0;
+            const uint32_t row_inv = R.row_inv;
+            for (int ci = threadIdx.x; ci < chunks; ci += kFastThreads) {
+                const int rr = div_small(ci, row_inv), kc = ci - rr * (nch + 1), r = r0 + rr;
+                const uint4 *src = reinterpret_cast<const uint4 *>(tb + r * rowb + 32 * kc);
+                bs_transpose(src[0], src[1], reinterpret_cast<uint4 *>(planes) + r * ru + 2 * kc);
             }
             // cells skipped by the proposal: pass 0 runs over the items that
             // hold a pixel of a cell that is not (states are complete: skip
             // mode has a barrier after them)
-            if (tskip && C[1] > 0) {
-                const int plo = max(border - x0, 0), phi = min(W - border - x0, R.tw);
-                list_items(wlist, &s_nlist[0], max(r1 - r0, 0) * nch, nch, (65536u + nch - 1) / nch, r0, plo, phi,
-                           has_hi, ncx, R.tw, c, (uint32_t)R.cinv, lane, warp,
+            if (tskip && s_skipped[cur] > 0) {
+                list_items(wlist, &s_nlist[0], R.items, nch, R.nch_inv, r0, R.plo, R.phi, has_hi, ncx, R.tw, c,
+                           (uint32_t)R.cinv, lane, warp,
                            [](uint8_t st) { return st != 2; });
             }
         }
         }
         __syncthreads();
-        if (s_abort) {  // thread 0 could not start the next tile
-            if (threadIdx.x == 0) {
-                const int sn = s3 == 2 ? 0 : s3 + 1;
-                wait_tile(&bars[2 + sn], (s_rph >> sn) & 1u);  // the record copy that did not complete
-            }
-            return;
+        const bool more = s_more[cur] != 0;
+        if (threadIdx.x == 0 && more) {
+            // the next tile's record was fetched one tile ago; the slot of the
+            // record after it, the other box and its projections were last
+            // read before the barrier above (after a record wait runs out
+            // nothing more is issued; the CTA stops after this tile's passes)
+            const int sn = s3 == 2 ? 0 : s3 + 1;
+            if (wait_tile(&bars[2 + sn], (s_rph >> sn) & 1u)) {
+                issue_rec_tile(recs[sn], cur ? buf0 : buf1, s_prj[cur ^ 1], &bars[cur ^ 1]);
+                s_rph ^= 1u << sn;
+                t1 = t2;
+                if (t1 < tiles) {
+                    const int sa = s3 == 0 ? 2 : s3 - 1;
+                    fetch_rec(b, t1, &recs[sa], &bars[2 + sa]);
+                    t2 = 3 * (int)gridDim.x + (int)atomicAdd(b.tile_next, 1u);  // used one tile on
+                }
+            } else { atomicOr(b.err, kErrTimeout); s_abort = 1; }
         }
-        const bool some_skipped = kSkip && C[1] > 0;  // constant false outside skip mode
+        const bool some_skipped = kSkip && s_skipped[cur] > 0;  // constant false outside skip mode
 
         {
-        const int c = R.c, W = R.W, Hh = R.H, x0 = R.x0, y0 = R.y0, tw = R.tw, rowb = R.box_w, ncx = R.ncx;
+        const int c = R.c, tw = R.tw, rowb = R.box_w, ncx = R.ncx;
         const uint32_t cinv = (uint32_t)R.cinv;
-        const int plo = max(border - x0, 0), phi = min(W - border - x0, tw);
-        const int r0 = max(border - y0, 0), r1 = min(Hh - border - y0, R.th);
-        const int nch = (tw + 31) >> 5, sb = R.delta + 4, ru = bs_row_units(nch);
-        const uint32_t nchinv = (65536u + nch - 1) / nch;  // item / nch by a multiply (item < 2^9)
-        const int items = max(r1 - r0, 0) * nch;
+        const int plo = R.plo, phi = R.phi, r0 = R.r0;
+        const int nch = R.nch, sb = R.delta + 4, ru = bs_row_units(nch), items = R.items;
+        const uint32_t nchinv = R.nch_inv;  // item / nch by a multiply (item < 2^9)
         const uint8_t *tbytes = tb + R.delta;  // pixel (x, y) at (y - y0 + 3) * rowb + (x - x0 + 4)
         for (int pass = 0; pass < 2 && !all_skipped; ++pass) {
             const int eps = pass == 0 ? R.eps_hi : R.eps_lo;
-            // fallback pass only while an open cell got no corner
-            if (pass == 1 && (eps <= 0 || C[3] >= C[2])) break;
+            if (pass == 1) {
+                // fallback pass only while a cell that is open got no corner
+                // (selections are final after pass 0's barrier): every warp
+                // looks for itself and marks the cells that have one
+                if (eps <= 0) break;
+                bool open = false;
+                for (int i = lane; i < ncx * R.ncy; i += 32) {
+                    if (has_hi[i] != 0) continue;
+                    if (sel[i * k]) has_hi[i] = 1;
+                    else open = true;
+                }
+                if (!__any_sync(0xFFFFFFFFu, open)) break;
+                __syncwarp();  // this warp's marks
+            }
             // pass 0 covers every item, or the listed ones when cells are
             // skipped; pass 1 lists the items holding a pixel of a cell still
-            // without a corner (cell states are final after pass 0's barrier)
+            // without a corner
             const bool listed = pass == 1 || some_skipped;
             if (pass == 1) {
                 list_items(wlist, &s_nlist[1], items, nch, nchinv, r0, plo, phi, has_hi, ncx, tw, c, cinv, lane, warp,
@@ -1041,6 +1028,9 @@ __global__ void __launch_bounds__(kFastThreads, 3) k_fast_bits(Batch b)
                 __syncthreads();
             }
             const int n_work = listed ? s_nlist[pass] : items;
+            uint32_t eps_mask[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) eps_mask[i] = 0u - (((uint32_t)eps >> i) & 1u);
             for (int base = warp * 32; base < n_work; base += kFastThreads) {
                 const int w = base + lane;
                 uint32_t bits = 0;
@@ -1051,12 +1041,14 @@ __global__ void __launch_bounds__(kFastThreads, 3) k_fast_bits(Batch b)
                     py = r0 + rr;
                     px0 = 32 * m;
                     uint32_t valid = border_bits(px0, plo, phi);
-                    const uint8_t *strow = has_hi + div_small(py, cinv) * ncx;
-                    if (pass == 1 && valid)  // only cells without a corner (and not skipped)
-                        valid &= cell_bits(strow, px0, tw, c, cinv, [](uint8_t st) { return st == 0; });
-                    else if (some_skipped && valid)  // not in a skipped cell
-                        valid &= cell_bits(strow, px0, tw, c, cinv, [](uint8_t st) { return st != 2; });
-                    if (valid) bits = bs_corners(planes, ru, py, m, sb, eps) & valid;
+                    if (listed && valid) {
+                        const uint8_t *strow = has_hi + div_small(py, cinv) * ncx;
+                        if (pass == 1)  // only cells without a corner (and not skipped)
+                            valid &= cell_bits(strow, px0, tw, c, cinv, [](uint8_t st) { return st == 0; });
+                        else            // not in a skipped cell
+                            valid &= cell_bits(strow, px0, tw, c, cinv, [](uint8_t st) { return st != 2; });
+                    }
+                    if (valid) bits = bs_corners(planes, ru, py, m, sb, eps_mask) & valid;
                 }
                 // the warp's corners in order, scored through windows of kBitsWin entries
                 const int nb = __popc(bits);
@@ -1067,36 +1059,25 @@ __global__ void __launch_bounds__(kFastThreads, 3) k_fast_bits(Batch b)
                     if (lane >= o) incl += y;
                 }
                 const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-                if (pass == 0 && bits) {
-                    // mark the open cells that got a corner, each counted once
-                    const int crow = div_small(py, cinv) * ncx;
-                    const int ca = div_small(px0 + __ffs(bits) - 1, cinv), cz = div_small(px0 + 31 - __clz(bits), cinv);
-                    for (int cx = ca; cx <= cz; ++cx) {
-                        const int a = max(cx * c - px0, 0), z = min((cx + 1) * c - px0, 32);
-                        const uint32_t span = (z >= 32 ? 0xFFFFFFFFu : ((1u << z) - 1u)) & (0xFFFFFFFFu << a);
-                        const int cell = crow + cx;
-                        if ((bits & span) && has_hi[cell] == 0) {
-                            const uint32_t sh = 8u * (uint32_t)(cell & 3);
-                            const uint32_t old = atomicOr(reinterpret_cast<uint32_t *>(has_hi) + (cell >> 2), 1u << sh);
-                            if (((old >> sh) & 0xFFu) == 0u) atomicAdd(&C[3], 1);
-                        }
-                    }
-                }
                 const int ebase = (py << 7) | px0;  // entry of pixel px0 + j: ebase + j
                 for (int w0 = 0; w0 < total; w0 += kBitsWin) {
+                    // this lane's corners from the highest (the order does not matter)
                     uint32_t bb = bits;
-                    for (int id = incl - nb; bb && id < w0 + kBitsWin; ++id) {
-                        const int j = __ffs(bb) - 1;
-                        bb &= bb - 1;
-                        if (id >= w0) wbuf[id - w0] = (uint16_t)(ebase + j);
+                    if (total <= kBitsWin) {
+                        for (uint16_t *to = wbuf + (incl - nb); bb; ++to) {
+                            const int j = 31 - __clz(bb);
+                            bb ^= 1u << j;
+                            *to = (uint16_t)(ebase + j);
+                        }
+                    } else {
+                        for (int id = incl - nb; bb && id < w0 + kBitsWin; ++id) {
+                            const int j = 31 - __clz(bb);
+                            bb ^= 1u << j;
+                            if (id >= w0) wbuf[id - w0] = (uint16_t)(ebase + j);
+                        }
                     }
                     __syncwarp();
                     const int n = min(total - w0, kBitsWin);
-                    int lbase = 0;
-                    if (k > 1) {
-                        if (lane == 0) lbase = atomicAdd(&C[0], n);
-                        lbase = __shfl_sync(0xFFFFFFFFu, lbase, 0);
-                    }
                     for (int i = lane; i < n; i += 32) {
                         const int e = wbuf[i];
                         const int cy_ = e >> 7, cx_ = e & 127;
@@ -1106,53 +1087,58 @@ __global__ void __launch_bounds__(kFastThreads, 3) k_fast_bits(Batch b)
                         const int ccy = div_small(cy_, cinv), ccx = div_small(cx_, cinv);
                         const uint32_t inidx = (uint32_t)((cy_ - ccy * c) * c + (cx_ - ccx * c));
                         const uint32_t key = ((uint32_t)r << 16) | (0xFFFFu - inidx);
-                        if (k == 1) atomicMax(&sel[ccy * ncx + ccx], key);
-                        else { clist[lbase + i] = (uint16_t)e; ckey[lbase + i] = key; }
+                        if (kTop1) {
+                            atomicMax(&sel[ccy * ncx + ccx], key);
+                        } else {
+                            // the cell's k largest keys in falling order: each
+                            // entry keeps the larger and passes the smaller on
+                            // (a key below the last entry, which only grows,
+                            // cannot be among them)
+                            uint32_t *const top = sel + (ccy * ncx + ccx) * k;
+                            if (key > *reinterpret_cast<volatile uint32_t *>(top + k - 1)) {
+                                uint32_t v = key;
+                                for (int j = 0; j < k && v; ++j) v = min(v, atomicMax(top + j, v));
+                            }
+                        }
                     }
                     __syncwarp();
                 }
             }
-            __syncthreads();  // selections, marks and counts of this pass complete
+            __syncthreads();  // the selections of this pass are complete
         }
         }
-        if (k > 1) {
-            const uint32_t cinv = (uint32_t)R.cinv;
-            const int ncx = R.ncx, nc = C[0];
-            for (int j = 0; j < k; ++j) {
-                for (int i = threadIdx.x; i < nc; i += kFastThreads) {
-                    const int e = clist[i];
-                    const int cell = div_small(e >> 7, cinv) * ncx + div_small(e & 127, cinv);
-                    const uint32_t key = ckey[i];
-                    if (j == 0 || key < sel[cell * k + j - 1]) atomicMax(&sel[cell * k + j], key);
-                }
-                __syncthreads();
+        if (s_abort) {  // thread 0 could not start the next tile
+            if (threadIdx.x == 0) {
+                const int sn = s3 == 2 ? 0 : s3 + 1;
+                wait_tile(&bars[2 + sn], (s_rph >> sn) & 1u);  // the record copy that did not complete
             }
+            return;
         }
 
         // slots and the s0 score map (as in k_fast_cull), projections from
         // the staged ranges
         const int c = R.c, ncx = R.ncx, cells = ncx * R.ncy;
         for (int e = threadIdx.x; e < cells * k; e += kFastThreads) {
-            const int cell = e / k, j = e - cell * k;
-            const int lcy = cell / ncx;
+            const int cell = kTop1 ? e : e / k, j = e - cell * k;
+            const int lcy = div_recip(cell, R.ncx_div);
             const int gcx = R.ccx0 + cell - lcy * ncx, gcy = R.ccy0 + lcy;
             const uint32_t key = sel[e];
             b.slots[R.slot_base + (gcy * R.cells_x + gcx) * k + j] = key;
             if (key) {
-                const int inidx = 0xFFFF - (int)(key & 0xFFFFu);
-                const int x = gcx * c + inidx % c, y = gcy * c + inidx / c;
+                const int inidx = 0xFFFF - (int)(key & 0xFFFFu), row = div_recip(inidx, R.cdiv);
+                const int x = gcx * c + inidx - row * c, y = gcy * c + row;
                 if (x >= R.W || y >= R.H) { atomicOr(b.err, kErrDecode); continue; }
                 const int X = prj[R.prj_off_x + x - R.x0], Y = prj[kPrjBytes / 2 + R.prj_off_y + y - R.y0];
                 atomicAdd(R.map + (size_t)Y * R.W0 + X, (1u << 16) + (key >> 16));
             }
         }
-        __syncthreads();  // every reader of this box, its projections, the planes and this set is done
+        if (!more) break;
     }
 }
 
 int fast_smem_bytes(int max_box, int max_px, int max_cells, int k, int max_planes)
 {
-    return max_planes > 0 ? bits_layout(max_box, max_px, max_cells, k, max_planes).total
+    return max_planes > 0 ? bits_layout(max_box, max_cells, k, max_planes).total
                           : fast_layout(max_box, max_px, max_cells, k).total;
 }
 

@@ -25,7 +25,7 @@ namespace jslam {
 __device__ __forceinline__ uint32_t slot_pos(const SegRec &R, uint32_t key, int i, int k)
 {
     const uint32_t inidx = 0xFFFFu - (key & 0xFFFFu);
-    const uint32_t row = R.cdiv ? __umulhi(inidx, R.cdiv) : inidx;  // inidx / c (cdiv = ceil(2^32 / c), 0 for c = 1)
+    const uint32_t row = R.cdiv ? __umulhi(inidx, R.cdiv) : inidx;  // inidx / c
     const uint32_t x = (uint32_t)(k == 1 ? i : i / k) * (uint32_t)R.c + (inidx - row * (uint32_t)R.c);
     return x | (((uint32_t)R.y0 + row) << 13) | ((uint32_t)R.level << 26);
 }

@@ -337,6 +337,7 @@ __device__ __forceinline__ void pyramid_strip(const Batch &b, const LevelDesc &L
 __global__ void __launch_bounds__(32, kPyrWarpsPerSm) k_pyramid(Batch b)
 {
     __shared__ PyrShared S;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *b.tile_next = 0u;  // for the detection launch that follows
     const int tile = __ldg(b.pyr_order + (b.pyr_pass < 0 ? 0 : b.pyr_pass_first[b.pyr_pass]) + blockIdx.x);
     const int li = __ldg(b.pyr_tile_level + tile);
     const LevelDesc &L = b.levels[li];
