@@ -193,7 +193,7 @@ struct jslam_ctx {
     // constant tables
     GrowBuf consts;  // pattern | cos | sin | corner table
     int8_t *d_pattern = nullptr;
-    uint32_t *d_pattern_off = nullptr;
+    uint32_t *d_pattern_off = nullptr, *d_disk_mask = nullptr;
     double *d_cos = nullptr, *d_sin = nullptr;
     float *d_cosf = nullptr, *d_sinf = nullptr;
     uint32_t *d_lut = nullptr;
@@ -591,6 +591,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     const size_t o_trec = reserve(sizeof(TileRec) * (n_fast_tiles + 1));
     const size_t o_lstart = reserve(sizeof(int32_t) * (kMaxLevels + 1) * n_img);
     const size_t o_tmaps = reserve(sizeof(CUtensorMap) * (size_t)n_levels);
+    const size_t o_omaps = reserve(2 * sizeof(CUtensorMap) * (size_t)n_levels);
     const size_t o_tables = reserve(table_bytes + 256);
     if ((e = ctx->plan.ensure(off, false, nullptr)) != cudaSuccess) return fail(ctx, e);
 
@@ -728,6 +729,20 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                         L.tmap = reinterpret_cast<const CUtensorMap *>(dplan + o_tmaps) + li;
                     }
                 }
+                // keypoint boxes of the raw and the blurred level
+                for (int q = 0; q < 2; ++q) {
+                    CUtensorMap map;
+                    const cuuint64_t dims[2] = { (cuuint64_t)L.W, (cuuint64_t)L.H };
+                    const cuuint64_t strides[1] = { (cuuint64_t)L.pitch };
+                    const cuuint32_t box[2] = { (cuuint32_t)kOrbBoxW, (cuuint32_t)(q ? kOrbBlurH : kOrbRawH) };
+                    const cuuint32_t estr[2] = { 1, 1 };
+                    if (!encode || encode(&map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, q ? L.blur : L.raw_w, dims, strides, box,
+                                          estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                          CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                        return fail(ctx, cudaErrorNotSupported);
+                    std::memcpy(host.data() + o_omaps + sizeof(CUtensorMap) * (2 * li + q), &map, sizeof(CUtensorMap));
+                }
                 L.slot_base = slot;
                 L.seg_base = seg;
                 for (int r = 0; r < L.cells_y; ++r) {
@@ -856,6 +871,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     Batch &b = ctx->batch;
     b.images = reinterpret_cast<const ImageDesc *>(dplan + o_images);
     b.levels = reinterpret_cast<const LevelDesc *>(dplan + o_levels);
+    b.orb_maps = reinterpret_cast<const CUtensorMap *>(dplan + o_omaps);
     b.pairs = reinterpret_cast<const PairDesc *>(dplan + o_pairs);
     b.pyr_tile_base = reinterpret_cast<const int32_t *>(dplan + o_pyr);
     b.pyr_tile_level = reinterpret_cast<const int32_t *>(dplan + o_ptl);
@@ -890,6 +906,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     for (int i = 0; i < n_img; ++i) b.max_slots = std::max(b.max_slots, images[i].slot_count);
     b.pattern = ctx->d_pattern;
     b.pattern_off = ctx->d_pattern_off;
+    b.disk_mask = ctx->d_disk_mask;
     b.bin_cos = ctx->d_cos;
     b.bin_sin = ctx->d_sin;
     b.bin_cosf = ctx->d_cosf;
@@ -1037,6 +1054,7 @@ jslam_status jslam_create(jslam_ctx **out, const jslam_config *cfg)
     }
     if (e == cudaSuccess) e = configure_kernels();
     if (e == cudaSuccess) e = configure_skipnet();
+    if (e == cudaSuccess) e = configure_orb();
     int32_t w[7];
     blur_weights(w);
     if (e == cudaSuccess) e = set_blur_weights(w);
@@ -1044,7 +1062,8 @@ jslam_status jslam_create(jslam_ctx **out, const jslam_config *cfg)
     const size_t lut_off = pat_bytes + 2 * kBins * sizeof(double);
     const size_t f_off = lut_off + kLutWords * sizeof(uint32_t);
     const size_t po_off = f_off + 2 * kBins * sizeof(float);
-    const size_t const_bytes = po_off + (size_t)kBins * kPairs * sizeof(uint32_t);
+    const size_t dm_off = po_off + (size_t)kBins * kPairs * sizeof(uint32_t);
+    const size_t const_bytes = dm_off + (size_t)4 * kDiskRows * 32 * sizeof(uint32_t);
     if (e == cudaSuccess) e = ctx->consts.ensure(const_bytes + 512, false, nullptr);
     if (e == cudaSuccess) {
         std::vector<char> h(const_bytes, 0);
@@ -1058,10 +1077,25 @@ jslam_status jslam_create(jslam_ctx **out, const jslam_config *cfg)
         const int8_t *pt = reinterpret_cast<const int8_t *>(h.data());
         uint32_t *po = reinterpret_cast<uint32_t *>(h.data() + po_off);
         for (int i = 0; i < kBins * kPairs; ++i) {
-            const int op = pt[4 * i + 1] * kPatPitch + pt[4 * i + 0];
-            const int oq = pt[4 * i + 3] * kPatPitch + pt[4 * i + 2];
-            po[i] = (uint32_t)(uint16_t)(int16_t)op | ((uint32_t)(uint16_t)(int16_t)oq << 16);
+            const int op = (pt[4 * i + 1] + kPatR) * kPatPitch + pt[4 * i + 0] + kPatR;
+            const int oq = (pt[4 * i + 3] + kPatR) * kPatPitch + pt[4 * i + 2] + kPatR;
+            po[i] = (uint32_t)op | ((uint32_t)oq << 16);
         }
+        // moment disk: lane l < 27 of a warp has word column l % 9 and rows
+        // l / 9, l / 9 + 3, ... of the 31; the word's first byte lies 15 + a
+        // columns left of the keypoint plus 4 per word column (alignment a)
+        uint32_t *dm = reinterpret_cast<uint32_t *>(h.data() + dm_off);
+        for (int a = 0; a < 4; ++a)
+            for (int r = 0; r < kDiskRows; ++r)
+                for (int l = 0; l < 27; ++l) {
+                    const int dy = l / 9 + 3 * r - kDiskR;
+                    uint32_t m = 0;
+                    for (int q = 0; q < 4; ++q) {
+                        const int dx = 4 * (l % 9) - kDiskR - a + q;
+                        if (dx * dx + dy * dy <= kDiskR * kDiskR) m |= 0xFFu << (8 * q);
+                    }
+                    dm[(a * kDiskRows + r) * 32 + l] = m;
+                }
         e = cudaMemcpy(ctx->consts.ptr, h.data(), h.size(), cudaMemcpyHostToDevice);
         ctx->d_pattern = ctx->consts.as<int8_t>();
         ctx->d_cos = ctx->consts.as<double>(pat_bytes);
@@ -1070,6 +1104,7 @@ jslam_status jslam_create(jslam_ctx **out, const jslam_config *cfg)
         ctx->d_cosf = ctx->consts.as<float>(f_off);
         ctx->d_sinf = ctx->d_cosf + kBins;
         ctx->d_pattern_off = ctx->consts.as<uint32_t>(po_off);
+        ctx->d_disk_mask = ctx->consts.as<uint32_t>(dm_off);
     }
     if (e == cudaSuccess) e = ctx->counts.ensure(sizeof(int32_t) * (2 * (size_t)c.max_pairs + 8), true, nullptr);
     if (e == cudaSuccess) {

@@ -22,7 +22,9 @@ constexpr int kBins = 30;        // orientation sectors of 12 degrees
 constexpr int kPairs = 256;      // BRIEF point pairs
 constexpr int kDiskR = 15;       // intensity-centroid disk radius
 constexpr int kPatR = 13;        // rotated BRIEF offsets lie in [-13, 13]
-constexpr int kPatPitch = 32;    // row pitch of the staged 27 x 27 BRIEF patch (8 aligned words)
+constexpr int kDiskRows = 11;    // disk rows of a lane: every third of the 31 (and past the last)
+constexpr int kOrbBoxW = 48, kOrbRawH = 31, kOrbBlurH = 27;  // a keypoint's boxes of the raw and the blurred level
+constexpr int kPatPitch = kOrbBoxW;  // row pitch of the staged 27 x 27 BRIEF patch
 constexpr int kMaxSegment = 4096;  // candidate slots per (level, cell row)
 constexpr int kMaxImages = 256;    // images per batch (two per stereo pair)
 
@@ -198,6 +200,7 @@ constexpr int kSlotEmpty = -2, kSlotSuppressed = -1;
 struct Batch {
     const ImageDesc *images;
     const LevelDesc *levels;
+    const CUtensorMap *orb_maps;    // per level: keypoint boxes of the raw and of the blurred level
     const PairDesc *pairs;
     const int32_t *pyr_tile_base;   // n_levels + 1
     const int32_t *pyr_tile_level;  // level index of each pyramid strip
@@ -227,7 +230,8 @@ struct Batch {
     int32_t max_slots;              // most candidate slots of an image
     int32_t n_sm;                   // streaming multiprocessors of the device
     const int8_t *pattern;          // kBins x kPairs x 4
-    const uint32_t *pattern_off;    // kBins x kPairs: int16 patch offsets of p | of q << 16 (pitch kPatPitch)
+    const uint32_t *pattern_off;    // kBins x kPairs: patch offsets of p | of q << 16 (pitch kPatPitch, from the corner)
+    const uint32_t *disk_mask;      // 4 alignments x kDiskRows x 32 lanes: bytes of a word inside the moment disk
     const double *bin_cos, *bin_sin;
     const float *bin_cosf, *bin_sinf;  // the same tables rounded to float (fast sector test)
     uint32_t *err;
@@ -268,6 +272,7 @@ cudaError_t launch_skipnet(const Batch &b, const SkipModelDev &m, float thresh, 
 cudaError_t set_blur_weights(const int32_t w[7]);
 cudaError_t configure_kernels();
 cudaError_t configure_skipnet();
+cudaError_t configure_orb();
 int skipnet_smem_bytes();
 
 }  // namespace jslam

@@ -2,181 +2,258 @@
 // streamlined multiscale detection and extraction; middle-end stereo
 // matching by descriptor-distance minimisation).
 //
-// k_orient_desc  one warp per keypoint of any image and level.  The lanes
-//                read the radius-15 disk of the raw level as aligned words
-//                (9 per row) and accumulate the intensity moments m10, m01
-//                with byte dot products over the bytes inside the disk; they
-//                stage the 27 x 27 blurred patch the BRIEF pattern reaches in
-//                shared memory the same way (8 words per row); lanes 0..29 each test
-//                one sector boundary (float with an error margin, IEEE double
-//                with explicit rounding inside it, so the sector equals the
-//                one the host-side definition gives); the 256 BRIEF
+// k_orient_desc  one warp per keypoint (and turn) of any image and level.  The
+//                tensor unit brings the keypoint's box of the raw level (the
+//                radius-15 disk) and of the blurred one (the 27 x 27 patch the
+//                BRIEF pattern reaches) to shared memory, those of the next
+//                keypoint while this one is computed.  The lanes read the disk
+//                as words and accumulate the intensity moments m10, m01 with
+//                byte dot products over the bytes inside the disk; lanes 0..29
+//                each test one sector boundary (float with an error margin,
+//                IEEE double with explicit rounding inside it, so the sector
+//                equals the one the host-side definition gives); the 256 BRIEF
 //                comparisons read the patch 32 at a time and are packed into
 //                words by a ballot.
-// k_match        one warp per left keypoint: for each right level within one
+// k_match        half a warp per left keypoint: for each right level within one
 //                of the keypoint's level, takes the s0 row band of the
 //                canonical (level, y, x) list (Y is non-decreasing in y) from
 //                the row index (two independent loads per level), scans the
 //                band with the lanes, and keeps the smallest (Hamming
-//                distance, disparity, index) by a warp min-reduction.
+//                distance, disparity, index) by a min-reduction.
+#include <algorithm>
+
+#include <cuda.h>
+
 #include "jslam_internal.h"
 
 namespace jslam {
 
-constexpr int kPatW = 2 * kPatR + 1;      // 27
 constexpr int kDiskWords = 9;             // aligned words covering the 31 disk columns of a row
-// largest |dx| with dx^2 + dy^2 <= kDiskR^2, by |dy|
-__constant__ int8_t c_disk_umax[kDiskR + 1] = { 15, 14, 14, 14, 14, 14, 13, 13, 12, 12, 11, 10, 9, 7, 5, 0 };
+constexpr int kOrbWarps = 4;              // warps per CTA
+constexpr int kOrbMaxTurns = 32;          // keypoints a warp takes, at most (a lane keeps each one's moments)
+static_assert(kDiskRows * 3 > 2 * kDiskR + 1 && 3 * kDiskWords <= 32, "a lane's rows cover the disk");
+constexpr int kOrbRaw = (kOrbBoxW * kOrbRawH + 127) / 128 * 128, kOrbBlur = (kOrbBoxW * kOrbBlurH + 127) / 128 * 128;
 
-__global__ void __launch_bounds__(256) k_orient_desc(Batch b)
+// A keypoint's boxes: rows of 48 bytes from the 16-byte boundary at or before
+// the disk's (the patch's) first column.
+struct __align__(128) OrbBuf {
+    uint8_t raw[kOrbRaw];
+    uint8_t blur[kOrbBlur];
+};
+constexpr int kOrbSmem = 2 * kOrbWarps * (int)sizeof(OrbBuf);  // two boxes a warp
+
+__device__ __forceinline__ uint32_t orb_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Wait for the mbarrier phase `parity`, giving up after about a second.
+__device__ __forceinline__ bool orb_wait(uint32_t bar, uint32_t parity)
 {
-    __shared__ __align__(16) uint8_t s_patch[8][kPatW * kPatPitch];
-    const int img = blockIdx.y;
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-    const ImageDesc &I = b.images[img];
-    if (i >= *I.count) return;
+    const long long start = clock64();
+    for (;;) {
+        uint32_t done;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        if (done) return true;
+        if (clock64() - start > (1ll << 31)) return false;
+    }
+}
+
+// One box of a keypoint by TMA; x is a multiple of 16 and the box starts
+// inside the level (it may end past its right edge: those bytes are zero and
+// unused).
+__device__ __forceinline__ void orb_box(const CUtensorMap *map, const uint8_t *to, int x, int y, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(orb_smem(to)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+
+// What bounds it: shared-memory and load latency (the dependent chain box ->
+// moments -> sector -> pattern -> patch, 32 warps an SM).  Reading disk and
+// patch with plain loads touches a line per row, 75 of the 170 load
+// wavefronts a keypoint took, and those bounded it: 400 000 keypoints 0.260 ms
+// with one warp each and 563 instructions a keypoint; 0.205 ms now, with 328.
+// A warp takes keypoints i, i + stride, ... of its image.
+__global__ void __launch_bounds__(32 * kOrbWarps) k_orient_desc(Batch b)
+{
+    extern __shared__ __align__(128) uint8_t orb_mem[];
+    __shared__ __align__(8) uint64_t s_bar[kOrbWarps][2];
+    const ImageDesc &I = b.images[blockIdx.y];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int count = *I.count, stride = gridDim.x * kOrbWarps;
+    const int first = blockIdx.x * kOrbWarps + warp;
+    if (first >= count) return;
     const KpOut &o = I.out;
-    const int lvl = o.level[i], x = o.x[i], y = o.y[i];
-    const LevelDesc &L = b.levels[I.level_base + lvl];
-    const uint8_t *raw = L.raw;
-    const int pitch = L.pitch;
-    const int bpitch = L.blur_pitch;
-    uint8_t *patch = s_patch[threadIdx.x >> 5];
+    const CUtensorMap *const maps = b.orb_maps + 2 * I.level_base;
+    OrbBuf *const buf = reinterpret_cast<OrbBuf *>(orb_mem) + 2 * warp;
+    const uint32_t bar = orb_smem(s_bar[warp]);
+    if (lane < 2) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8 * lane) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    __syncwarp();
+    const uint16_t *const xs = o.x, *const ys = o.y;
+    const uint8_t *const lv = o.level;
+    // the boxes of the keypoint at (x, y) into buffer k.  The keypoint is at
+    // least `border` (>= 16) from every edge, so the 31 x 31 square of the
+    // moment disk and the 27 x 27 patch are inside the level.
+    const auto issue = [&](int x, int y, int level, int k) {
+        if (lane == 0) {
+            const CUtensorMap *map = maps + 2 * level;
+            const uint32_t bk = bar + 8 * k;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bk),
+                         "r"((uint32_t)(kOrbBoxW * (kOrbRawH + kOrbBlurH))) : "memory");
+            orb_box(map, buf[k].raw, (x - kDiskR) & ~15, y - kDiskR, bk);
+            orb_box(map + 1, buf[k].blur, (x - kPatR) & ~15, y - kPatR, bk);
+        }
+    };
+    int x = xs[first], y = ys[first], level = lv[first];
+    issue(x, y, level, 0);
+    int nx = 0, ny = 0, nlev = 0;
+    if (first + stride < count) { nx = xs[first + stride]; ny = ys[first + stride]; nlev = lv[first + stride]; }
+    uint32_t *const desc = o.desc;
+    // lane < 27 of the disk: word column w, rows r0, r0 + 3, ...
+    const int w = lane % kDiskWords, r0 = lane / kDiskWords;
+    const float cosf_l = lane < kBins ? __ldg(b.bin_cosf + lane) : 0.0f;
+    const float sinf_l = lane < kBins ? __ldg(b.bin_sinf + lane) : 0.0f;
+    int my10 = 0, my01 = 0;  // the moments of the keypoint of turn `lane`
 
-    // The keypoint is at least `border` (>= 16) from every edge, so the
-    // 31 x 31 square of the moment disk and the 27 x 27 patch of the BRIEF
-    // pattern are inside the level.  Both are read as aligned 32-bit words
-    // (rows start on 128-byte boundaries; a row's last word may reach 3
-    // bytes past the level's width, into the pitch or the buffer's slack),
-    // every load independent of the others.
-    // Patch: 27 rows x 8 words from word column (x - 13) / 4 of the blurred
-    // level, staged with a pitch of 32 bytes.
-    const int pw0 = (x - kPatR) >> 2;
-    {
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(L.blur + (size_t)(y - kPatR) * bpitch) + pw0;
-        uint32_t *dst = reinterpret_cast<uint32_t *>(patch);
+    int turn = 0;
+    for (int i = first; i < count; i += stride, ++turn) {
+        const int k2 = turn & 1;
+        if (i + stride < count) issue(nx, ny, nlev, k2 ^ 1);
+        int n2x = 0, n2y = 0, n2l = 0;
+        if (i + 2 * stride < count) { n2x = xs[i + 2 * stride]; n2y = ys[i + 2 * stride]; n2l = lv[i + 2 * stride]; }
+        // Disk moments: 31 rows x 9 words from the word that holds column x -
+        // 15; a lane has one word column and every third row.  Per word the
+        // bytes inside the disk are kept (a table's masks, by the alignment)
+        // and two byte dot products add to the sum S of the pixels and to that
+        // of (dx + 18) I; U sums S after every row, so that the sum of k I_k is
+        // 11 S - U for the lane's row number k, row dy = r0 + 3 k - 15.
+        const int al = (x - kDiskR) & 3;
+        uint32_t mask[kDiskRows];
 #pragma unroll
-        for (int k = 0; k < (kPatW * 8 + 31) / 32; ++k) {
-            const int it = k * 32 + lane;
-            if (it < kPatW * 8) {
-                const int r = it >> 3, w = it & 7;
-                dst[it] = __ldg(src + (size_t)r * (bpitch >> 2) + w);
+        for (int k = 0; k < kDiskRows; ++k) mask[k] = __ldg(b.disk_mask + (al * kDiskRows + k) * 32 + lane);
+        if (!orb_wait(bar + 8 * k2, (turn >> 1) & 1)) {
+            // flag it, and wait once more, with the same limit, for the copies
+            // in flight, so that none lands in the memory of a CTA that ended
+            if (lane == 0) atomicOr(b.err, kErrTimeout);
+            orb_wait(bar + 8 * k2, (turn >> 1) & 1);
+            if (i + stride < count) orb_wait(bar + 8 * (k2 ^ 1), ((turn + 1) >> 1) & 1);
+            return;
+        }
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(buf[k2].raw) + r0 * (kOrbBoxW / 4) +
+                              (((x - kDiskR) & 15) >> 2) + w;
+        const uint32_t wdx = (uint32_t)(4 * w + 3 - al) * 0x01010101u + 0x03020100u;  // dx + 18 of the word's bytes
+        uint32_t Sm = 0, U = 0, Sw = 0;
+#pragma unroll
+        for (int k = 0; k < kDiskRows; ++k) {
+            const uint32_t v = src[k * 3 * (kOrbBoxW / 4)] & mask[k];
+            Sm = __dp4a(v, 0x01010101u, Sm);
+            Sw = __dp4a(v, wdx, Sw);
+            U += Sm;
+        }
+        const int m10 = __reduce_add_sync(0xFFFFFFFFu, (int)Sw - 18 * (int)Sm);
+        const int m01 = __reduce_add_sync(0xFFFFFFFFu, (r0 - kDiskR + 3 * kDiskRows) * (int)Sm - 3 * (int)U);
+
+        // Sector b is the one whose lower boundary has the moment vector on its
+        // left (m01 cos - m10 sin >= 0 in IEEE double) and whose upper boundary
+        // does not.  The test runs in float first: |m| < 2^24 is exact, and the
+        // float result is within (|m01| + |m10|) 2^-22 of the exact value with
+        // the double table entries, so outside 2^-20 times that its sign is the
+        // double test's; lanes inside the margin (rare) take the double test.
+        bool left_of = false;
+        if (lane < kBins) {
+            const float fa = (float)m01, fb = (float)m10;
+            const float t = __fsub_rn(__fmul_rn(fa, cosf_l), __fmul_rn(fb, sinf_l));
+            const float margin = (fabsf(fa) + fabsf(fb)) * 0x1p-20f;
+            if (fabsf(t) > margin) {
+                left_of = t > 0.0f;
+            } else {
+                const double t1 = __dmul_rn((double)m01, b.bin_cos[lane]);
+                const double t2 = __dmul_rn((double)m10, b.bin_sin[lane]);
+                left_of = __dsub_rn(t1, t2) >= 0.0;
             }
         }
-    }
-    // Disk moments: 31 rows x 9 words from word column (x - 15) / 4 of the
-    // raw level.  Lane l < 27 keeps word column l mod 9 and takes rows
-    // l / 9, l / 9 + 3, ...; per word, the bytes inside the disk
-    // (|dx| <= umax(|dy|)) are kept and two byte dot products give the row
-    // sum and the sum of (dx + 18) I (weights 3..36, unsigned, fixed per
-    // lane); m10 = that - 18 sum I.
-    int m10 = 0, m01 = 0;
-    if (lane < 3 * kDiskWords) {
-        const int dw0 = (x - kDiskR) >> 2;
-        const int w = lane % kDiskWords, r0 = lane / kDiskWords;
-        const int cx0 = 4 * (dw0 + w) - x;  // dx of the word's byte 0
-        const uint32_t wdx = (uint32_t)(cx0 + 18) * 0x01010101u + 0x03020100u;
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(raw + (size_t)(y - kDiskR + r0) * pitch) + dw0 + w;
-        const size_t step = (size_t)3 * (pitch >> 2);
-        int s = 0, sw = 0;
-#pragma unroll
-        for (int k = 0; k < (2 * kDiskR + 1 + 2) / 3; ++k) {
-            const int r = r0 + 3 * k;
-            if (r <= 2 * kDiskR) {
-                const uint32_t v = __ldg(src + k * step);
-                const int dy = r - kDiskR;
-                const int um = c_disk_umax[abs(dy)];
-                const int lo = max(-um - cx0, 0), hi = min(um - cx0, 3);
-                const uint32_t mask = hi < lo ? 0u : (0xFFFFFFFFu >> (24 - 8 * (hi - lo))) << (8 * lo);
-                const uint32_t vm = v & mask;
-                const int rs = (int)__dp4a(vm, 0x01010101u, 0u);
-                s += rs;
-                m01 += dy * rs;
-                sw += (int)__dp4a(vm, wdx, 0u);
-            }
-        }
-        m10 = sw - 18 * s;
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        m10 += __shfl_xor_sync(0xFFFFFFFFu, m10, off);
-        m01 += __shfl_xor_sync(0xFFFFFFFFu, m01, off);
-    }
+        const uint32_t Lt = __ballot_sync(0xFFFFFFFFu, left_of) & ((1u << kBins) - 1u);
+        const uint32_t next = (Lt >> 1) | ((Lt & 1u) << (kBins - 1));
+        const uint32_t T = Lt & ~next & ((1u << kBins) - 1u);
+        const bool zero = (m10 == 0 && m01 == 0);
+        const int bin = (zero || T == 0) ? 0 : __ffs(T) - 1;
 
-    // Sector b is the one whose lower boundary has the moment vector on its
-    // left (m01 cos - m10 sin >= 0 in IEEE double) and whose upper boundary
-    // does not.  The test runs in float first: |m| < 2^24 is exact, and the
-    // float result is within (|m01| + |m10|) 2^-22 of the exact value with
-    // the double table entries, so outside 2^-20 times that its sign is the
-    // double test's; lanes inside the margin (rare) take the double test.
-    bool left_of = false;
-    if (lane < kBins) {
-        const float fa = (float)m01, fb = (float)m10;
-        const float t = __fsub_rn(__fmul_rn(fa, __ldg(b.bin_cosf + lane)), __fmul_rn(fb, __ldg(b.bin_sinf + lane)));
-        const float margin = (fabsf(fa) + fabsf(fb)) * 0x1p-20f;
-        if (fabsf(t) > margin) {
-            left_of = t > 0.0f;
-        } else {
-            const double t1 = __dmul_rn((double)m01, b.bin_cos[lane]);
-            const double t2 = __dmul_rn((double)m10, b.bin_sin[lane]);
-            left_of = __dsub_rn(t1, t2) >= 0.0;
-        }
-    }
-    const uint32_t S = __ballot_sync(0xFFFFFFFFu, left_of) & ((1u << kBins) - 1u);
-    const uint32_t next = (S >> 1) | ((S & 1u) << (kBins - 1));
-    const uint32_t T = S & ~next & ((1u << kBins) - 1u);
-    const bool zero = (m10 == 0 && m01 == 0);
-    const int bin = (zero || T == 0) ? 0 : __ffs(T) - 1;
-
-    __syncwarp();  // the patch is complete
-    const uint32_t *pat = b.pattern_off + (size_t)bin * kPairs;
-    const uint8_t *centre = patch + kPatR * kPatPitch + (x - kPatR - 4 * pw0) + kPatR;
-    uint32_t myword = 0;
+        // shared addresses of p (low half) and q of a pair: offsets from the
+        // patch's corner, and its place
+        const uint32_t *pat = b.pattern_off + (size_t)bin * kPairs + lane;
+        const uint32_t at = (orb_smem(buf[k2].blur) + (uint32_t)((x - kPatR) & 15)) * 0x00010001u;
+        uint32_t myword = 0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) {
-        const uint32_t o = __ldg(pat + w * 32 + lane);  // offsets of p and q in the staged patch
-        const int a = centre[(int16_t)(o & 0xFFFFu)];
-        const int c = centre[(int16_t)(o >> 16)];
-        const uint32_t word = __ballot_sync(0xFFFFFFFFu, a < c);
-        if (lane == w) myword = word;
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t pq = __ldg(pat + 32 * k) + at;
+            uint32_t p8, q8;
+            asm volatile("ld.shared.u8 %0, [%1];" : "=r"(p8) : "r"(pq & 0xFFFFu));
+            asm volatile("ld.shared.u8 %0, [%1];" : "=r"(q8) : "r"(pq >> 16));
+            const uint32_t word = __ballot_sync(0xFFFFFFFFu, p8 < q8);
+            if (lane == k) myword = word;
+        }
+        if (lane < 8) desc[(size_t)i * 8 + lane] = myword;
+        if (lane == 0) o.angle_bin[i] = (uint8_t)bin;
+        if (lane == turn) { my10 = m10; my01 = m01; }
+        x = nx; y = ny; level = nlev;
+        nx = n2x; ny = n2y; nlev = n2l;
+        __syncwarp();  // the buffer has been read
     }
-    if (lane < 8) o.desc[(size_t)i * 8 + lane] = myword;
-    if (lane == 0) {
-        o.angle[i] = zero ? 0.0f : atan2f((float)m01, (float)m10);
-        o.angle_bin[i] = (uint8_t)bin;
-    }
+    // the angles of all turns at once
+    if (lane < turn) o.angle[first + lane * stride] = my10 == 0 && my01 == 0 ? 0.0f : atan2f((float)my01, (float)my10);
+}
+
+// Keypoints per warp: as many as leave two rounds of resident warps (32 an
+// SM), so that a warp brings the next boxes while it computes and shares what
+// it does once (its tables, the angles); one in small batches.  1 / 2 / 4 / 8 /
+// 16 (us): 100 pairs of 1241x376 340 / 256 / 217 / 210 / 205, 16 mixed pairs 59
+// / 52 / 47 / 45 / 45, one pair of 1241x376 10 / 12 / 13 / 16 / 24.
+static int orb_turns(const Batch &b)
+{
+    const long long keypoints = (long long)b.max_capacity * b.n_images;
+    return (int)std::min<long long>(std::max<long long>(keypoints / (64 * b.n_sm), 1), 16);
+}
+
+cudaError_t configure_orb()
+{
+    return cudaFuncSetAttribute(k_orient_desc, cudaFuncAttributeMaxDynamicSharedMemorySize, kOrbSmem);
 }
 
 cudaError_t launch_orient_desc(const Batch &b, cudaStream_t stream)
 {
     if (b.n_images == 0 || b.max_capacity == 0) return cudaSuccess;
-    dim3 grid((b.max_capacity + 7) / 8, b.n_images);
-    k_orient_desc<<<grid, 256, 0, stream>>>(b);
+    const int turns = orb_turns(b);
+    static_assert(16 <= kOrbMaxTurns, "a lane keeps each turn's moments");
+    dim3 grid((b.max_capacity + kOrbWarps * turns - 1) / (kOrbWarps * turns), b.n_images);
+    k_orient_desc<<<grid, 32 * kOrbWarps, kOrbSmem, stream>>>(b);
     return cudaGetLastError();
 }
 
-// Eight CTAs per SM (32 registers): the kernel waits on gathers from L2, and
-// the fuller SM hides more of them than the spill of the eight descriptor
-// words costs (0.148 -> 0.123 ms per KITTI-shaped launch).
+// Half a warp per left keypoint: its band holds a few dozen candidates at
+// most, of which a good part lies outside the search range.  What bounds it:
+// the chain of gathers from L2 (keypoint -> row index -> X -> descriptor);
+// eight CTAs an SM hide most of it.  200 000 left keypoints: 0.121 ms with a
+// warp each, 0.072 now (0.078 with six CTAs an SM).
 __global__ void __launch_bounds__(256, 8) k_match(Batch b)
 {
-    const int pair = blockIdx.y;
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-    const PairDesc &P = b.pairs[pair];
+    const PairDesc &P = b.pairs[blockIdx.y];
+    const int l16 = threadIdx.x & 15;
     const ImageDesc &Il = b.images[P.left];
     const ImageDesc &Ir = b.images[P.right];
-    if (i >= *Il.count) return;
+    const int count = *Il.count;
+    int i = blockIdx.x * 16 + (threadIdx.x >> 4);
+    if ((i & ~1) >= count) return;  // whole warps only
+    const bool valid = i < count;
+    i = min(i, count - 1);
     const KpOut &ol = Il.out, &orr = Ir.out;
     const int n = ol.level[i];
     const int X = ol.X[i], Y = ol.Y[i];
     const int band = b.levels[Il.level_base + n].band;
-    uint32_t dl[8];
-#pragma unroll
-    for (int w = 0; w < 8; ++w) dl[w] = ol.desc[(size_t)i * 8 + w];
+    const uint4 *dp = reinterpret_cast<const uint4 *>(ol.desc + (size_t)i * 8);
+    const uint4 l0 = dp[0], l1 = dp[1];
 
-    unsigned long long best = ~0ull;
     const int m_lo = max(0, n - 1), m_hi = min(Ir.levels - 1, n + 1);
     // the band [Y - band, Y + band] of each level: lower bounds of Y - band
     // and Y + band + 1 from the row index (rows clamped to [0, H0]; a level
@@ -196,39 +273,35 @@ __global__ void __launch_bounds__(256, 8) k_match(Batch b)
     }
     // the three bands as one run of candidates over the lanes (a band of a
     // level outside the frame, or of an empty level, is empty), so a few
-    // dozen candidates take one pass of loads, not one per level
+    // dozen candidates take one or two passes of loads, not one per level
     const int c0 = rz[0] - ra[0], c01 = c0 + (rz[1] - ra[1]), T = c01 + (rz[2] - ra[2]);
-    for (int t = lane; t < T; t += 32) {
+    const uint16_t *const Xr = orr.X;
+    const uint32_t *const descr = orr.desc;
+    // smallest (distance, disparity), then index: a lane's candidates come in
+    // index order
+    uint32_t best = 0xFFFFFFFFu, best_j = 0xFFFFFFFFu;
+    for (int t = l16; t < T; t += 16) {
         const int j = t < c0 ? ra[0] + t : (t < c01 ? ra[1] + (t - c0) : ra[2] + (t - c01));
-        const int disp = X - (int)orr.X[j];
-        if (disp < 0 || disp > b.prm.max_disp) continue;
-        const uint4 *dr = reinterpret_cast<const uint4 *>(orr.desc + (size_t)j * 8);
+        const int disp = X - (int)Xr[j];
+        if ((uint32_t)disp > (uint32_t)b.prm.max_disp) continue;
+        const uint4 *dr = reinterpret_cast<const uint4 *>(descr + (size_t)j * 8);
         const uint4 r0 = dr[0], r1 = dr[1];
-        const int d = __popc(dl[0] ^ r0.x) + __popc(dl[1] ^ r0.y) + __popc(dl[2] ^ r0.z) +
-                      __popc(dl[3] ^ r0.w) + __popc(dl[4] ^ r1.x) + __popc(dl[5] ^ r1.y) +
-                      __popc(dl[6] ^ r1.z) + __popc(dl[7] ^ r1.w);
-        const unsigned long long key = ((unsigned long long)d << 48) |
-                                       ((unsigned long long)disp << 32) | (unsigned)j;
-        best = key < best ? key : best;
+        const uint32_t d = __popc(l0.x ^ r0.x) + __popc(l0.y ^ r0.y) + __popc(l0.z ^ r0.z) + __popc(l0.w ^ r0.w) +
+                           __popc(l1.x ^ r1.x) + __popc(l1.y ^ r1.y) + __popc(l1.z ^ r1.z) + __popc(l1.w ^ r1.w);
+        const uint32_t key = (d << 16) | (uint32_t)disp;
+        if (key < best) { best = key; best_j = (uint32_t)j; }
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xFFFFFFFFu, best, off);
-        best = other < best ? other : best;
+    for (int off = 8; off > 0; off >>= 1) {
+        const uint32_t k2 = __shfl_xor_sync(0xFFFFFFFFu, best, off), j2 = __shfl_xor_sync(0xFFFFFFFFu, best_j, off);
+        if (k2 < best || (k2 == best && j2 < best_j)) { best = k2; best_j = j2; }
     }
-    if (lane == 0) {
-        if (best == ~0ull) {
-            P.match_idx[i] = -1; P.disparity[i] = 0; P.dist[i] = 0xFFFF;
-        } else {
-            const int d = (int)(best >> 48);
-            if (d <= b.prm.max_dist) {
-                P.match_idx[i] = (int)(best & 0xFFFFFFFFu);
-                P.disparity[i] = (int16_t)((best >> 32) & 0xFFFFu);
-                P.dist[i] = (uint16_t)d;
-            } else {
-                P.match_idx[i] = -1; P.disparity[i] = 0; P.dist[i] = (uint16_t)d;
-            }
-        }
+    if (l16 == 0 && valid) {
+        const int d = (int)(best >> 16);  // 0xFFFF: no candidate
+        const bool ok = d <= b.prm.max_dist && best != 0xFFFFFFFFu;
+        P.match_idx[i] = ok ? (int)best_j : -1;
+        P.disparity[i] = ok ? (int16_t)(best & 0xFFFFu) : (int16_t)0;
+        P.dist[i] = (uint16_t)d;
     }
 }
 
@@ -315,7 +388,7 @@ cudaError_t launch_track(const Batch &b, const TrackArgs &a, cudaStream_t stream
 cudaError_t launch_match(const Batch &b, cudaStream_t stream)
 {
     if (b.n_pairs == 0 || b.max_capacity == 0) return cudaSuccess;
-    dim3 grid((b.max_capacity + 7) / 8, b.n_pairs);
+    dim3 grid((b.max_capacity + 15) / 16, b.n_pairs);
     k_match<<<grid, 256, 0, stream>>>(b);
     return cudaGetLastError();
 }
