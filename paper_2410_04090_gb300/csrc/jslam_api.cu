@@ -219,6 +219,7 @@ struct jslam_ctx {
     cudaEvent_t abl_ev[3] = {};
     bool have_ablation = false;
     Batch batch{};
+    Inputs in{};  // level-0 pixels of the last call's images
     Params prm{};
 
     // stage timing: events[0] before the first stage, events[i + 1] after stage i
@@ -416,7 +417,7 @@ void detect_blocks(const std::vector<Geometry> &geo, bool bits, int k, int borde
             }
             sum += of_pair;
         }
-        const double time = sum / (5.0 * n_sm) + tile;
+        const double time = sum / ((double)kFastCtasPerSm * n_sm) + tile;
         if (best < 0.0 || time < best) { best = time; blocks = cand; }
         if (chosen) break;
     }
@@ -572,7 +573,6 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     const size_t o_images = reserve(sizeof(ImageDesc) * n_img);
     const size_t o_levels = reserve(sizeof(LevelDesc) * n_levels);
     const size_t o_pairs = reserve(sizeof(PairDesc) * n);
-    const size_t o_pyr = reserve(sizeof(int32_t) * (n_levels + 1));
     const size_t o_fast = reserve(sizeof(int32_t) * (n_levels + 1));
     const size_t o_seg = reserve(sizeof(SegRec) * (size_t)(n_segs + 1));
     int pyr_rows[kMaxLevels];
@@ -586,8 +586,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
             n_fast_tiles += 2 * (size_t)(((cx + bx - 1) / bx) * ((cy + by - 1) / by));
         }
     const size_t o_ftl = reserve(sizeof(int32_t) * (n_fast_tiles + 1));
-    const size_t o_ptl = reserve(sizeof(int32_t) * (n_pyr_tiles + 1));
-    const size_t o_porder = reserve(sizeof(int32_t) * (n_pyr_tiles + 1));
+    const size_t o_prec = reserve(sizeof(PyrRec) * (n_pyr_tiles + 1));
     const size_t o_trec = reserve(sizeof(TileRec) * (n_fast_tiles + 1));
     const size_t o_lstart = reserve(sizeof(int32_t) * (kMaxLevels + 1) * n_img);
     const size_t o_tmaps = reserve(sizeof(CUtensorMap) * (size_t)n_levels);
@@ -600,13 +599,11 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     auto images = reinterpret_cast<ImageDesc *>(host.data() + o_images);
     auto levels = reinterpret_cast<LevelDesc *>(host.data() + o_levels);
     auto pairs = reinterpret_cast<PairDesc *>(host.data() + o_pairs);
-    auto pyr_base = reinterpret_cast<int32_t *>(host.data() + o_pyr);
     auto fast_base = reinterpret_cast<int32_t *>(host.data() + o_fast);
     auto seg_rec = reinterpret_cast<SegRec *>(host.data() + o_seg);
     auto ftile_level = reinterpret_cast<int32_t *>(host.data() + o_ftl);
-    auto ptile_level = reinterpret_cast<int32_t *>(host.data() + o_ptl);
     size_t t_off = o_tables, lvl_off = 0, map_off = 0, stage_off = 0, row_off = 0;
-    int li = 0, slot = 0, seg = 0, pyr = 0, fast = 0;
+    int li = 0, slot = 0, seg = 0, fast = 0;
     ctx->staging_off.assign(n_img, 0);
     int32_t *dcounts = ctx->counts.as<int32_t>();
 
@@ -756,10 +753,6 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 }
                 slot += L.cells_x * L.cells_y * k;
                 seg += L.cells_y;
-                pyr_base[li] = pyr;
-                const int ptiles = pyramid_strips(L.W, L.H, L.pyr_rows);
-                for (int q = 0; q < ptiles; ++q) ptile_level[pyr + q] = li;
-                pyr += ptiles;
                 fast_base[li] = fast;
                 const int ftiles = ((L.cells_x + L.bx - 1) / L.bx) * ((L.cells_y + L.by - 1) / L.by);
                 for (int q = 0; q < ftiles; ++q) ftile_level[fast + q] = li;
@@ -777,7 +770,6 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
         P.depth = reinterpret_cast<float *>(rblock + pl.depth);
         P.corr = reinterpret_cast<uint32_t *>(rblock + pl.corr);
     }
-    pyr_base[n_levels] = pyr;
     fast_base[n_levels] = fast;
 
     // detection tile records (the device-side tile geometry, evaluated here)
@@ -857,14 +849,20 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     // one image's levels side by side wait for instructions)
     int pass_first[kMaxLevels + 1] = {};
     {
-        auto porder = reinterpret_cast<int32_t *>(host.data() + o_porder);
-        int count[kMaxLevels] = {};
-        for (int t = 0; t < pyr; ++t) ++count[levels[ptile_level[t]].level];
-        for (int d = 0; d < kMaxLevels; ++d) pass_first[d + 1] = pass_first[d] + count[d];
-        int fill[kMaxLevels];
-        for (int d = 0; d < kMaxLevels; ++d) fill[d] = pass_first[d];
-        for (int t = 0; t < pyr; ++t) porder[fill[levels[ptile_level[t]].level]++] = t;
+        auto prec = reinterpret_cast<PyrRec *>(host.data() + o_prec);
+        int at = 0;
+        for (int d = 0; d < kMaxLevels; ++d) {
+            pass_first[d] = at;
+            for (int l = 0; l < n_levels; ++l) {
+                const LevelDesc &L = levels[l];
+                if (L.level != d) continue;
+                for (int y0 = 0; y0 < L.H; y0 += L.pyr_rows)
+                    for (int x0 = 0; x0 < L.W; x0 += kPyrCols) prec[at++] = { l, x0, y0, 0 };
+            }
+        }
+        pass_first[kMaxLevels] = at;
     }
+    const int pyr = pass_first[kMaxLevels];
     e = cudaMemcpyAsync(ctx->plan.ptr, host.data(), off, cudaMemcpyHostToDevice, ctx->stream);
     if (e != cudaSuccess) return fail(ctx, e);
 
@@ -873,9 +871,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     b.levels = reinterpret_cast<const LevelDesc *>(dplan + o_levels);
     b.orb_maps = reinterpret_cast<const CUtensorMap *>(dplan + o_omaps);
     b.pairs = reinterpret_cast<const PairDesc *>(dplan + o_pairs);
-    b.pyr_tile_base = reinterpret_cast<const int32_t *>(dplan + o_pyr);
-    b.pyr_tile_level = reinterpret_cast<const int32_t *>(dplan + o_ptl);
-    b.pyr_order = reinterpret_cast<const int32_t *>(dplan + o_porder);
+    b.pyr_rec = reinterpret_cast<const PyrRec *>(dplan + o_prec);
     b.pyr_pass = cfg.pyramid_mode == 1 ? 0 : -1;
     for (int d = 0; d <= kMaxLevels; ++d) b.pyr_pass_first[d] = pass_first[d];
     b.fast_tile_base = reinterpret_cast<const int32_t *>(dplan + o_fast);
@@ -913,6 +909,8 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     b.bin_sinf = ctx->d_sinf;
     b.err = reinterpret_cast<uint32_t *>(dcounts + 2 * cfg.max_pairs);
     b.tile_next = reinterpret_cast<uint32_t *>(dcounts + 2 * cfg.max_pairs + 1);
+    b.host_counts = ctx->h_counts;
+    b.host_err = reinterpret_cast<uint32_t *>(ctx->h_counts + 2 * cfg.max_pairs);
     b.prm = ctx->prm;
 
     ctx->keys = keys;
@@ -1145,14 +1143,15 @@ jslam_status jslam_extract_batch(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
     // copies run far below the link rate); other host images use one 2-D
     // copy each into a 128-aligned pitch.
     Batch &b = ctx->batch;
+    Inputs &in = ctx->in;
     const int n_img = 2 * n;
     auto image_of = [&](int img) -> const jslam_image & { return img & 1 ? jobs[img >> 1].right : jobs[img >> 1].left; };
     auto fits_slot = [](const jslam_image &im) { return (size_t)im.pitch <= align_up((size_t)im.width, 128); };
     for (int img = 0; img < n_img;) {
         const jslam_image &im = image_of(img);
         if (im.memory != JSLAM_MEM_HOST) {
-            b.in.ptr[img] = im.data;
-            b.in.pitch[img] = im.pitch;
+            in.ptr[img] = im.data;
+            in.pitch[img] = im.pitch;
             ++img;
             continue;
         }
@@ -1162,8 +1161,8 @@ jslam_status jslam_extract_batch(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
             cudaError_t e = cudaMemcpy2DAsync(dst, dpitch, im.data, im.pitch, im.width, im.height,
                                               cudaMemcpyHostToDevice, ctx->stream);
             if (e != cudaSuccess) return fail(ctx, e);
-            b.in.ptr[img] = dst;
-            b.in.pitch[img] = dpitch;
+            in.ptr[img] = dst;
+            in.pitch[img] = dpitch;
             ++img;
             continue;
         }
@@ -1181,8 +1180,8 @@ jslam_status jslam_extract_batch(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
         if (e != cudaSuccess) return fail(ctx, e);
         for (int k = img; k <= last; ++k) {
             const jslam_image &ik = image_of(k);
-            b.in.ptr[k] = dst + (ik.data - im.data);
-            b.in.pitch[k] = ik.pitch;
+            in.ptr[k] = dst + (ik.data - im.data);
+            in.pitch[k] = ik.pitch;
         }
         img = last + 1;
     }
@@ -1194,7 +1193,7 @@ jslam_status jslam_extract_batch(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
     for (int i = 0; i < JSLAM_STAGE_MATCH; ++i) {
         const NvtxRange range(kStageNames[i]);
         switch (i) {
-        case JSLAM_STAGE_PYRAMID: e = launch_pyramid(b, ctx->stream); break;
+        case JSLAM_STAGE_PYRAMID: e = launch_pyramid(b, in, ctx->stream); break;
         case JSLAM_STAGE_SKIP:
             e = ctx->skip_on ? launch_skipnet(b, ctx->skip_model, ctx->skip_thresh, ctx->stream) : cudaSuccess;
             break;
@@ -1213,7 +1212,7 @@ jslam_status jslam_extract_batch(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
     ctx->have_match = false;
     ctx->have_refine = false;
     ctx->synced = false;
-    return enqueue_counts(ctx);
+    return JSLAM_OK;  // the last kernel wrote the counts to the host
 }
 
 jslam_status jslam_extract(jslam_ctx *ctx, jslam_image left, jslam_image right, int32_t levels, float scale,
@@ -1429,7 +1428,8 @@ jslam_status jslam_sync(jslam_ctx *ctx)
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return fail(ctx, e);
     ctx->synced = true;
-    const uint32_t err = static_cast<uint32_t>(ctx->h_counts[2 * ctx->cfg.max_pairs]);
+    const int32_t *const words = ctx->h_counts + 2 * ctx->cfg.max_pairs;
+    const uint32_t err = static_cast<uint32_t>(words[0] | words[kHostErrOrb]);
     if (err & kErrTimeout) ctx->status = JSLAM_ERR_TIMEOUT;
     else if (err) ctx->status = JSLAM_ERR_CAPACITY;
     return ctx->status;
@@ -1827,7 +1827,7 @@ jslam_status jslam_graph_capture(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
         cudaKernelNodeParams kp{};
         if ((e = cudaGraphKernelNodeGetParams(nodes[i], &kp)) != cudaSuccess) break;
         if (kp.func == pyramid_kernel()) {
-            if (!kp.kernelParams || !kp.kernelParams[0]) { e = cudaErrorInvalidValue; break; }
+            if (!kp.kernelParams || !kp.kernelParams[0] || !kp.kernelParams[1]) { e = cudaErrorInvalidValue; break; }
             ctx->graph_pyr.push_back(nodes[i]);
             ctx->graph_pyr_params.push_back(kp);
             ctx->graph_pyr_batch.push_back(*static_cast<const Batch *>(kp.kernelParams[0]));
@@ -1879,7 +1879,7 @@ jslam_status jslam_graph_launch_jobs(jslam_ctx *ctx, const jslam_stereo_job *job
     if (st != JSLAM_OK) return st;
     // each pyramid launch as captured, with this call's frames; the nodes
     // keep copies of their parameters, so `b` may go out of scope after
-    Inputs in = ctx->batch.in;
+    Inputs in = ctx->in;
     for (int img = 0; img < 2 * n; ++img) {
         const jslam_image &im = img & 1 ? jobs[img >> 1].right : jobs[img >> 1].left;
         in.ptr[img] = im.data;
@@ -1887,9 +1887,7 @@ jslam_status jslam_graph_launch_jobs(jslam_ctx *ctx, const jslam_stereo_job *job
     }
     cudaError_t e = cudaSuccess;
     for (size_t i = 0; i < ctx->graph_pyr.size() && e == cudaSuccess; ++i) {
-        Batch b = ctx->graph_pyr_batch[i];
-        b.in = in;
-        void *args[] = { &b };
+        void *args[] = { &ctx->graph_pyr_batch[i], &in };
         cudaKernelNodeParams kp = ctx->graph_pyr_params[i];
         kp.kernelParams = args;
         kp.extra = nullptr;
@@ -1897,7 +1895,7 @@ jslam_status jslam_graph_launch_jobs(jslam_ctx *ctx, const jslam_stereo_job *job
     }
     if (e == cudaSuccess) e = cudaGraphLaunch(ctx->graph, ctx->stream);
     if (e != cudaSuccess) return fail(ctx, e);
-    ctx->batch.in = in;
+    ctx->in = in;
     return graph_launched(ctx);
 }
 

@@ -12,6 +12,7 @@
 #pragma once
 
 #include <cstdint>
+#include <utility>
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -41,7 +42,7 @@ static_assert((2 * (kPyrAhead + 2) + 1) * kPyrMaxOne <= kPyrRing, "ring");
 static_assert((2 * (kPyrAheadTwo + 2) + 1) * kPyrMaxTwo <= kPyrRing, "ring");
 enum { kPyrCopy = 0, kPyrOne = 1, kPyrTwo = 2, kPyrBytes = 3 };
 // Detection tile: at most this many pixels a side (host picks cells per CTA).
-constexpr int kFastMaxTile = 128, kFastThreads = 128;
+constexpr int kFastMaxTile = 128, kFastThreads = 128, kFastCtasPerSm = 5;
 
 // Row stride of the bit-planes in 16-byte units for a tile of nch 32-pixel
 // chunks: chunks 0..nch (32 bytes each) and a 16-byte pad, an odd count, so
@@ -55,6 +56,10 @@ constexpr int kSkipTileW = 26, kSkipTileH = 12;  // its logits per CTA (grid pit
 constexpr int kRefineMaxW = 10, kRefineMaxL = 7;  // correlation window half-size and search radius limits
 constexpr int kNmsThreads = 128;
 constexpr int kFinThreads = 512;
+
+// Of the host's words after the counts: 0 mirrors the error word, this one has
+// the descriptor kernel's own errors.
+constexpr int kHostErrOrb = 2;
 
 // Device error bits (OR-ed into the context's error word).
 constexpr uint32_t kErrSegment = 1u << 0;  // a segment was larger than kMaxSegment
@@ -194,6 +199,10 @@ struct __align__(16) SegRec {
     uint32_t cdiv;           // reciprocal of c (see recip_of)
     int32_t W0, H0, level;
 };
+// One pyramid strip: its level and first output column and row.
+struct __align__(16) PyrRec {
+    int32_t level, x0, y0, pad;
+};
 // Rank of a slot that is no survivor (SlotInfo's w): no corner, suppressed.
 constexpr int kSlotEmpty = -2, kSlotSuppressed = -1;
 
@@ -202,10 +211,8 @@ struct Batch {
     const LevelDesc *levels;
     const CUtensorMap *orb_maps;    // per level: keypoint boxes of the raw and of the blurred level
     const PairDesc *pairs;
-    const int32_t *pyr_tile_base;   // n_levels + 1
-    const int32_t *pyr_tile_level;  // level index of each pyramid strip
-    const int32_t *pyr_order;       // pyramid strips ordered by level number (cascaded pyramid)
-    int32_t pyr_pass_first[kMaxLevels + 1];  // first entry of pyr_order of each level number
+    const PyrRec *pyr_rec;          // pyramid strips, ordered by level number
+    int32_t pyr_pass_first[kMaxLevels + 1];  // first strip of each level number
     int32_t pyr_pass;               // -1: one launch over every strip; n: the strips of level number n
     const int32_t *fast_tile_base;  // n_levels + 1
     const int32_t *fast_tile_level; // level index of each detection tile
@@ -240,11 +247,12 @@ struct Batch {
     int32_t *skip_any;              // learned skip: per image, nonzero once its proposal skipped a cell
     int32_t nms_kernel;             // 0: a warp per segment where segments allow, 1: a CTA per segment
     int32_t fast_ctas_per_sm;       // persistent detection CTAs per SM (0: as many as fit)
-    Inputs in;
+    int32_t *host_counts;           // pinned host memory: keypoint count per image
+    uint32_t *host_err;             // pinned host memory: the error word as the last kernel of an extraction saw it
 };
 
 // Kernel launchers (one per stage), all on `stream`.
-cudaError_t launch_pyramid(const Batch &b, cudaStream_t stream);
+cudaError_t launch_pyramid(const Batch &b, const Inputs &in, cudaStream_t stream);
 cudaError_t launch_fast_cull(const Batch &b, cudaStream_t stream);
 cudaError_t launch_wait_selftest(uint32_t *err, cudaStream_t stream);
 cudaError_t launch_pfa_nms(const Batch &b, cudaStream_t stream);
@@ -274,5 +282,52 @@ cudaError_t configure_kernels();
 cudaError_t configure_skipnet();
 cudaError_t configure_orb();
 int skipnet_smem_bytes();
+
+#ifdef __CUDACC__
+// Programmatic dependent launch along an extraction's kernels: a kernel
+// launched with launch_after may start while the one before it on the stream
+// still runs, does what needs none of its results (plan tables, barriers), and
+// waits for its completion in after_previous(); let_next() in a kernel says
+// that all its CTAs have started, so that the next one may.  Every kernel of
+// the chain waits before it reads or writes anything that another one touches,
+// so each sees the results of all before it.  Without a predecessor on the
+// stream that allows it, a launch is an ordinary one.
+//
+// Descriptors, matching and what follows always start so, detection, NMS and
+// finalisation only while the detection tiles all run at once (start_early).
+// Beyond that the CTAs that sit and wait take the slots of the kernel before,
+// and persistent ones are spread over the SMs by where that one ended first: us
+// per call with none / with descriptors and matching / with all: one pair of
+// 320x240 76 / 69 / 66, of 1241x376 with refinement and tracking 126 / 115 /
+// 105, of 1920x1080 143 / 142 / 142; 100 of 1241x376 1251 / 1258 / 1348, 16
+// streams of four sizes 375 / 368 / 415, 24 pairs of 647x363 343 / 338 / 381, 16
+// of 800x602 on a cascaded pyramid 390 / 373 / 502.
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+static inline bool start_early(const Batch &b) { return b.fast_tiles <= kFastCtasPerSm * b.n_sm; }
+
+template <class... P, class... A>
+cudaError_t launch_if(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A &&...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A &&...args)
+{
+    return launch_if(true, kernel, grid, block, smem, stream, std::forward<A>(args)...);
+}
+#endif
 
 }  // namespace jslam

@@ -486,7 +486,7 @@ __device__ __forceinline__ void list_items(uint16_t *wlist, int *n, int items, i
 
 // Byte-lane ring test with the cardinal pre-test and the corner table (any
 // P_min, P_max).
-__global__ void __launch_bounds__(kFastThreads) k_fast_cull(Batch b)
+__global__ void __launch_bounds__(kFastThreads) k_fast_cull(const __grid_constant__ Batch b)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ int n_corner, need_lo, n_skipped, n_cand[2];
@@ -514,6 +514,8 @@ __global__ void __launch_bounds__(kFastThreads) k_fast_cull(Batch b)
     }
     for (int i = threadIdx.x; i < kLutWords; i += kFastThreads) lut[i] = __ldg(b.corner_lut + i);
     __syncthreads();
+    after_previous();
+    let_next();
     if (threadIdx.x == 0 && blockIdx.x < b.fast_tiles) issue_tile(b, blockIdx.x, buf0, &bars[0]);
     uint32_t phase0 = 0u, phase1 = 0u;
 
@@ -823,7 +825,7 @@ __device__ __forceinline__ void drain_bits(uint64_t *bars, bool more, int cur, i
 // reading, or the whole ring's SAD); kSkip, the learned cell-skip mode;
 // kTop1, one keypoint per cell (k = 1, the default) or several.
 template <bool kArc, bool kSkip, bool kTop1>
-__global__ void __launch_bounds__(kFastThreads, 5) k_fast_bits(Batch b)
+__global__ void __launch_bounds__(kFastThreads, kFastCtasPerSm) k_fast_bits(const __grid_constant__ Batch b)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ int s_skipped[2];  // skipped cells, by tile parity
@@ -860,6 +862,9 @@ __global__ void __launch_bounds__(kFastThreads, 5) k_fast_bits(Batch b)
         t1 = (int)(blockIdx.x + gridDim.x);
         t2 = t1 + (int)gridDim.x;
         if (t1 < tiles) fetch_rec(b, t1, &recs[1], &bars[3]);
+    }
+    after_previous();
+    if (threadIdx.x == 0) {
         if (wait_tile(&bars[2], 0u)) issue_rec_tile(recs[0], buf0, s_prj[0], &bars[0]);
         else {
             // give up, after waiting once more (same limit) for both
@@ -976,6 +981,7 @@ __global__ void __launch_bounds__(kFastThreads, 5) k_fast_bits(Batch b)
         }
         __syncthreads();
         const bool more = s_more[cur] != 0;
+        if (!more) let_next();  // this CTA's last tile
         if (threadIdx.x == 0 && more) {
             // the next tile's record was fetched one tile ago; the slot of the
             // record after it, the other box and its projections were last
@@ -1187,7 +1193,17 @@ cudaError_t launch_fast_cull(const Batch &b, cudaStream_t stream)
     if (b.fast_ctas_per_sm > 0) per_sm = std::min(per_sm, b.fast_ctas_per_sm);
     const int grid = std::min(b.fast_tiles, per_sm * n_sm);
     void *args[] = { const_cast<Batch *>(&b) };
-    return cudaLaunchKernel(fn, dim3(grid), dim3(kFastThreads), args, (size_t)b.fast_smem, stream);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kFastThreads);
+    cfg.dynamicSmemBytes = (size_t)b.fast_smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];  // as launch_after
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = start_early(b) ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 // Detection CTAs of this batch's launch that fit on one SM at once.

@@ -74,22 +74,38 @@ __device__ __forceinline__ void orb_box(const CUtensorMap *map, const uint8_t *t
 // wavefronts a keypoint took, and those bounded it: 400 000 keypoints 0.260 ms
 // with one warp each and 563 instructions a keypoint; 0.205 ms now, with 328.
 // A warp takes keypoints i, i + stride, ... of its image.
-__global__ void __launch_bounds__(32 * kOrbWarps) k_orient_desc(Batch b)
+__global__ void __launch_bounds__(32 * kOrbWarps) k_orient_desc(const __grid_constant__ Batch b)
 {
     extern __shared__ __align__(128) uint8_t orb_mem[];
     __shared__ __align__(8) uint64_t s_bar[kOrbWarps][2];
     const ImageDesc &I = b.images[blockIdx.y];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t bar = orb_smem(s_bar[warp]);
+    if (lane < 2) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8 * lane) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    __syncwarp();
+    // lane < 27 of the disk: word column w, rows r0, r0 + 3, ...
+    const int w = lane % kDiskWords, r0 = lane / kDiskWords;
+    const float cosf_l = lane < kBins ? __ldg(b.bin_cosf + lane) : 0.0f;
+    const float sinf_l = lane < kBins ? __ldg(b.bin_sinf + lane) : 0.0f;
+    let_next();
+    after_previous();
     const int count = *I.count, stride = gridDim.x * kOrbWarps;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        // the host's mirror of the counts and of the error word (what this
+        // kernel adds goes into a word of its own, so that neither store
+        // replaces the other)
+        b.host_counts[blockIdx.y] = count;
+        if (blockIdx.y == 0) {
+            const uint32_t err = *b.err;
+            if (err) *reinterpret_cast<volatile uint32_t *>(b.host_err) = err;
+        }
+    }
     const int first = blockIdx.x * kOrbWarps + warp;
     if (first >= count) return;
     const KpOut &o = I.out;
     const CUtensorMap *const maps = b.orb_maps + 2 * I.level_base;
     OrbBuf *const buf = reinterpret_cast<OrbBuf *>(orb_mem) + 2 * warp;
-    const uint32_t bar = orb_smem(s_bar[warp]);
-    if (lane < 2) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8 * lane) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    __syncwarp();
     const uint16_t *const xs = o.x, *const ys = o.y;
     const uint8_t *const lv = o.level;
     // the boxes of the keypoint at (x, y) into buffer k.  The keypoint is at
@@ -111,10 +127,6 @@ __global__ void __launch_bounds__(32 * kOrbWarps) k_orient_desc(Batch b)
     int nx = 0, ny = 0, nlev = 0;
     if (first + stride < count) { nx = xs[first + stride]; ny = ys[first + stride]; nlev = lv[first + stride]; }
     uint32_t *const desc = o.desc;
-    // lane < 27 of the disk: word column w, rows r0, r0 + 3, ...
-    const int w = lane % kDiskWords, r0 = lane / kDiskWords;
-    const float cosf_l = lane < kBins ? __ldg(b.bin_cosf + lane) : 0.0f;
-    const float sinf_l = lane < kBins ? __ldg(b.bin_sinf + lane) : 0.0f;
     int my10 = 0, my01 = 0;  // the moments of the keypoint of turn `lane`
 
     int turn = 0;
@@ -136,7 +148,10 @@ __global__ void __launch_bounds__(32 * kOrbWarps) k_orient_desc(Batch b)
         if (!orb_wait(bar + 8 * k2, (turn >> 1) & 1)) {
             // flag it, and wait once more, with the same limit, for the copies
             // in flight, so that none lands in the memory of a CTA that ended
-            if (lane == 0) atomicOr(b.err, kErrTimeout);
+            if (lane == 0) {
+                atomicOr(b.err, kErrTimeout);
+                *reinterpret_cast<volatile uint32_t *>(b.host_err + kHostErrOrb) = kErrTimeout;
+            }
             orb_wait(bar + 8 * k2, (turn >> 1) & 1);
             if (i + stride < count) orb_wait(bar + 8 * (k2 ^ 1), ((turn + 1) >> 1) & 1);
             return;
@@ -227,8 +242,7 @@ cudaError_t launch_orient_desc(const Batch &b, cudaStream_t stream)
     const int turns = orb_turns(b);
     static_assert(16 <= kOrbMaxTurns, "a lane keeps each turn's moments");
     dim3 grid((b.max_capacity + kOrbWarps * turns - 1) / (kOrbWarps * turns), b.n_images);
-    k_orient_desc<<<grid, 32 * kOrbWarps, kOrbSmem, stream>>>(b);
-    return cudaGetLastError();
+    return launch_after(k_orient_desc, grid, dim3(32 * kOrbWarps), kOrbSmem, stream, b);
 }
 
 // Half a warp per left keypoint: its band holds a few dozen candidates at
@@ -236,12 +250,14 @@ cudaError_t launch_orient_desc(const Batch &b, cudaStream_t stream)
 // the chain of gathers from L2 (keypoint -> row index -> X -> descriptor);
 // eight CTAs an SM hide most of it.  200 000 left keypoints: 0.121 ms with a
 // warp each, 0.072 now (0.078 with six CTAs an SM).
-__global__ void __launch_bounds__(256, 8) k_match(Batch b)
+__global__ void __launch_bounds__(256, 8) k_match(const __grid_constant__ Batch b)
 {
     const PairDesc &P = b.pairs[blockIdx.y];
     const int l16 = threadIdx.x & 15;
     const ImageDesc &Il = b.images[P.left];
     const ImageDesc &Ir = b.images[P.right];
+    let_next();
+    after_previous();
     const int count = *Il.count;
     int i = blockIdx.x * 16 + (threadIdx.x >> 4);
     if ((i & ~1) >= count) return;  // whole warps only
@@ -310,10 +326,12 @@ __global__ void __launch_bounds__(256, 8) k_match(Batch b)
 // conservative Y range; lanes take the exact float window test and the
 // Hamming distance, and a warp reduction keeps the smallest (distance,
 // index) and the second-smallest distance.
-__global__ void __launch_bounds__(256) k_track(Batch b, TrackArgs a)
+__global__ void __launch_bounds__(256) k_track(const __grid_constant__ Batch b, const __grid_constant__ TrackArgs a)
 {
     const int lane = threadIdx.x & 31;
     const int q = blockIdx.x * 8 + (threadIdx.x >> 5);
+    let_next();
+    after_previous();
     if (q >= a.n) return;
     const ImageDesc &I = b.images[a.image];
     const int lv = a.level[q];
@@ -381,16 +399,14 @@ __global__ void __launch_bounds__(256) k_track(Batch b, TrackArgs a)
 cudaError_t launch_track(const Batch &b, const TrackArgs &a, cudaStream_t stream)
 {
     if (a.n == 0) return cudaSuccess;
-    k_track<<<(a.n + 7) / 8, 256, 0, stream>>>(b, a);
-    return cudaGetLastError();
+    return launch_after(k_track, dim3((a.n + 7) / 8), dim3(256), 0, stream, b, a);
 }
 
 cudaError_t launch_match(const Batch &b, cudaStream_t stream)
 {
     if (b.n_pairs == 0 || b.max_capacity == 0) return cudaSuccess;
     dim3 grid((b.max_capacity + 15) / 16, b.n_pairs);
-    k_match<<<grid, 256, 0, stream>>>(b);
-    return cudaGetLastError();
+    return launch_after(k_match, grid, dim3(256), 0, stream, b);
 }
 
 }  // namespace jslam

@@ -49,7 +49,7 @@ __device__ __forceinline__ uint4 slot_info(uint32_t pos, int X, int Y, uint32_t 
                       (uint32_t)rank);
 }
 
-__global__ void __launch_bounds__(kNmsThreads) k_pfa_nms(Batch b)
+__global__ void __launch_bounds__(kNmsThreads) k_pfa_nms(const __grid_constant__ Batch b)
 {
     __shared__ uint32_t sk[kMaxSegment];
     __shared__ int alive_total;
@@ -57,6 +57,8 @@ __global__ void __launch_bounds__(kNmsThreads) k_pfa_nms(Batch b)
     const SegRec &R = b.seg_rec[seg];
     const int k = b.prm.k, rad = b.prm.nms_rad, rule = b.prm.rule;
     const int m = R.m, base = R.slot, W0 = R.W0, H0 = R.H0;
+    let_next();
+    after_previous();
     if (m > kMaxSegment) {
         for (int i = threadIdx.x; i < m; i += kNmsThreads)
             b.slot_info[base + i] = slot_info(0u, 0, 0, 0u, 0u, kSlotEmpty);
@@ -109,15 +111,17 @@ __global__ void __launch_bounds__(kNmsThreads) k_pfa_nms(Batch b)
 // projection -> own score and neighbours) is issued for all S slots before
 // the next, so the chains overlap; a CTA of four warps takes four segments.
 template <int S, int RAD>
-__global__ void __launch_bounds__(kNmsThreads) k_pfa_nms_warp(Batch b)
+__global__ void __launch_bounds__(kNmsThreads) k_pfa_nms_warp(const __grid_constant__ Batch b)
 {
     __shared__ __align__(16) uint32_t sk[kNmsThreads / 32][32 * S];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int seg = blockIdx.x * (kNmsThreads / 32) + warp;
+    let_next();
     if (seg >= b.n_segments) return;  // whole warps only
     const SegRec R = b.seg_rec[seg];
     const int k = b.prm.k, rule = b.prm.rule;
     const int m = R.m, base = R.slot, W0 = R.W0, H0 = R.H0;
+    after_previous();
     if (m > 32 * S) {  // the host launches this kernel only when no segment is wider
         for (int i = lane; i < m; i += 32) b.slot_info[base + i] = slot_info(0u, 0, 0, 0u, 0u, kSlotEmpty);
         if (lane == 0) { atomicOr(b.err, kErrSegment); b.seg_count[seg] = 0; }
@@ -194,29 +198,27 @@ __global__ void __launch_bounds__(kNmsThreads) k_pfa_nms_warp(Batch b)
 }
 
 template <int RAD>
-static void launch_nms_warp(const Batch &b, cudaStream_t stream)
+static cudaError_t launch_nms_warp(const Batch &b, cudaStream_t stream)
 {
     constexpr int per = kNmsThreads / 32;
     const int grid = (b.n_segments + per - 1) / per;
-    if (b.max_segment <= 32) k_pfa_nms_warp<1, RAD><<<grid, kNmsThreads, 0, stream>>>(b);
-    else if (b.max_segment <= 64) k_pfa_nms_warp<2, RAD><<<grid, kNmsThreads, 0, stream>>>(b);
-    else k_pfa_nms_warp<3, RAD><<<grid, kNmsThreads, 0, stream>>>(b);
+    const bool early = start_early(b);
+    if (b.max_segment <= 32) return launch_if(early, k_pfa_nms_warp<1, RAD>, dim3(grid), dim3(kNmsThreads), 0, stream, b);
+    if (b.max_segment <= 64) return launch_if(early, k_pfa_nms_warp<2, RAD>, dim3(grid), dim3(kNmsThreads), 0, stream, b);
+    return launch_if(early, k_pfa_nms_warp<3, RAD>, dim3(grid), dim3(kNmsThreads), 0, stream, b);
 }
 
 cudaError_t launch_pfa_nms(const Batch &b, cudaStream_t stream)
 {
     if (b.n_segments == 0) return cudaSuccess;
-    if (b.nms_kernel == 1 || b.max_segment > 96) {
-        k_pfa_nms<<<b.n_segments, kNmsThreads, 0, stream>>>(b);
-    } else {
-        switch (b.prm.nms_rad) {
-        case 0: launch_nms_warp<0>(b, stream); break;
-        case 1: launch_nms_warp<1>(b, stream); break;
-        case 2: launch_nms_warp<2>(b, stream); break;
-        default: launch_nms_warp<3>(b, stream); break;
-        }
+    if (b.nms_kernel == 1 || b.max_segment > 96)
+        return launch_if(start_early(b), k_pfa_nms, dim3(b.n_segments), dim3(kNmsThreads), 0, stream, b);
+    switch (b.prm.nms_rad) {
+    case 0: return launch_nms_warp<0>(b, stream);
+    case 1: return launch_nms_warp<1>(b, stream);
+    case 2: return launch_nms_warp<2>(b, stream);
+    default: return launch_nms_warp<3>(b, stream);
     }
-    return cudaGetLastError();
 }
 
 // Exclusive block-wide prefix sum of v; *total receives the block sum.  `ws`
@@ -319,7 +321,7 @@ constexpr int kFinSegs = 1024;   // segment offsets kept in shared memory (the r
 constexpr int kFinKeep = 4;      // positions of a thread in a round
 constexpr int kFinCluster = 8;   // most CTAs of an image
 
-__global__ void __launch_bounds__(kFinThreads, 2) k_pfa_finalize(Batch b)
+__global__ void __launch_bounds__(kFinThreads, 3) k_pfa_finalize(const __grid_constant__ Batch b)
 {
     __shared__ __align__(16) uint32_t hist[kSelPasses][kSelBins];
     __shared__ uint32_t ws[2][kFinThreads / 32];
@@ -334,6 +336,8 @@ __global__ void __launch_bounds__(kFinThreads, 2) k_pfa_finalize(Batch b)
     const int nl = I.levels, cap = I.max_feats, slot_base = I.slot_base;
     const int seg_base = I.seg_base, seg_count = I.seg_count;
     for (int i = threadIdx.x; i < kSelPasses * kSelBins; i += kFinThreads) (&hist[0][0])[i] = 0;
+    let_next();
+    after_previous();
 
     // Canonical offsets of the segments (level-major, then cell row), by
     // every CTA for itself (the same values).
@@ -573,12 +577,14 @@ cudaError_t launch_pfa_finalize(const Batch &b, cudaStream_t stream)
     cfg.gridDim = dim3(b.n_images * C);
     cfg.blockDim = dim3(kFinThreads);
     cfg.stream = stream;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = C;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_after
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = start_early(b) ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, k_pfa_finalize, b);
 }
 

@@ -334,22 +334,22 @@ __device__ __forceinline__ void pyramid_strip(const Batch &b, const LevelDesc &L
 }
 
 // One warp per CTA: every branch on a strip's rows is uniform for the compiler.
-__global__ void __launch_bounds__(32, kPyrWarpsPerSm) k_pyramid(Batch b)
+__global__ void __launch_bounds__(32, kPyrWarpsPerSm) k_pyramid(const __grid_constant__ Batch b,
+                                                                 const __grid_constant__ Inputs in)
 {
     __shared__ PyrShared S;
+    after_previous();
+    let_next();
     if (blockIdx.x == 0 && threadIdx.x == 0) *b.tile_next = 0u;  // for the detection launch that follows
-    const int tile = __ldg(b.pyr_order + (b.pyr_pass < 0 ? 0 : b.pyr_pass_first[b.pyr_pass]) + blockIdx.x);
-    const int li = __ldg(b.pyr_tile_level + tile);
-    const LevelDesc &L = b.levels[li];
+    const PyrRec R = b.pyr_rec[(b.pyr_pass < 0 ? 0 : b.pyr_pass_first[b.pyr_pass]) + blockIdx.x];
+    const LevelDesc &L = b.levels[R.level];
     const ImageDesc &I = b.images[L.image];
-    const int t = tile - __ldg(b.pyr_tile_base + li);
-    const int tiles_x = (L.W + kPyrCols - 1) / kPyrCols;
-    const int x0 = (t % tiles_x) * kPyrCols, y0 = (t / tiles_x) * L.pyr_rows;
+    const int x0 = R.x0, y0 = R.y0;
     // level 0 reads the input; deeper levels resample the input, or in the
     // cascaded pyramid the level above (complete: an earlier launch)
-    const uint8_t *base = L.src ? L.src : b.in.ptr[L.image];
+    const uint8_t *base = L.src ? L.src : in.ptr[L.image];
     const int W0 = L.src ? L.src_W : I.W0, H0 = L.src ? L.src_H : I.H0;
-    const int pitch0 = L.src ? L.src_pitch : b.in.pitch[L.image];
+    const int pitch0 = L.src ? L.src_pitch : in.pitch[L.image];
     switch (L.pyr_mode) {
     case kPyrCopy: pyramid_strip<kPyrCopy>(b, L, S, base, pitch0, W0, H0, x0, y0); break;
     case kPyrOne: pyramid_strip<kPyrOne>(b, L, S, base, pitch0, W0, H0, x0, y0); break;
@@ -360,11 +360,11 @@ __global__ void __launch_bounds__(32, kPyrWarpsPerSm) k_pyramid(Batch b)
 
 const void *pyramid_kernel() { return reinterpret_cast<const void *>(k_pyramid); }
 
-cudaError_t launch_pyramid(const Batch &b, cudaStream_t stream)
+cudaError_t launch_pyramid(const Batch &b, const Inputs &in, cudaStream_t stream)
 {
     if (b.pyr_tiles == 0) return cudaSuccess;
     if (b.pyr_pass < 0) {
-        k_pyramid<<<b.pyr_tiles, 32, 0, stream>>>(b);
+        k_pyramid<<<b.pyr_tiles, 32, 0, stream>>>(b, in);
         return cudaGetLastError();
     }
     // cascaded: level number n after n - 1, each launch over every image
@@ -373,8 +373,7 @@ cudaError_t launch_pyramid(const Batch &b, cudaStream_t stream)
         if (tiles == 0) continue;
         Batch bn = b;
         bn.pyr_pass = n;
-        k_pyramid<<<tiles, 32, 0, stream>>>(bn);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_after(k_pyramid, dim3(tiles), dim3(32), 0, stream, bn, in);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

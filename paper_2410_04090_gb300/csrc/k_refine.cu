@@ -73,7 +73,7 @@ constexpr int kR5 = 5, kR5Side = 2 * kR5 + 1;  // the default window
 // kernels of the refinement: 86 us with a warp per keypoint and a difference
 // per operation (and the median's digits searched by one thread), 33 now; one pair 27 and
 // 14 us.
-__global__ void __launch_bounds__(256) k_refine5(Batch b, int L, double bf)
+__global__ void __launch_bounds__(256) k_refine5(const __grid_constant__ Batch b, int L, double bf)
 {
     // per half warp: right strip rows of 8 words, left rows of 4 (as loaded),
     // the left window's pixels in 16-bit pairs (0, 2), (1, 3), ... (8, 10), (9, none)
@@ -84,6 +84,8 @@ __global__ void __launch_bounds__(256) k_refine5(Batch b, int L, double bf)
     const PairDesc &P = b.pairs[blockIdx.y];
     const ImageDesc &Il = b.images[P.left];
     const ImageDesc &Ir = b.images[P.right];
+    let_next();
+    after_previous();
     const int count = *Il.count;
     int i = blockIdx.x * 16 + hw;
     if ((i & ~1) >= count) return;  // whole warps only
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(256) k_refine5(Batch b, int L, double bf)
     }
 }
 
-__global__ void __launch_bounds__(256) k_refine(Batch b, int w, int L, double bf)
+__global__ void __launch_bounds__(256) k_refine(const __grid_constant__ Batch b, int w, int L, double bf)
 {
     __shared__ uint8_t s_left[8][kRefLeft];
     __shared__ uint8_t s_right[8][kRefRight];
@@ -199,6 +201,8 @@ __global__ void __launch_bounds__(256) k_refine(Batch b, int w, int L, double bf
     const PairDesc &P = b.pairs[pair];
     const ImageDesc &Il = b.images[P.left];
     const ImageDesc &Ir = b.images[P.right];
+    let_next();
+    after_previous();
     if (i >= *Il.count) return;
     const int j = P.match_idx[i];
     float disp_out = -1.0f, depth_out = 0.0f;
@@ -257,12 +261,15 @@ __global__ void __launch_bounds__(256) k_refine(Batch b, int w, int L, double bf
 
 constexpr int kMedThreads = 512, kMedKeep = 4;  // SADs a thread keeps in registers (the rest read again)
 
-__global__ void __launch_bounds__(kMedThreads) k_refine_median(Batch b)
+__global__ void __launch_bounds__(kMedThreads) k_refine_median(const __grid_constant__ Batch b)
 {
     __shared__ uint32_t hist[2][kMedThreads];
     __shared__ uint32_t ws[kMedThreads / 32];
     __shared__ uint32_t s_digit[2], s_rank[2];
     const PairDesc &P = b.pairs[blockIdx.x];
+    hist[0][threadIdx.x] = hist[1][threadIdx.x] = 0u;
+    let_next();
+    after_previous();
     const int n = *b.images[P.left].count;
     // SADs of the surviving matches (0xFFFFFFFF for the others: a SAD is at
     // most 441 x 510 < 2^18)
@@ -279,7 +286,6 @@ __global__ void __launch_bounds__(kMedThreads) k_refine_median(Batch b)
             if (v != 0xFFFFFFFFu) f(i, v);
         }
     };
-    hist[0][threadIdx.x] = hist[1][threadIdx.x] = 0u;
     __syncthreads();
     uint32_t high = 0, rank = 0;
 #pragma unroll
@@ -324,15 +330,11 @@ __global__ void __launch_bounds__(kMedThreads) k_refine_median(Batch b)
 cudaError_t launch_refine(const Batch &b, int w, int L, double bf, cudaStream_t stream)
 {
     if (b.n_pairs == 0 || b.max_capacity == 0) return cudaSuccess;
-    if (w == kR5) {
-        k_refine5<<<dim3((b.max_capacity + 15) / 16, b.n_pairs), 256, 0, stream>>>(b, L, bf);
-    } else {
-        k_refine<<<dim3((b.max_capacity + 7) / 8, b.n_pairs), 256, 0, stream>>>(b, w, L, bf);
-    }
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e =
+        w == kR5 ? launch_after(k_refine5, dim3((b.max_capacity + 15) / 16, b.n_pairs), dim3(256), 0, stream, b, L, bf)
+                 : launch_after(k_refine, dim3((b.max_capacity + 7) / 8, b.n_pairs), dim3(256), 0, stream, b, w, L, bf);
     if (e != cudaSuccess) return e;
-    k_refine_median<<<b.n_pairs, kMedThreads, 0, stream>>>(b);
-    return cudaGetLastError();
+    return launch_after(k_refine_median, dim3(b.n_pairs), dim3(kMedThreads), 0, stream, b);
 }
 
 }  // namespace jslam

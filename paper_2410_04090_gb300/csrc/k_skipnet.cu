@@ -170,7 +170,7 @@ __device__ __forceinline__ void sync_for_mma()
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-__global__ void __launch_bounds__(kSkipThreads) k_skipnet(Batch b, const SkipModelDev m)
+__global__ void __launch_bounds__(kSkipThreads) k_skipnet(const __grid_constant__ Batch b, const __grid_constant__ SkipModelDev m)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ int s_ok;
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kSkipThreads) k_skipnet(Batch b, const SkipMod
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
-__global__ void k_skipcells(Batch b, float thresh)
+__global__ void k_skipcells(const __grid_constant__ Batch b, float thresh)
 {
     const int img = blockIdx.y;
     const ImageDesc &I = b.images[img];
