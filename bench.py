@@ -73,7 +73,7 @@ WORKLOAD_DESC = {
 # Stage -> kernel name, for the roofline and the ncu summaries.
 KERNELS = {"pyramid": "k_pyramid", "detect": "k_fast_bits", "pfa_nms": "k_pfa_nms",
            "pfa_final": "k_pfa_finalize", "orb": "k_orient_desc", "match": "k_match"}
-KERNEL_SOURCES = {"k_pyramid": "k_pyramid.cu", "k_fast_cull": "k_detect.cu", "k_fast_bits": "k_detect.cu",
+KERNEL_SOURCES = {"k_pyramid": "k_pyramid.cu", "k_fast_bits": "k_detect.cu",
                   "k_pfa_nms": "k_pyca.cu",
                   "k_pfa_finalize": "k_pyca.cu", "k_orient_desc": "k_orb_match.cu", "k_match": "k_orb_match.cu",
                   "k_skipnet": "k_skipnet.cu"}

@@ -16,7 +16,7 @@
 #include "tables.h"
 
 namespace jslam {
-int fast_smem_bytes(int max_box, int max_px, int max_cells, int k, int max_planes);
+int fast_smem_bytes(int max_box, int max_cells, int k, int max_planes);
 const void *pyramid_kernel();
 cudaError_t detect_ctas_that_fit(const Batch &b, int *per_sm);
 }
@@ -296,23 +296,7 @@ jslam_status check_job(const jslam_ctx *ctx, const jslam_stereo_job &j)
     return JSLAM_OK;
 }
 
-// Cells per tile of the per-pixel detection kernel: about tile_w x tile_h
-// pixels, capped in cells x k; the tile width is kept a multiple of 4 pixels
-// where possible so that tiles start on word boundaries.
-void cull_block(int c, int k, int tile_w, int tile_h, int *bx, int *by)
-{
-    int x = tile_w / c > 1 ? tile_w / c : 1;
-    for (int cand = x; cand >= 1; --cand)
-        if ((cand * c) % 4 == 0) { x = cand; break; }
-    int y = tile_h / c > 1 ? tile_h / c : 1;
-    while (x * y * k > kFastMaxCellsPerCta) {
-        if (y > 1) --y; else --x;
-    }
-    *bx = x;
-    *by = y;
-}
-
-// Shared memory of a bit-sliced tile's two boxes and planes.
+// Shared memory of a detection tile's two boxes and planes.
 int bits_tile_bytes(int tw, int th)
 {
     int bw, bh;
@@ -320,7 +304,7 @@ int bits_tile_bytes(int tw, int th)
     return bh * (2 * bw + 16 * bs_row_units((tw + 31) / 32));
 }
 
-// Issue slots of a tile of the bit-sliced kernel with `rows` evaluated rows of
+// Issue slots of a detection tile with `rows` evaluated rows of
 // nch 32-pixel chunks: measured on the 1241x376 sequence, about 1000 a warp's
 // round of ring tests and responses, 115 a round of transposed chunks, 300 a
 // tile.
@@ -336,7 +320,7 @@ struct BitsBlock {
     double cost, tile;  // of the level's tiles, of its dearest one
 };
 
-// Cells per tile of the bit-sliced kernel on a level.  A tile's evaluated
+// Cells per detection tile of a level.  A tile's evaluated
 // rows x 32-pixel chunks are items, a lane each, so cells whose size divides
 // neither 32 nor the CTA leave lanes and warps idle: with about 128 x 64
 // pixels, 22-pixel cells made 132 items for 128 threads.  Of the blocks at
@@ -379,7 +363,7 @@ BitsBlock bits_block(int W, int H, int c, int k, int border, int max_w, int max_
 // 680 / 748 / 783 (default 585), 24 pairs of 647x363 with three keypoints a
 // cell 210 / 201 / 201 / 223 / 238 (202), one pair of 320x240 14.2 / 14.2 / 14.2
 // / 13.0 / 12.3 (12.6).
-void detect_blocks(const std::vector<Geometry> &geo, bool bits, int k, int border, int tile_w, int tile_h, bool chosen,
+void detect_blocks(const std::vector<Geometry> &geo, int k, int border, int tile_w, int tile_h, bool chosen,
                    int n_sm, std::vector<std::array<std::pair<int, int>, kMaxLevels>> &blocks)
 {
     const int n = (int)geo.size();
@@ -390,12 +374,6 @@ void detect_blocks(const std::vector<Geometry> &geo, bool bits, int k, int borde
             eq = geo[p].W[l] == geo[q].W[l] && geo[p].H[l] == geo[q].H[l] && geo[p].c[l] == geo[q].c[l];
         return eq;
     };
-    if (!bits) {
-        for (int p = 0; p < n; ++p)
-            for (int l = 0; l < geo[p].levels; ++l)
-                cull_block(geo[p].c[l], k, tile_w, tile_h, &blocks[p][l].first, &blocks[p][l].second);
-        return;
-    }
     static const int heights[] = { 96, 64, 48, 32, 24, 16 };
     std::vector<std::array<std::pair<int, int>, kMaxLevels>> cand(n);
     double best = -1.0;
@@ -493,18 +471,17 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
 
     const int n_img = 2 * n;
     const int k = cfg.k_per_cell;
-    const bool bits = ctx->prm.p_min == 9 && ctx->prm.p_max == 13;  // the bit-sliced detection kernel
     std::vector<Geometry> geo(n);
     std::vector<std::array<std::pair<int, int>, kMaxLevels>> blocks;  // cells per detection tile of each level
     std::vector<PairLayout> layouts(n);
     std::vector<size_t> result_off(n);
     size_t result_bytes = 0, level_bytes = 0, map_bytes = 0, staging_bytes = 0, table_bytes = 0;
     int n_levels = 0, n_slots = 0, n_segs = 0, max_cap = 0;
-    int max_box = 0, max_px = 0, max_cells = 0, max_planes = 0;
+    int max_box = 0, max_cells = 0, max_planes = 0;
     for (int p = 0; p < n; ++p) {
         geo[p] = level_geometry(jobs[p].left.width, jobs[p].left.height, jobs[p].levels, jobs[p].scale, jobs[p].cell);
     }
-    detect_blocks(geo, bits, k, cfg.border, ctx->tune.tile_w_px, ctx->tune.tile_h_px, ctx->tune_chosen, ctx->n_sm, blocks);
+    detect_blocks(geo, k, cfg.border, ctx->tune.tile_w_px, ctx->tune.tile_h_px, ctx->tune_chosen, ctx->n_sm, blocks);
     for (int p = 0; p < n; ++p) {
         layouts[p] = pair_layout(jobs[p].max_feats);
         result_off[p] = result_bytes;
@@ -526,7 +503,6 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 detect_box(tw, th, &bw, &bh);
                 max_box = std::max(max_box, bw * bh);
                 max_planes = std::max(max_planes, bh * bs_row_units((tw + 31) / 32) * 16);
-                max_px = std::max(max_px, tw * th);
                 max_cells = std::max(max_cells, bx * by);
             }
             n_levels += g.levels;
@@ -573,7 +549,6 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     const size_t o_images = reserve(sizeof(ImageDesc) * n_img);
     const size_t o_levels = reserve(sizeof(LevelDesc) * n_levels);
     const size_t o_pairs = reserve(sizeof(PairDesc) * n);
-    const size_t o_fast = reserve(sizeof(int32_t) * (n_levels + 1));
     const size_t o_seg = reserve(sizeof(SegRec) * (size_t)(n_segs + 1));
     int pyr_rows[kMaxLevels];
     pyramid_strip_rows(geo, cfg.pyramid_mode == 1, ctx->n_sm, pyr_rows);
@@ -585,7 +560,6 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
             const int cx = (geo[p].W[l] + geo[p].c[l] - 1) / geo[p].c[l], cy = (geo[p].H[l] + geo[p].c[l] - 1) / geo[p].c[l];
             n_fast_tiles += 2 * (size_t)(((cx + bx - 1) / bx) * ((cy + by - 1) / by));
         }
-    const size_t o_ftl = reserve(sizeof(int32_t) * (n_fast_tiles + 1));
     const size_t o_prec = reserve(sizeof(PyrRec) * (n_pyr_tiles + 1));
     const size_t o_trec = reserve(sizeof(TileRec) * (n_fast_tiles + 1));
     const size_t o_lstart = reserve(sizeof(int32_t) * (kMaxLevels + 1) * n_img);
@@ -599,9 +573,8 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     auto images = reinterpret_cast<ImageDesc *>(host.data() + o_images);
     auto levels = reinterpret_cast<LevelDesc *>(host.data() + o_levels);
     auto pairs = reinterpret_cast<PairDesc *>(host.data() + o_pairs);
-    auto fast_base = reinterpret_cast<int32_t *>(host.data() + o_fast);
+    std::vector<int32_t> fast_base(n_levels + 1);
     auto seg_rec = reinterpret_cast<SegRec *>(host.data() + o_seg);
-    auto ftile_level = reinterpret_cast<int32_t *>(host.data() + o_ftl);
     size_t t_off = o_tables, lvl_off = 0, map_off = 0, stage_off = 0, row_off = 0;
     int li = 0, slot = 0, seg = 0, fast = 0;
     ctx->staging_off.assign(n_img, 0);
@@ -709,11 +682,10 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 t_off += align_up((size_t)(L.W + L.H) * 2, 16);
 
                 // TMA map of the raw level (the box x is rounded down to 16
-                // bytes); the per-pixel kernel reads words, so its tiles have
-                // to start on word boundaries
+                // bytes)
                 L.tmap = nullptr;
                 PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
-                if (encode && (bits || (L.bx * L.c) % 4 == 0)) {
+                if (encode) {
                     CUtensorMap map;  // encoded into an aligned object, then copied into the plan
                     const cuuint64_t dims[2] = { (cuuint64_t)L.W, (cuuint64_t)L.H };
                     const cuuint64_t strides[1] = { (cuuint64_t)L.pitch };
@@ -755,7 +727,6 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 seg += L.cells_y;
                 fast_base[li] = fast;
                 const int ftiles = ((L.cells_x + L.bx - 1) / L.bx) * ((L.cells_y + L.by - 1) / L.by);
-                for (int q = 0; q < ftiles; ++q) ftile_level[fast + q] = li;
                 fast += ftiles;
             }
             I.slot_count = slot - I.slot_base;
@@ -830,7 +801,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     // changes no result.  Used by default too (100 pairs of 1241x376: detection
     // 0.597 -> 0.585 ms, 12 of 752x480 with the learned skip 101 -> 95 us, one
     // of 1920x1080 45 -> 42 us); with a chosen tuning its own order.
-    if (ctx->tune.tile_order == 1 || (bits && !ctx->tune_chosen)) {
+    if (ctx->tune.tile_order == 1 || !ctx->tune_chosen) {
         std::vector<std::pair<int, int>> work(fast);
         for (int t = 0; t < fast; ++t) {
             const TileRec &R = trec[t];
@@ -874,18 +845,15 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     b.pyr_rec = reinterpret_cast<const PyrRec *>(dplan + o_prec);
     b.pyr_pass = cfg.pyramid_mode == 1 ? 0 : -1;
     for (int d = 0; d <= kMaxLevels; ++d) b.pyr_pass_first[d] = pass_first[d];
-    b.fast_tile_base = reinterpret_cast<const int32_t *>(dplan + o_fast);
     b.seg_rec = reinterpret_cast<const SegRec *>(dplan + o_seg);
-    b.fast_tile_level = reinterpret_cast<const int32_t *>(dplan + o_ftl);
     b.tile_rec = reinterpret_cast<const TileRec *>(dplan + o_trec);
     b.n_images = n_img; b.n_levels = n_levels; b.n_pairs = n; b.n_segments = n_segs;
     b.max_segment = 0;
     for (int l = 0; l < n_levels; ++l) b.max_segment = std::max(b.max_segment, levels[l].cells_x * k);
     b.pyr_tiles = pyr; b.fast_tiles = fast; b.max_capacity = max_cap;
-    b.fast_max_box = max_box; b.fast_max_px = max_px; b.fast_max_cells = max_cells;
-    b.fast_bits = bits;
+    b.fast_max_box = max_box; b.fast_max_cells = max_cells;
     b.fast_max_planes = max_planes;
-    b.fast_smem = fast_smem_bytes(max_box, max_px, max_cells, k, b.fast_bits ? max_planes : 0);
+    b.fast_smem = fast_smem_bytes(max_box, max_cells, k, max_planes);
     b.corner_lut = ctx->d_lut;
     b.skip_max_tiles = skip_max_tiles;
     b.skip_any = ctx->skip_on ? ctx->skipbuf.as<int32_t>(skip_off) : nullptr;
@@ -1197,7 +1165,7 @@ jslam_status jslam_extract_batch(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
         case JSLAM_STAGE_SKIP:
             e = ctx->skip_on ? launch_skipnet(b, ctx->skip_model, ctx->skip_thresh, ctx->stream) : cudaSuccess;
             break;
-        case JSLAM_STAGE_DETECT: e = launch_fast_cull(b, ctx->stream); break;
+        case JSLAM_STAGE_DETECT: e = launch_detect(b, ctx->stream); break;
         case JSLAM_STAGE_PFA_NMS: e = launch_pfa_nms(b, ctx->stream); break;
         case JSLAM_STAGE_PFA_FINAL: e = launch_pfa_finalize(b, ctx->stream); break;
         default: e = launch_orient_desc(b, ctx->stream); break;

@@ -159,7 +159,7 @@ struct Inputs {
 };
 
 // Everything the kernels of one extraction need.
-// One detection tile of the bit-sliced kernel, prepared on the host: the
+// One detection tile, prepared on the host: the
 // tile's place in its level, the level's and image's scalars, and the
 // 16-byte-aligned ranges of the level's s0 projection tables that cover the
 // tile's columns and rows.  The kernel copies it into shared memory with a
@@ -214,17 +214,14 @@ struct Batch {
     const PyrRec *pyr_rec;          // pyramid strips, ordered by level number
     int32_t pyr_pass_first[kMaxLevels + 1];  // first strip of each level number
     int32_t pyr_pass;               // -1: one launch over every strip; n: the strips of level number n
-    const int32_t *fast_tile_base;  // n_levels + 1
-    const int32_t *fast_tile_level; // level index of each detection tile
     const SegRec *seg_rec;          // one per segment
     int32_t n_images, n_levels, n_pairs, n_segments;
     int32_t max_segment;            // largest segment (cells_x x k slots) of the batch
     int32_t pyr_tiles, fast_tiles;  // pyramid strips, detection tiles
     int32_t max_capacity;           // largest keypoint capacity of any image
     int32_t fast_smem;              // dynamic shared memory of the detection kernel
-    int32_t fast_max_box, fast_max_px, fast_max_cells;  // its tile layout maxima
+    int32_t fast_max_box, fast_max_cells;  // its tile layout maxima
     int32_t fast_max_planes;        // bit-plane bytes of the largest tile box
-    int32_t fast_bits;              // 1: bit-sliced ring test (P_min = 9, P_max = 13)
     const TileRec *tile_rec;        // one per detection tile
     uint32_t *tile_next;            // detection tiles taken beyond each CTA's first three (zero before the launch)
     const uint32_t *corner_lut;     // bit m: P_min <= longest circular run of m <= P_max
@@ -253,7 +250,7 @@ struct Batch {
 
 // Kernel launchers (one per stage), all on `stream`.
 cudaError_t launch_pyramid(const Batch &b, const Inputs &in, cudaStream_t stream);
-cudaError_t launch_fast_cull(const Batch &b, cudaStream_t stream);
+cudaError_t launch_detect(const Batch &b, cudaStream_t stream);
 cudaError_t launch_wait_selftest(uint32_t *err, cudaStream_t stream);
 cudaError_t launch_pfa_nms(const Batch &b, cudaStream_t stream);
 cudaError_t launch_pfa_finalize(const Batch &b, cudaStream_t stream);
