@@ -117,7 +117,7 @@ struct ImageDesc {
     int32_t *level_start;    // kMaxLevels + 1 entries
     // row index of the canonical list, per level H0 + 1 entries: entry v is
     // the first index of the level whose Y is >= v (the level's end if none);
-    // written by k_pfa_finalize for levels with keypoints, read by k_match
+    // written by k_orient_desc for levels with keypoints, read by k_match
     int32_t *row_first;
     KpOut out;
     // learned cell-skip (skip == nullptr: exact mode)

@@ -13,7 +13,8 @@
 //                IEEE double with explicit rounding inside it, so the sector
 //                equals the one the host-side definition gives); the 256 BRIEF
 //                comparisons read the patch 32 at a time and are packed into
-//                words by a ballot.
+//                words by a ballot.  The row index of the canonical list that the
+//                matching reads is written here too.
 // k_match        half a warp per left keypoint: for each right level within one
 //                of the keypoint's level, takes the s0 row band of the
 //                canonical (level, y, x) list (Y is non-decreasing in y) from
@@ -101,9 +102,27 @@ __global__ void __launch_bounds__(32 * kOrbWarps) k_orient_desc(const __grid_con
             if (err) *reinterpret_cast<volatile uint32_t *>(b.host_err) = err;
         }
     }
+    const KpOut &o = I.out;
+    // The row index of the canonical list, for the stereo matching: entry v of
+    // level l's table is the first index of the level whose Y is >= v, else
+    // the level's end, for v = 0 .. H0.  Keypoint j owns the entries (Y[j - 1],
+    // Y[j]] when it is not the level's first (below); a CTA fills a level's
+    // entries up to the first keypoint's Y (the level's start) and after the
+    // last one's (its end).  Here and not at the end of the finalisation, where
+    // it took one more barrier of the cluster.
+    const int rows = I.H0 + 1;
+    for (int l = blockIdx.x; l < I.levels; l += gridDim.x) {
+        const int s = I.level_start[l], e = I.level_start[l + 1];
+        if (s == e) continue;
+        const int ys = o.Y[s], ye = o.Y[e - 1];
+        int32_t *const rf = I.row_first + (size_t)l * rows;
+        for (int v = threadIdx.x; v < rows; v += 32 * kOrbWarps) {
+            if (v <= ys) rf[v] = s;
+            else if (v > ye) rf[v] = e;
+        }
+    }
     const int first = blockIdx.x * kOrbWarps + warp;
     if (first >= count) return;
-    const KpOut &o = I.out;
     const CUtensorMap *const maps = b.orb_maps + 2 * I.level_base;
     OrbBuf *const buf = reinterpret_cast<OrbBuf *>(orb_mem) + 2 * warp;
     const uint16_t *const xs = o.x, *const ys = o.y;
@@ -124,6 +143,16 @@ __global__ void __launch_bounds__(32 * kOrbWarps) k_orient_desc(const __grid_con
     };
     int x = xs[first], y = ys[first], level = lv[first];
     issue(x, y, level, 0);
+    // the row-index entries of this warp's keypoints, a lane each (a warp has
+    // at most kOrbMaxTurns)
+    if (const int j = first + lane * stride; j < count) {
+        const int l = lv[j], Yj = o.Y[j], Yp = j > 0 ? (int)o.Y[j - 1] : 0;
+        if (j != I.level_start[l]) {
+            int32_t *const rf = I.row_first + (size_t)l * rows;
+            for (int v = Yp + 1; v <= Yj; ++v) rf[v] = j;
+        }
+    }
+    __syncwarp();
     int nx = 0, ny = 0, nlev = 0;
     if (first + stride < count) { nx = xs[first + stride]; ny = ys[first + stride]; nlev = lv[first + stride]; }
     uint32_t *const desc = o.desc;

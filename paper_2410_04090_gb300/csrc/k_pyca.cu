@@ -15,7 +15,7 @@
 //                 into canonical positions (level, y, x), clears the score map
 //                 entries it used, applies the keypoint cap by a radix select
 //                 on (K_l, K_r, response) with canonical order breaking ties,
-//                 and writes the compacted keypoint list and its row index.
+//                 and writes the compacted keypoint list.
 #include "jslam_internal.h"
 
 namespace jslam {
@@ -246,13 +246,17 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *ws, ui
 // launch_pfa_finalize): the candidate slots and then the canonical positions
 // are shared out over its CTAs, the histograms of the cap's radix select are
 // summed through distributed shared memory, and a cluster barrier ends each
-// phase.
+// phase: the slots' and those of the select's three passes.  A thread that sums
+// the others' histograms also keeps what the CTAs before its own have of it, so
+// the place of a CTA's first keypoint needs no barrier more.
 //
 // What bounds it: latency -- a chain of barriers and dependent reads whose
 // data lie in L2; the bytes are few.  One CTA of 1024 threads an image left
 // the chip idle for small batches.  Stage times, before and now (us): one
-// 1920x1080 pair (16 000 slots an image) 96 and 29, one 1241x376 pair 31 and
-// 22, 16 mixed pairs 98 and 33, 100 pairs of 1241x376 47 and 37.
+// 1920x1080 pair (16 000 slots an image) 96 and 25, one 1241x376 pair 31 and
+// 18, 16 mixed pairs 98 and 27, 100 pairs of 1241x376 47 and 33 (29, 22, 33 and
+// 37 with two barriers more, one of them for the row index that
+// k_orient_desc makes now).
 
 __device__ __forceinline__ uint32_t cluster_rank()
 {
@@ -282,37 +286,6 @@ __device__ __forceinline__ uint4 ld_cluster(const void *p, uint32_t rank)
     return v;
 }
 
-// Row index of an image's canonical list, for the stereo matching (all
-// threads of the cluster, after the barrier that completes the keypoints'
-// levels and Y; level starts in lstart, kMaxLevels + 1 entries whose last is
-// the count).  Entry v of level l's table is the first index of the level
-// whose Y is >= v, else the level's end: keypoint j owns the entries
-// (Y[j - 1], Y[j]] when it is not the level's first; the entries up to the
-// first keypoint's Y (the level's start) and after the last one's (its end)
-// are spread over the threads.  Every level with keypoints gets all H0 + 1
-// entries.
-__device__ __forceinline__ void fill_row_index(const ImageDesc &I, const int *lstart, int thread, int threads)
-{
-    const int rows = I.H0 + 1, keep = lstart[kMaxLevels];
-    const KpOut &o = I.out;
-    for (int j = thread; j < keep; j += threads) {
-        const int l = o.level[j], Yj = o.Y[j], Yp = j > 0 ? (int)o.Y[j - 1] : 0;
-        if (j == lstart[l]) continue;
-        int32_t *rf = I.row_first + (size_t)l * rows;
-        for (int v = Yp + 1; v <= Yj; ++v) rf[v] = j;
-    }
-    for (int l = 0; l < I.levels; ++l) {
-        const int s = lstart[l], e = lstart[l + 1];
-        if (s == e) continue;
-        const int ys = o.Y[s], ye = o.Y[e - 1];
-        int32_t *rf = I.row_first + (size_t)l * rows;
-        for (int v = thread; v < rows; v += threads) {
-            if (v <= ys) rf[v] = s;
-            else if (v > ye) rf[v] = e;
-        }
-    }
-}
-
 // Digits of the radix select over the cap priorities K_l << 27 | K_r << 12 |
 // r (31 bits: K_l <= 8, K_r <= 8 x 4080, r <= 4080), high to low, of 11, 11
 // and 9 bits: the first one reaches into K_r, since almost every K_l is 1 or 2.
@@ -325,9 +298,9 @@ __global__ void __launch_bounds__(kFinThreads, 3) k_pfa_finalize(const __grid_co
 {
     __shared__ __align__(16) uint32_t hist[kSelPasses][kSelBins];
     __shared__ uint32_t ws[2][kFinThreads / 32];
-    __shared__ __align__(16) uint32_t s_above[4];  // of this CTA's positions: above the threshold, at it
+    __shared__ uint32_t s_before[2];  // positions of the CTAs before: above the threshold, at it
     __shared__ uint32_t sh_digit[kSelPasses], sh_need[kSelPasses];
-    __shared__ int lfirst[kMaxLevels + 1], lstart[kMaxLevels + 1];
+    __shared__ int lfirst[kMaxLevels + 1];
     __shared__ int s_off[kFinSegs];
     const int C = (int)cluster_size(), rank = (int)cluster_rank();
     const int lg = 31 - __clz(C);  // a power of two
@@ -336,6 +309,7 @@ __global__ void __launch_bounds__(kFinThreads, 3) k_pfa_finalize(const __grid_co
     const int nl = I.levels, cap = I.max_feats, slot_base = I.slot_base;
     const int seg_base = I.seg_base, seg_count = I.seg_count;
     for (int i = threadIdx.x; i < kSelPasses * kSelBins; i += kFinThreads) (&hist[0][0])[i] = 0;
+    if (threadIdx.x < 2) s_before[threadIdx.x] = 0u;
     let_next();
     after_previous();
 
@@ -408,6 +382,9 @@ __global__ void __launch_bounds__(kFinThreads, 3) k_pfa_finalize(const __grid_co
     const bool capped = S > cap;
     uint32_t T = 0, mask = 0;
     int quota = 0;
+    // this thread's digits' share of the positions of the CTAs before this one:
+    // with a prefix of T and a larger digit, and equal to T
+    uint32_t before_up = 0, before_tie = 0;
     // f(priority) of every position of this thread
     const auto each = [&](auto f) {
         for (int base = g0; base < g1; base += kRound) {
@@ -432,12 +409,13 @@ __global__ void __launch_bounds__(kFinThreads, 3) k_pfa_finalize(const __grid_co
             // has four digits, from the largest down
             static_assert(kSelBins == 4 * kFinThreads, "four digits a thread");
             const int d0 = kSelBins - 4 - 4 * (int)threadIdx.x;
-            uint4 n4 = make_uint4(0u, 0u, 0u, 0u);
+            uint4 n4 = make_uint4(0u, 0u, 0u, 0u), p4 = n4;
 #pragma unroll
             for (int c = 0; c < kFinCluster; ++c)
                 if (c < C) {
                     const uint4 h = ld_cluster(&hist[pass][d0], (uint32_t)c);
                     n4.x += h.x; n4.y += h.y; n4.z += h.z; n4.w += h.w;
+                    if (c + 1 == rank) p4 = n4;
                 }
             const int n[4] = { (int)n4.w, (int)n4.z, (int)n4.y, (int)n4.x };
             uint32_t tot;
@@ -451,12 +429,21 @@ __global__ void __launch_bounds__(kFinThreads, 3) k_pfa_finalize(const __grid_co
                 cum += n[j];
             }
             __syncthreads();
-            T |= sh_digit[pass] << sh;
+            const int digit = (int)sh_digit[pass];
+            const uint32_t p[4] = { p4.w, p4.z, p4.y, p4.x };
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                before_up += d0 + 3 - j > digit ? p[j] : 0u;
+                if (pass == kSelPasses - 1) before_tie += d0 + 3 - j == digit ? p[j] : 0u;
+            }
+            T |= (uint32_t)digit << sh;
             mask = ~((1u << sh) - 1u);
             need = (int)sh_need[pass];
         }
         quota = need;
     }
+    // this CTA has read the others' histograms (waited for at the end)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     const int keep = capped ? cap : S;
 
     // Positions before this CTA's that are above the threshold and at it (not
@@ -469,33 +456,17 @@ __global__ void __launch_bounds__(kFinThreads, 3) k_pfa_finalize(const __grid_co
         return c;
     };
     static_assert(kRound < 65536, "a round's counts fit 16 bits");
-    if (capped) {  // T >= 1: the positions past g1 (priority 0) count for nothing
-        uint32_t up = 0, tie = 0;
-        for (int base = g0; base < g1; base += kRound) {
-            if (base != g0) load(base);
-            const uint32_t c = counts();
-            up += c & 0xFFFFu;
-            tie += c >> 16;
-        }
-        if (g1 - g0 > kRound) load(g0);
-        if (threadIdx.x < 2) s_above[threadIdx.x] = 0u;
-        __syncthreads();
-        up = __reduce_add_sync(0xFFFFFFFFu, up);
-        tie = __reduce_add_sync(0xFFFFFFFFu, tie);
+    if (capped && C > 1) {
+        before_up = __reduce_add_sync(0xFFFFFFFFu, before_up);
+        before_tie = __reduce_add_sync(0xFFFFFFFFu, before_tie);
         if ((threadIdx.x & 31) == 0) {
-            atomicAdd(&s_above[0], up);
-            atomicAdd(&s_above[1], tie);
+            atomicAdd(&s_before[0], before_up);
+            atomicAdd(&s_before[1], before_tie);
         }
-        cluster_sync();
-        carry_up = 0;
-#pragma unroll
-        for (int c = 0; c < kFinCluster - 1; ++c)
-            if (c < rank) {
-                const uint4 v = ld_cluster(s_above, (uint32_t)c);
-                carry_up += (int)v.x;
-                carry_tie += (int)v.y;
-            }
+        __syncthreads();
+        carry_tie = (int)s_before[1];
     }
+    if (capped) carry_up = (int)s_before[0];
 
     // the kept positions in order; position g is preceded by up + min(tie, quota) kept ones
     const KpOut &o = I.out;
@@ -545,10 +516,8 @@ __global__ void __launch_bounds__(kFinThreads, 3) k_pfa_finalize(const __grid_co
             *I.count_hdr = keep;
         }
     }
-    cluster_sync();
-    if (threadIdx.x <= kMaxLevels) lstart[threadIdx.x] = I.level_start[threadIdx.x];
-    __syncthreads();
-    fill_row_index(I, lstart, rank * kFinThreads + (int)threadIdx.x, C * kFinThreads);
+    // no CTA ends while another may read its histograms
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // CTAs per image.  More of them shorten the chains of a small batch, each
