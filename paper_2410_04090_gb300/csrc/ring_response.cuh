@@ -17,26 +17,39 @@
 
 namespace jslam {
 
+// What bounds it: instructions (a lane a corner), so no step loops or branches
+// by its data: ring flags are shifted in by their sign bits, runs and the
+// positions on them come by doubling, and the sum over the positions is four
+// byte dot products.  Detection of 24 pairs of 647x363 with three keypoints a
+// cell and this response: 201 us by walking the ring's bits, 100 so (86 with
+// the whole ring's response).
+
 // Longest circular run of set bits of a 16-bit mask (16 for 0xFFFF), and the
 // positions lying on a run of that length.
 __device__ __forceinline__ uint32_t ring_arc_positions(uint32_t m, int *len)
 {
-    const uint32_t m32 = m | (m << 16);  // bit i is ring position i mod 16
-    uint32_t x = m32;
+    // x_k, bit i: a run of k from position i on (bit i is position i mod 16)
+    const uint32_t x1 = m | (m << 16), x2 = x1 & (x1 >> 1), x4 = x2 & (x2 >> 2), x8 = x4 & (x4 >> 4);
+    uint32_t starts = 0xFFFFu, t;  // of the runs of n or more
     int n = 0;
-    while (x) {
-        x &= x >> 1;
-        ++n;
-    }
-    n = n > 16 ? 16 : n;
+    t = starts & x8;
+    if (t) { starts = t; n = 8; }
+    t = starts & (x4 >> n);
+    if (t) { starts = t; n += 4; }
+    t = starts & (x2 >> n);
+    if (t) { starts = t; n += 2; }
+    t = starts & (x1 >> n);
+    if (t) { starts = t; n += 1; }
+    if (m == 0xFFFFu) { starts = m; n = 16; }
     *len = n;
-    if (n == 0) return 0u;
-    uint32_t starts = m32;  // bit q: positions q .. q + n - 1 all set
-    for (int i = 1; i < n; ++i) starts &= m32 >> i;
-    starts &= 0xFFFFu;
-    uint32_t on = 0;
-    for (int j = 0; j < n; ++j) on |= (starts << j) | (starts >> (16 - j));
-    return on & 0xFFFFu;
+    // every start's n positions: windows of the largest power of two, twice
+    uint32_t on = starts;
+    int w = 1;
+    if (n >= 2) { on |= on << 1; w = 2; }
+    if (n >= 4) { on |= on << 2; w = 4; }
+    if (n >= 8) { on |= on << 4; w = 8; }
+    if (n > 0) on |= on << (n - w);  // a full ring's starts are all positions
+    return n > 0 ? (on | (on >> 16)) & 0xFFFFu : 0u;
 }
 
 // Arc response of the pixel at p (rows rowb bytes apart) for threshold eps
@@ -45,27 +58,36 @@ __device__ __forceinline__ int ring_arc(const uint8_t *p, int rowb, int eps, int
 {
     constexpr int DX[16] = { 0, 1, 2, 3, 3, 3, 2, 1, 0, -1, -2, -3, -3, -3, -2, -1 };
     constexpr int DY[16] = { 3, 3, 2, 1, 0, -1, -2, -3, -3, -3, -2, -1, 0, 1, 2, 3 };
-    const int ic = p[0];
-    int ad[16];
-    uint32_t mb = 0, md = 0;
+    const int hi = (int)p[0] + eps, lo = (int)p[0] - eps;
+    uint32_t v[16], mb = 0, md = 0;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const int d = (int)p[DY[k] * rowb + DX[k]] - ic;
-        ad[k] = d < 0 ? -d : d;
-        mb |= (uint32_t)(d > eps) << k;
-        md |= (uint32_t)(d < -eps) << k;
+    for (int k = 15; k >= 0; --k) {
+        v[k] = p[DY[k] * rowb + DX[k]];
+        mb = __funnelshift_l((uint32_t)(hi - (int)v[k]), mb, 1);
+        md = __funnelshift_l((uint32_t)((int)v[k] - lo), md, 1);
     }
+    uint32_t ring[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        ring[i] = v[4 * i] + (v[4 * i + 1] << 8) + ((v[4 * i + 2] << 16) + (v[4 * i + 3] << 24));
     int best = 0;
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
+    const auto polarity = [&](bool bright) {
         int n;
-        const uint32_t on = ring_arc_positions(s ? md : mb, &n);
-        if (n < p_min || n > p_max || n == 0) continue;
-        int sum = 0;
+        const uint32_t on = ring_arc_positions(bright ? mb : md, &n);
+        uint32_t sum = 0;  // of the pixels on the runs
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-            if ((on >> k) & 1u) sum += ad[k] - eps;
-        best = sum > best ? sum : best;
+        for (int i = 0; i < 4; ++i)  // four bits to the low bits of four bytes
+            sum = __dp4a(ring[i], (((on >> (4 * i)) & 0xFu) * 0x00204081u) & 0x01010101u, sum);
+        const int c = __popc(on);
+        const int r = bright ? (int)sum - c * hi : c * lo - (int)sum;
+        if (n >= p_min && n <= p_max) best = max(best, r);
+    };
+    // nine of the sixteen positions: one polarity at most
+    if (p_min >= 9) {
+        polarity(__popc(mb) > __popc(md));
+    } else {
+        polarity(true);
+        polarity(false);
     }
     return best;
 }
