@@ -220,6 +220,10 @@ struct jslam_ctx {
     bool have_ablation = false;
     Batch batch{};
     Inputs in{};  // level-0 pixels of the last call's images
+    // upload of host frames in parts (plan: parts and the first strip of each)
+    cudaStream_t copy_stream = nullptr;
+    cudaEvent_t copy_ev[kUploadParts + 1] = {};  // [0] the context stream's work before, [p + 1] part p is up
+    int up_parts = 1, up_first[kUploadParts + 1] = {};
     Params prm{};
 
     // stage timing: events[0] before the first stage, events[i + 1] after stage i
@@ -450,6 +454,9 @@ int pyramid_mode_of(const uint32_t *tapx, int W, int src_W)
 }
 
 // Build (or reuse) the plan of a batch and upload it.
+// The image after the last one of upload part `part` of a batch of n pairs.
+int upload_end(int n, int part, int parts) { return 2 * (int)((long long)n * (part + 1) / parts); }
+
 jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
 {
     const jslam_config &cfg = ctx->cfg;
@@ -818,22 +825,40 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     // number n once level n - 1 of every image is complete; in one launch the
     // strips that run together then mostly execute the same code (strips of
     // one image's levels side by side wait for instructions)
-    int pass_first[kMaxLevels + 1] = {};
+    // A batch of host frames comes up in parts (neighbouring images), and its
+    // strips are ordered by part first.
+    int pass_first[kMaxLevels + 1] = {}, pyr = 0;
+    ctx->up_parts = 1;
+    if (cfg.pyramid_mode == 0) {
+        size_t bytes = 0;
+        bool host_only = true;
+        for (int p = 0; p < n; ++p) {
+            bytes += 2 * (size_t)geo[p].W[0] * geo[p].H[0];
+            host_only &= jobs[p].left.memory == JSLAM_MEM_HOST && jobs[p].right.memory == JSLAM_MEM_HOST;
+        }
+        if (host_only)
+            ctx->up_parts = (int)std::min<size_t>(std::max<size_t>(bytes / kUploadPartBytes, 1), std::min(n, kUploadParts));
+    }
     {
         auto prec = reinterpret_cast<PyrRec *>(host.data() + o_prec);
-        int at = 0;
-        for (int d = 0; d < kMaxLevels; ++d) {
-            pass_first[d] = at;
-            for (int l = 0; l < n_levels; ++l) {
-                const LevelDesc &L = levels[l];
-                if (L.level != d) continue;
-                for (int y0 = 0; y0 < L.H; y0 += L.pyr_rows)
-                    for (int x0 = 0; x0 < L.W; x0 += kPyrCols) prec[at++] = { l, x0, y0, 0 };
+        for (int part = 0, l0 = 0; part < ctx->up_parts; ++part) {
+            const int end = upload_end(n, part, ctx->up_parts);
+            int l1 = l0;
+            while (l1 < n_levels && levels[l1].image < end) ++l1;
+            ctx->up_first[part] = pyr;
+            for (int d = 0; d < kMaxLevels; ++d) {
+                pass_first[d] = pyr;
+                for (int l = l0; l < l1; ++l) {
+                    const LevelDesc &L = levels[l];
+                    if (L.level != d) continue;
+                    for (int y0 = 0; y0 < L.H; y0 += L.pyr_rows)
+                        for (int x0 = 0; x0 < L.W; x0 += kPyrCols) prec[pyr++] = { l, x0, y0, 0 };
+                }
             }
+            l0 = l1;
         }
-        pass_first[kMaxLevels] = at;
+        pass_first[kMaxLevels] = ctx->up_first[ctx->up_parts] = pyr;
     }
-    const int pyr = pass_first[kMaxLevels];
     e = cudaMemcpyAsync(ctx->plan.ptr, host.data(), off, cudaMemcpyHostToDevice, ctx->stream);
     if (e != cudaSuccess) return fail(ctx, e);
 
@@ -843,7 +868,8 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     b.orb_maps = reinterpret_cast<const CUtensorMap *>(dplan + o_omaps);
     b.pairs = reinterpret_cast<const PairDesc *>(dplan + o_pairs);
     b.pyr_rec = reinterpret_cast<const PyrRec *>(dplan + o_prec);
-    b.pyr_pass = cfg.pyramid_mode == 1 ? 0 : -1;
+    b.pyr_cascaded = cfg.pyramid_mode == 1;
+    b.pyr_first = 0;
     for (int d = 0; d <= kMaxLevels; ++d) b.pyr_pass_first[d] = pass_first[d];
     b.seg_rec = reinterpret_cast<const SegRec *>(dplan + o_seg);
     b.tile_rec = reinterpret_cast<const TileRec *>(dplan + o_trec);
@@ -1115,7 +1141,52 @@ jslam_status jslam_extract_batch(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
     const int n_img = 2 * n;
     auto image_of = [&](int img) -> const jslam_image & { return img & 1 ? jobs[img >> 1].right : jobs[img >> 1].left; };
     auto fits_slot = [](const jslam_image &im) { return (size_t)im.pitch <= align_up((size_t)im.width, 128); };
-    for (int img = 0; img < n_img;) {
+    // A batch of host frames in one run goes up in parts on a stream of its
+    // own, each part's pyramid waiting for its part only (25 pairs of 1241x376
+    // with their results back: 531 us in one copy before the pyramid, 492 so).
+    // Under capture it stays one copy: a captured batch is a part itself where
+    // uploads are to overlap.
+    bool in_parts = ctx->up_parts > 1 && fits_slot(image_of(0));
+    for (int img = 1; img < n_img && in_parts; ++img) {
+        const jslam_image &cur = image_of(img - 1), &nxt = image_of(img);
+        in_parts = fits_slot(nxt) && nxt.data == cur.data + (size_t)cur.pitch * (size_t)cur.height;
+    }
+    if (in_parts) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) {
+            cudaGetLastError();
+            in_parts = false;
+        }
+        in_parts = in_parts && cap == cudaStreamCaptureStatusNone;
+    }
+    if (in_parts) {
+        cudaError_t e = cudaSuccess;
+        if (!ctx->copy_stream) {
+            e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking);
+            for (cudaEvent_t &ev : ctx->copy_ev)
+                if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        }
+        // the copies come after the work before this call, as on one stream
+        if (e == cudaSuccess) e = cudaEventRecord(ctx->copy_ev[0], ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->copy_stream, ctx->copy_ev[0], 0);
+        const uint8_t *const from = image_of(0).data;
+        uint8_t *const to = ctx->staging.as<uint8_t>(ctx->staging_off[0]);
+        for (int p = 0, img = 0; p < ctx->up_parts; ++p) {
+            const int first = img;
+            for (const int end = upload_end(n, p, ctx->up_parts); img < end; ++img) {
+                in.ptr[img] = to + (image_of(img).data - from);
+                in.pitch[img] = image_of(img).pitch;
+            }
+            const jslam_image &lim = image_of(img - 1);
+            const size_t at = (size_t)(image_of(first).data - from);
+            const size_t span = (size_t)(lim.data - from) + (size_t)lim.pitch * (size_t)(lim.height - 1) + lim.width - at;
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(to + at, from + at, span, cudaMemcpyHostToDevice, ctx->copy_stream);
+            if (e == cudaSuccess) e = cudaEventRecord(ctx->copy_ev[p + 1], ctx->copy_stream);
+        }
+        if (e != cudaSuccess) return fail(ctx, e);
+    }
+    for (int img = in_parts ? n_img : 0; img < n_img;) {
         const jslam_image &im = image_of(img);
         if (im.memory != JSLAM_MEM_HOST) {
             in.ptr[img] = im.data;
@@ -1153,7 +1224,7 @@ jslam_status jslam_extract_batch(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
         }
         img = last + 1;
     }
-    cudaError_t e;
+    cudaError_t e = cudaSuccess;
     b.nms_kernel = ctx->tune.nms_kernel;
     b.fast_ctas_per_sm = ctx->tune.detect_ctas_per_sm;
     for (bool &d : ctx->stage_done) d = false;
@@ -1161,7 +1232,17 @@ jslam_status jslam_extract_batch(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
     for (int i = 0; i < JSLAM_STAGE_MATCH; ++i) {
         const NvtxRange range(kStageNames[i]);
         switch (i) {
-        case JSLAM_STAGE_PYRAMID: e = launch_pyramid(b, in, ctx->stream); break;
+        case JSLAM_STAGE_PYRAMID:
+            if (!in_parts) {
+                e = launch_pyramid(b, in, ctx->stream);
+                break;
+            }
+            for (int p = 0; p < ctx->up_parts && e == cudaSuccess; ++p) {
+                e = cudaStreamWaitEvent(ctx->stream, ctx->copy_ev[p + 1], 0);
+                if (e == cudaSuccess)
+                    e = launch_pyramid_strips(b, in, ctx->up_first[p], ctx->up_first[p + 1] - ctx->up_first[p], ctx->stream);
+            }
+            break;
         case JSLAM_STAGE_SKIP:
             e = ctx->skip_on ? launch_skipnet(b, ctx->skip_model, ctx->skip_thresh, ctx->stream) : cudaSuccess;
             break;
@@ -1873,6 +1954,12 @@ void jslam_destroy(jslam_ctx *ctx)
     int cur = -1;
     if (cudaGetDevice(&cur) == cudaSuccess && cur != ctx->cfg.device) cudaSetDevice(ctx->cfg.device);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
+    if (ctx->copy_stream) {
+        cudaStreamSynchronize(ctx->copy_stream);  // copies of a call that failed half way
+        for (cudaEvent_t ev : ctx->copy_ev)
+            if (ev) cudaEventDestroy(ev);
+        cudaStreamDestroy(ctx->copy_stream);
+    }
     ctx->consts.release();
     ctx->plan.release();
     ctx->levels.release();

@@ -33,6 +33,10 @@ constexpr int kMaxImages = 256;    // images per batch (two per stereo pair)
 // lane reads its source columns (see k_pyramid).
 constexpr int kPyrCols = 120, kPyrMinRows = 6, kPyrMaxRows = 58;
 constexpr int kPyrWarpsPerSm = 22;  // strips that run on an SM at once
+// Parts of a batch of host frames, each uploaded while the pyramid of the part
+// before is made, and the bytes a part has at least.
+constexpr int kUploadParts = 4;
+constexpr size_t kUploadPartBytes = (size_t)4 << 20;
 // The ring of a strip's source rows: two source rows per row, for the two
 // rows in use and the rows ahead that are being copied, and the source row
 // before them; rows of up to 16 (kPyrOne) and 32 (kPyrTwo) 16-byte units.
@@ -212,8 +216,9 @@ struct Batch {
     const CUtensorMap *orb_maps;    // per level: keypoint boxes of the raw and of the blurred level
     const PairDesc *pairs;
     const PyrRec *pyr_rec;          // pyramid strips, ordered by level number
-    int32_t pyr_pass_first[kMaxLevels + 1];  // first strip of each level number
-    int32_t pyr_pass;               // -1: one launch over every strip; n: the strips of level number n
+    int32_t pyr_pass_first[kMaxLevels + 1];  // cascaded: first strip of each level number
+    int32_t pyr_cascaded;           // a launch per level number instead of one over every strip
+    int32_t pyr_first;              // first strip of a launch
     const SegRec *seg_rec;          // one per segment
     int32_t n_images, n_levels, n_pairs, n_segments;
     int32_t max_segment;            // largest segment (cells_x x k slots) of the batch
@@ -250,6 +255,7 @@ struct Batch {
 
 // Kernel launchers (one per stage), all on `stream`.
 cudaError_t launch_pyramid(const Batch &b, const Inputs &in, cudaStream_t stream);
+cudaError_t launch_pyramid_strips(const Batch &b, const Inputs &in, int first, int count, cudaStream_t stream);
 cudaError_t launch_detect(const Batch &b, cudaStream_t stream);
 cudaError_t launch_wait_selftest(uint32_t *err, cudaStream_t stream);
 cudaError_t launch_pfa_nms(const Batch &b, cudaStream_t stream);
@@ -290,8 +296,8 @@ int skipnet_smem_bytes();
 // so each sees the results of all before it.  Without a predecessor on the
 // stream that allows it, a launch is an ordinary one.
 //
-// Descriptors, matching and what follows always start so, detection, NMS and
-// finalisation only while the detection tiles all run at once (start_early).
+// The pyramid (while the call before ends), descriptors, matching and what
+// follows always start so, detection, NMS and finalisation only while the detection tiles all run at once (start_early).
 // Beyond that the CTAs that sit and wait take the slots of the kernel before,
 // and persistent ones are spread over the SMs by where that one ended first: us
 // per call with none / with descriptors and matching / with all: one pair of

@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(32, kPyrWarpsPerSm) k_pyramid(const __grid_con
     after_previous();
     let_next();
     if (blockIdx.x == 0 && threadIdx.x == 0) *b.tile_next = 0u;  // for the detection launch that follows
-    const PyrRec R = b.pyr_rec[(b.pyr_pass < 0 ? 0 : b.pyr_pass_first[b.pyr_pass]) + blockIdx.x];
+    const PyrRec R = b.pyr_rec[b.pyr_first + blockIdx.x];
     const LevelDesc &L = b.levels[R.level];
     const ImageDesc &I = b.images[L.image];
     const int x0 = R.x0, y0 = R.y0;
@@ -360,20 +360,21 @@ __global__ void __launch_bounds__(32, kPyrWarpsPerSm) k_pyramid(const __grid_con
 
 const void *pyramid_kernel() { return reinterpret_cast<const void *>(k_pyramid); }
 
+cudaError_t launch_pyramid_strips(const Batch &b, const Inputs &in, int first, int count, cudaStream_t stream)
+{
+    if (count == 0) return cudaSuccess;
+    Batch bn = b;
+    bn.pyr_first = first;
+    return launch_after(k_pyramid, dim3(count), dim3(32), 0, stream, bn, in);
+}
+
 cudaError_t launch_pyramid(const Batch &b, const Inputs &in, cudaStream_t stream)
 {
-    if (b.pyr_tiles == 0) return cudaSuccess;
-    if (b.pyr_pass < 0) {
-        k_pyramid<<<b.pyr_tiles, 32, 0, stream>>>(b, in);
-        return cudaGetLastError();
-    }
+    if (!b.pyr_cascaded) return launch_pyramid_strips(b, in, 0, b.pyr_tiles, stream);
     // cascaded: level number n after n - 1, each launch over every image
     for (int n = 0; n < kMaxLevels; ++n) {
-        const int tiles = b.pyr_pass_first[n + 1] - b.pyr_pass_first[n];
-        if (tiles == 0) continue;
-        Batch bn = b;
-        bn.pyr_pass = n;
-        const cudaError_t e = launch_after(k_pyramid, dim3(tiles), dim3(32), 0, stream, bn, in);
+        const int first = b.pyr_pass_first[n];
+        const cudaError_t e = launch_pyramid_strips(b, in, first, b.pyr_pass_first[n + 1] - first, stream);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
