@@ -364,9 +364,8 @@ BitsBlock bits_block(int W, int H, int c, int k, int border, int max_w, int max_
 // of a 128 x 74 tile).  Detection of 100 pairs of 1241x376: 0.729 ms with the
 // largest blocks of 128 x 64 pixels whose width is a multiple of 4, 0.692 with
 // these.  Heights up to 96 / 64 / 48 / 32 / 24 (us): those 100 pairs 585 / 596 /
-// 680 / 748 / 783 (default 585), 24 pairs of 647x363 with three keypoints a
-// cell 210 / 201 / 201 / 223 / 238 (202), one pair of 320x240 14.2 / 14.2 / 14.2
-// / 13.0 / 12.3 (12.6).
+// 680 / 748 / 783 (default 585), one pair of 320x240 14.2 / 14.2 / 14.2 / 13.0 /
+// 12.3 (12.6).
 void detect_blocks(const std::vector<Geometry> &geo, int k, int border, int tile_w, int tile_h, bool chosen,
                    int n_sm, std::vector<std::array<std::pair<int, int>, kMaxLevels>> &blocks)
 {

@@ -71,8 +71,8 @@ constexpr int kR5 = 5, kR5Side = 2 * kR5 + 1;  // the default window
 // What bounds it: instruction issue, the absolute differences (1331 a
 // keypoint at L = 5).  20 pairs of 1241x376 (40 000 left keypoints), both
 // kernels of the refinement: 86 us with a warp per keypoint and a difference
-// per operation (and the median's digits searched by one thread), 33 now; one pair 27 and
-// 14 us.
+// per operation (and the median's digits searched by one thread), 28 now; one
+// pair 27 and 12 us.
 __global__ void __launch_bounds__(256) k_refine5(const __grid_constant__ Batch b, int L, double bf)
 {
     // per half warp: right strip rows of 8 words, left rows of 4 (as loaded),
