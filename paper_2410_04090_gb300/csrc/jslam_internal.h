@@ -296,8 +296,8 @@ int skipnet_smem_bytes();
 // so each sees the results of all before it.  Without a predecessor on the
 // stream that allows it, a launch is an ordinary one.
 //
-// The pyramid (while the call before ends), descriptors, matching and what
-// follows always start so, detection, NMS and finalisation only while the detection tiles all run at once (start_early).
+// Descriptors, matching and what follows always start so, the pyramid by a rule
+// of its own (launch_pyramid_strips), detection, NMS and finalisation only while the detection tiles all run at once (start_early).
 // Beyond that the CTAs that sit and wait take the slots of the kernel before,
 // and persistent ones are spread over the SMs by where that one ended first: us
 // per call with none / with descriptors and matching / with all: one pair of

@@ -360,12 +360,19 @@ __global__ void __launch_bounds__(32, kPyrWarpsPerSm) k_pyramid(const __grid_con
 
 const void *pyramid_kernel() { return reinterpret_cast<const void *>(k_pyramid); }
 
+// The launch may start while the call before ends where its strips are more
+// than two rounds of those that run at once, and in a cascaded pyramid.  With
+// fewer, the strips that start early are not spread evenly, and the last ones
+// wait for them.  us a call, early or not: 100 pairs of 640x480 230 / 233, 16
+// mixed pairs 363 / 366, 16 of 800x602 cascaded 321 / 324; 12 of 752x480 with
+// the learned skip (1.4 rounds) 218 / 212, 24 of 647x363 240 / 239.
 cudaError_t launch_pyramid_strips(const Batch &b, const Inputs &in, int first, int count, cudaStream_t stream)
 {
     if (count == 0) return cudaSuccess;
     Batch bn = b;
     bn.pyr_first = first;
-    return launch_after(k_pyramid, dim3(count), dim3(32), 0, stream, bn, in);
+    const bool early = b.pyr_cascaded || count > 2 * b.n_sm * kPyrWarpsPerSm;
+    return launch_if(early, k_pyramid, dim3(count), dim3(32), 0, stream, bn, in);
 }
 
 cudaError_t launch_pyramid(const Batch &b, const Inputs &in, cudaStream_t stream)
