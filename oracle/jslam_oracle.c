@@ -829,6 +829,8 @@ static void sp_levels(const uint8_t *L0, int32_t W0, int32_t H0, int32_t pitch0,
         lev[n] = (uint8_t *)malloc((size_t)Wn[n] * (size_t)Hn[n]);
         if (n == 0) {
             for (int32_t y = 0; y < H0; ++y) memcpy(lev[0] + (size_t)y * W0, L0 + (size_t)y * pitch0, (size_t)W0);
+        } else if (p->pyramid_mode == 1) {  /* the cascaded levels, as the keypoints come from */
+            or_pyramid_level(lev[n - 1], Wn[n - 1], Hn[n - 1], Wn[n - 1], p->scale, 1, lev[n], Wn[n], Hn[n], Wn[n]);
         } else {
             or_pyramid_level(L0, W0, H0, pitch0, p->scale, n, lev[n], Wn[n], Hn[n], Wn[n]);
         }
