@@ -294,7 +294,11 @@ int skipnet_smem_bytes();
 // that all its CTAs have started, so that the next one may.  Every kernel of
 // the chain waits before it reads or writes anything that another one touches,
 // so each sees the results of all before it.  Without a predecessor on the
-// stream that allows it, a launch is an ordinary one.
+// stream that allows it, a launch is an ordinary one.  What other kernels (or a
+// user's kernel before the first one) write is read with ordinary loads: a
+// read-only one (__ldg) may be served from before the wait, since its data has
+// to be constant while the kernel is resident.  Tables of the plan and of the
+// context are.
 //
 // Descriptors, matching and what follows always start so, the pyramid by a rule
 // of its own (launch_pyramid_strips), detection, NMS and finalisation only while the detection tiles all run at once (start_early).

@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(kFastThreads, kFastCtasPerSm) k_fast_bits(cons
         // learned skip: the image's proposal skipped at least one cell (an
         // image with none takes the exact path: no per-cell flags, no extra
         // barrier)
-        const bool tskip = kSkip && R.skip != nullptr && __ldg(b.skip_any + R.image) != 0;
+        const bool tskip = kSkip && R.skip != nullptr && b.skip_any[R.image] != 0;
         if (!R.tmap) {
             // levels whose tiles cannot start on a word boundary: plain loads
             // (box rows of box_w bytes, delta = 0)
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(kFastThreads, kFastCtasPerSm) k_fast_bits(cons
                 const int gx = R.xs + 4 * wi;
                 uint32_t v = 0;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) v |= (uint32_t)__ldg(row + min(max(gx + q, 0), W - 1)) << (8 * q);
+                for (int q = 0; q < 4; ++q) v |= (uint32_t)row[min(max(gx + q, 0), W - 1)] << (8 * q);
                 tw32[i] = v;
             }
         }

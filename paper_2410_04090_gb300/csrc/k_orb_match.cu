@@ -310,10 +310,10 @@ __global__ void __launch_bounds__(256, 8) k_match(const __grid_constant__ Batch 
         const int m = m_lo + q;
         ra[q] = rz[q] = 0;
         if (m <= m_hi) {
-            const int s = __ldg(Ir.level_start + m), e = __ldg(Ir.level_start + m + 1);
+            const int s = Ir.level_start[m], e = Ir.level_start[m + 1];
             const int32_t *rf = Ir.row_first + (size_t)m * (Ir.H0 + 1);
-            ra[q] = e > s ? __ldg(rf + va) : s;
-            rz[q] = e > s ? __ldg(rf + vz) : s;
+            ra[q] = e > s ? rf[va] : s;
+            rz[q] = e > s ? rf[vz] : s;
         }
     }
     // the three bands as one run of candidates over the lanes (a band of a
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(256) k_track(const __grid_constant__ Batch b, 
         const float r = __fmul_rn(a.radius, a.zeta_f[lv]);
         uint32_t dq[8];
 #pragma unroll
-        for (int w = 0; w < 8; ++w) dq[w] = __ldg(a.desc + (size_t)q * 8 + w);
+        for (int w = 0; w < 8; ++w) dq[w] = a.desc[(size_t)q * 8 + w];
         const KpOut &o = I.out;
         const int m_lo = max(0, lv - 1), m_hi = min(I.levels - 1, lv + 1);
         const int ylo = (int)floorf(v - r) - 1, yhi = (int)ceilf(v + r) + 1;  // covers every Y that can pass
@@ -384,8 +384,8 @@ __global__ void __launch_bounds__(256) k_track(const __grid_constant__ Batch b, 
         for (int m = m_lo; m <= m_hi; ++m) {
             const int s = I.level_start[m], e = I.level_start[m + 1];
             const int32_t *rf = I.row_first + (size_t)m * (I.H0 + 1);
-            const int z0 = e > s ? __ldg(rf + va) : s;
-            const int z1 = e > s ? max(__ldg(rf + vz), z0) : s;
+            const int z0 = e > s ? rf[va] : s;
+            const int z1 = e > s ? max(rf[vz], z0) : s;
             for (int j = z0 + lane; j < z1; j += 32) {
                 const float dx = __fsub_rn((float)o.X[j], u), dy = __fsub_rn((float)o.Y[j], v);
                 if (fabsf(dx) > r || fabsf(dy) > r) continue;

@@ -132,7 +132,7 @@ template <int MODE> struct PyrTaps {
         if constexpr (MODE == kPyrBytes) {
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                h[k] = (wgt[k] & 0xFFFFu) * __ldg(row + off[2 * k]) + (wgt[k] >> 16) * __ldg(row + off[2 * k + 1]);
+                h[k] = (wgt[k] & 0xFFFFu) * row[off[2 * k]] + (wgt[k] >> 16) * row[off[2 * k + 1]];
         } else {
             uint32_t a[kWin], z[kWin];
 #pragma unroll

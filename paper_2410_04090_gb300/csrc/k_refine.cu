@@ -71,7 +71,7 @@ constexpr int kR5 = 5, kR5Side = 2 * kR5 + 1;  // the default window
 // What bounds it: instruction issue, the absolute differences (1331 a
 // keypoint at L = 5).  20 pairs of 1241x376 (40 000 left keypoints), both
 // kernels of the refinement: 86 us with a warp per keypoint and a difference
-// per operation (and the median's digits searched by one thread), 28 now; one
+// per operation (and the median's digits searched by one thread), 27 now; one
 // pair 27 and 12 us.
 __global__ void __launch_bounds__(256) k_refine5(const __grid_constant__ Batch b, int L, double bf)
 {
@@ -109,15 +109,29 @@ __global__ void __launch_bounds__(256) k_refine5(const __grid_constant__ Batch b
         if (in) {
             const uint32_t *lsrc = reinterpret_cast<const uint32_t *>(A.raw + (size_t)y0 * pitch) + (xl >> 2);
             const uint32_t *rsrc = reinterpret_cast<const uint32_t *>(B.raw + (size_t)y0 * pitch) + (xr >> 2);
+            // all loads before the stores, which may write to what is loaded for
+            // all the compiler knows (the call below 32.3 us with a store after
+            // each load, 26.8 so)
+            uint32_t rw[6], lw[3];
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
                 const int r = 2 * k + (l16 >> 3);
-                if (r < kR5Side) s_right[hw][r][l16 & 7] = __ldg(rsrc + (size_t)r * (pitch >> 2) + (l16 & 7));
+                rw[k] = r < kR5Side ? rsrc[(size_t)r * (pitch >> 2) + (l16 & 7)] : 0u;
             }
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const int r = 4 * k + (l16 >> 2);
-                if (r < kR5Side) s_left[hw][r][l16 & 3] = __ldg(lsrc + (size_t)r * (pitch >> 2) + (l16 & 3));
+                lw[k] = r < kR5Side ? lsrc[(size_t)r * (pitch >> 2) + (l16 & 3)] : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const int r = 2 * k + (l16 >> 3);
+                if (r < kR5Side) s_right[hw][r][l16 & 7] = rw[k];
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int r = 4 * k + (l16 >> 2);
+                if (r < kR5Side) s_left[hw][r][l16 & 3] = lw[k];
             }
         }
         __syncwarp();
