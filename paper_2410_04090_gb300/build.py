@@ -18,7 +18,7 @@ LIB = os.path.join(HERE, "libjslam.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 CUDA_SOURCES = ["k_pyramid.cu", "k_detect.cu", "k_pyca.cu", "k_orb_match.cu", "k_refine.cu", "k_fc_ablation.cu", "k_skipnet.cu", "jslam_api.cu", "pfa_static.cu"]
-HOST_SOURCES = ["tables.cpp", "tune_cache.cpp"]
+HOST_SOURCES = ["tables.cpp", "tile_plan.cpp", "tune_cache.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

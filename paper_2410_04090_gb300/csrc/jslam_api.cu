@@ -14,6 +14,7 @@
 #include "jslam.h"
 #include "jslam_internal.h"
 #include "tables.h"
+#include "tile_plan.h"
 
 namespace jslam {
 int fast_smem_bytes(int max_box, int max_cells, int k, int max_planes);
@@ -56,16 +57,6 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
         cudaGetLastError();
     }
     return fn;
-}
-
-// Detection tile box of a level: rows of box_w bytes -- the tile's 32-byte
-// chunks and one more, which covers its 4-pixel halo on both sides and up to
-// 15 bytes of alignment slack on the left -- and box_h rows (3-row halo above
-// and below).
-void detect_box(int tw, int th, int *box_w, int *box_h)
-{
-    *box_w = 32 * ((tw + 31) / 32 + 1);
-    *box_h = th + 6;
 }
 
 constexpr size_t kLevelSlack = 256;  // bytes after each level buffer
@@ -300,110 +291,6 @@ jslam_status check_job(const jslam_ctx *ctx, const jslam_stereo_job &j)
     return JSLAM_OK;
 }
 
-// Shared memory of a detection tile's two boxes and planes.
-int bits_tile_bytes(int tw, int th)
-{
-    int bw, bh;
-    detect_box(tw, th, &bw, &bh);
-    return bh * (2 * bw + 16 * bs_row_units((tw + 31) / 32));
-}
-
-// Issue slots of a detection tile with `rows` evaluated rows of
-// nch 32-pixel chunks: measured on the 1241x376 sequence, about 1000 a warp's
-// round of ring tests and responses, 115 a round of transposed chunks, 300 a
-// tile.
-double bits_tile_cost(int rows, int nch)
-{
-    const int rounds = (rows * nch + kFastThreads - 1) / kFastThreads;
-    const int chunks = rows ? ((rows + 6) * (nch + 1) + kFastThreads - 1) / kFastThreads : 0;
-    return 1000.0 * rounds + 115.0 * chunks + 300.0;
-}
-
-struct BitsBlock {
-    int bx, by;
-    double cost, tile;  // of the level's tiles, of its dearest one
-};
-
-// Cells per detection tile of a level.  A tile's evaluated
-// rows x 32-pixel chunks are items, a lane each, so cells whose size divides
-// neither 32 nor the CTA leave lanes and warps idle: with about 128 x 64
-// pixels, 22-pixel cells made 132 items for 128 threads.  Of the blocks at
-// most max_w x max_h pixels (one cell at least) whose two boxes and planes
-// take at most `budget` bytes of shared memory, the one whose tiles over the
-// level cost least.
-BitsBlock bits_block(int W, int H, int c, int k, int border, int max_w, int max_h, int budget)
-{
-    const int cells_x = (W + c - 1) / c, cells_y = (H + c - 1) / c;
-    BitsBlock best{ 1, 1, -1.0, 0.0 };
-    for (int x = 1; x <= cells_x && (x == 1 || x * c <= max_w); ++x)
-        for (int y = 1; y <= cells_y && (y == 1 || y * c <= max_h); ++y) {
-            if (x * y > 1 && (x * y * k > kFastMaxCellsPerCta ||
-                              bits_tile_bytes(std::min(x * c, W), std::min(y * c, H)) > budget))
-                break;
-            double cost = 0.0, tile = 0.0;
-            for (int ty = 0; ty < cells_y; ty += y) {
-                const int y0 = ty * c, th = std::min(y * c, H - y0);
-                const int rows = std::max(std::min(H - border - y0, th) - std::max(border - y0, 0), 0);
-                for (int tx = 0; tx < cells_x; tx += x) {
-                    const double one = bits_tile_cost(rows, (std::min(x * c, W - tx * c) + 31) / 32);
-                    cost += one;
-                    tile = std::max(tile, one);
-                }
-            }
-            if (best.cost < 0.0 || cost < best.cost) best = { x, y, cost, tile };
-        }
-    return best;
-}
-
-// Detection tiles of every level of a batch (pairs of one shape share them).
-// A chosen tile size is about what the tiles get (up to half as tall again
-// where that fits).  By default the tallest tiles whose launch takes least
-// time: large tiles waste less on their halo, but a launch of few tiles ends
-// with most CTAs idle, so the estimate adds the dearest tile to the tiles'
-// cost shared out over the CTAs that run at once (five an SM fit the budget
-// of a 128 x 74 tile).  Detection of 100 pairs of 1241x376: 0.729 ms with the
-// largest blocks of 128 x 64 pixels whose width is a multiple of 4, 0.692 with
-// these.  Heights up to 96 / 64 / 48 / 32 / 24 (us): those 100 pairs 585 / 596 /
-// 680 / 748 / 783 (default 585), one pair of 320x240 14.2 / 14.2 / 14.2 / 13.0 /
-// 12.3 (12.6).
-void detect_blocks(const std::vector<Geometry> &geo, int k, int border, int tile_w, int tile_h, bool chosen,
-                   int n_sm, std::vector<std::array<std::pair<int, int>, kMaxLevels>> &blocks)
-{
-    const int n = (int)geo.size();
-    blocks.resize(n);
-    auto same = [&](int p, int q) {
-        bool eq = geo[p].levels == geo[q].levels;
-        for (int l = 0; eq && l < geo[p].levels; ++l)
-            eq = geo[p].W[l] == geo[q].W[l] && geo[p].H[l] == geo[q].H[l] && geo[p].c[l] == geo[q].c[l];
-        return eq;
-    };
-    static const int heights[] = { 96, 64, 48, 32, 24, 16 };
-    std::vector<std::array<std::pair<int, int>, kMaxLevels>> cand(n);
-    double best = -1.0;
-    for (int h : heights) {
-        const int max_h = chosen ? std::min(tile_h * 3 / 2, kFastMaxTile) : h;
-        const int budget = bits_tile_bytes(tile_w, tile_h * 23 / 20);
-        double sum = 0.0, tile = 0.0, of_pair = 0.0;
-        for (int p = 0; p < n; ++p) {
-            if (p > 0 && same(p, p - 1)) {
-                cand[p] = cand[p - 1];
-            } else {
-                of_pair = 0.0;
-                for (int l = 0; l < geo[p].levels; ++l) {
-                    const BitsBlock B = bits_block(geo[p].W[l], geo[p].H[l], geo[p].c[l], k, border, tile_w, max_h, budget);
-                    cand[p][l] = { B.bx, B.by };
-                    of_pair += 2.0 * B.cost;
-                    tile = std::max(tile, B.tile);
-                }
-            }
-            sum += of_pair;
-        }
-        const double time = sum / ((double)kFastCtasPerSm * n_sm) + tile;
-        if (best < 0.0 || time < best) { best = time; blocks = cand; }
-        if (chosen) break;
-    }
-}
-
 // Pyramid strips of a level.
 int pyramid_strips(int W, int H, int rows) { return ((W + kPyrCols - 1) / kPyrCols) * ((H + rows - 1) / rows); }
 
@@ -478,7 +365,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     const int n_img = 2 * n;
     const int k = cfg.k_per_cell;
     std::vector<Geometry> geo(n);
-    std::vector<std::array<std::pair<int, int>, kMaxLevels>> blocks;  // cells per detection tile of each level
+    std::vector<LevelBlocks> blocks;  // cells per detection tile of each level
     std::vector<PairLayout> layouts(n);
     std::vector<size_t> result_off(n);
     size_t result_bytes = 0, level_bytes = 0, map_bytes = 0, staging_bytes = 0, table_bytes = 0;

@@ -16,9 +16,10 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "tile_plan.h"
+
 namespace jslam {
 
-constexpr int kMaxLevels = 8;
 constexpr int kBins = 30;        // orientation sectors of 12 degrees
 constexpr int kPairs = 256;      // BRIEF point pairs
 constexpr int kDiskR = 15;       // intensity-centroid disk radius
@@ -45,15 +46,6 @@ constexpr int kPyrMaxOne = 256, kPyrMaxTwo = 512;
 static_assert((2 * (kPyrAhead + 2) + 1) * kPyrMaxOne <= kPyrRing, "ring");
 static_assert((2 * (kPyrAheadTwo + 2) + 1) * kPyrMaxTwo <= kPyrRing, "ring");
 enum { kPyrCopy = 0, kPyrOne = 1, kPyrTwo = 2, kPyrBytes = 3 };
-// Detection tile: at most this many pixels a side (host picks cells per CTA).
-constexpr int kFastMaxTile = 128, kFastThreads = 128, kFastCtasPerSm = 5;
-
-// Row stride of the bit-planes in 16-byte units for a tile of nch 32-pixel
-// chunks: chunks 0..nch (32 bytes each) and a 16-byte pad, an odd count, so
-// that the 128-bit loads of two neighbouring rows fall on the two halves of
-// the shared-memory banks.
-__host__ __device__ inline int bs_row_units(int nch) { return 2 * (nch + 1) + 1; }
-constexpr int kFastMaxCellsPerCta = 2048;  // cells x k per CTA
 constexpr int kLutWords = 2048;            // 2^16-entry corner bit table
 constexpr int kSkipC = 16;                 // channels of the learned cell-skip net
 constexpr int kSkipTileW = 26, kSkipTileH = 12;  // its logits per CTA (grid pitch 26 + 6 = 32)
