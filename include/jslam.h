@@ -388,10 +388,12 @@ jslam_status jslam_stage_times(jslam_ctx *ctx, float *ms /* JSLAM_NUM_STAGES ent
 
 /* Launch-shape tuning.  None of these changes a result: detection tiles hold
  * whole culling cells, and every kernel variant computes the same outputs.
- * Until a tuning is set (or tuned), tile heights and order follow the batch. */
+ * The default tile, 128 x 64, stands for tile heights that follow the batch
+ * and tiles in order of decreasing work, whatever tile_order says; setting the
+ * defaults is the same as setting nothing, and the way back from a tuning. */
 typedef struct {
     int32_t tile_w_px;           /* detection tile width, at most: 32..128, multiple of 4 (default 128) */
-    int32_t tile_h_px;           /* detection tile height, about: 8..128 (default 64) */
+    int32_t tile_h_px;           /* detection tile height, about (up to half as much again): 8..128 (default 64) */
     int32_t nms_kernel;          /* PFA NMS: 0 one warp per segment when every segment of the batch has at most
                                   * 96 candidate slots, else one CTA per segment (default); 1 one CTA per
                                   * segment always */
@@ -399,7 +401,8 @@ typedef struct {
                                   * that many (never more than fit) */
     int32_t tile_order;          /* order in which the persistent detection CTAs take the tiles: 0 by image,
                                   * level and tile row (default); 1 by decreasing work (evaluated rows x
-                                  * 32-pixel chunks), so the last rounds hold the smallest tiles */
+                                  * 32-pixel chunks), so the last rounds hold the smallest tiles; with the
+                                  * default tile both go by decreasing work */
 } jslam_tuning;
 
 /* Use `t` for the following extractions (plans are rebuilt when the tile
@@ -410,10 +413,12 @@ jslam_status jslam_set_tuning(jslam_ctx *ctx, const jslam_tuning *t);
 
 /* Tune the launch shapes on the batch `jobs` (n pairs, as for
  * jslam_extract_batch), timing the stages with the stage events: the
- * detection tile among five shapes, then the number of persistent detection
- * CTAs per SM, then (when every segment fits a warp) the NMS kernel, then the
- * tile order.  Keeps
- * the fastest for the context and returns it in *out (may be NULL).  Runs the
+ * detection tile among six shapes, the default first, then the number of
+ * persistent detection CTAs per SM, then (when every segment fits a warp) the
+ * NMS kernel, then the tile order of a tile that is not the default, then the
+ * pick for detection against the default once more.  Keeps
+ * the fastest for the context and returns it in *out (may be NULL); a call
+ * that fails leaves tuning and stage timing as they were.  Runs the
  * batch several times; results are unaffected.  No counterpart in the paper
  * (an autotuner in place of the fixed thread allocation of Sec. II-C-1). */
 jslam_status jslam_autotune(jslam_ctx *ctx, const jslam_stereo_job *jobs, int32_t n, jslam_tuning *out);

@@ -230,9 +230,7 @@ struct jslam_ctx {
     bool plan_skip = false;  // the current plan has skip buffers
 
     // launch-shape tuning and the captured graph
-    jslam_tuning tune{128, 64, 0, 0, 0};
-    bool tune_chosen = false;               // by jslam_set_tuning or the autotuner
-    bool plan_chosen = false;
+    jslam_tuning tune{ kDefaultTileW, kDefaultTileH, 0, 0, 0 };
     jslam_tuning plan_tune{0, 0, 0, 0, 0};  // tuning the current plan was built with (tile fields)
     cudaGraphExec_t graph = nullptr;
     cudaGraph_t graph_src = nullptr;    // the captured graph (its node handles address `graph`)
@@ -358,7 +356,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     }
     if (keys == ctx->keys && ctx->plan_tune.tile_w_px == ctx->tune.tile_w_px &&
         ctx->plan_tune.tile_h_px == ctx->tune.tile_h_px && ctx->plan_tune.tile_order == ctx->tune.tile_order &&
-        ctx->plan_chosen == ctx->tune_chosen && ctx->plan_skip == ctx->skip_on)
+        ctx->plan_skip == ctx->skip_on)
         return JSLAM_OK;
     ++ctx->plan_gen;
 
@@ -374,7 +372,8 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     for (int p = 0; p < n; ++p) {
         geo[p] = level_geometry(jobs[p].left.width, jobs[p].left.height, jobs[p].levels, jobs[p].scale, jobs[p].cell);
     }
-    detect_blocks(geo, k, cfg.border, ctx->tune.tile_w_px, ctx->tune.tile_h_px, ctx->tune_chosen, ctx->n_sm, blocks);
+    const bool chosen = !default_tile(ctx->tune.tile_w_px, ctx->tune.tile_h_px);
+    detect_blocks(geo, k, cfg.border, ctx->tune.tile_w_px, ctx->tune.tile_h_px, chosen, ctx->n_sm, blocks);
     for (int p = 0; p < n; ++p) {
         layouts[p] = pair_layout(jobs[p].max_feats);
         result_off[p] = result_bytes;
@@ -691,10 +690,10 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     // ordered by decreasing work (evaluated rows x 32-pixel chunks, the items
     // of a threshold pass) the last ones are the smallest tiles.  Each record
     // is self-contained (its tile's geometry, slots and buffers), so the order
-    // changes no result.  Used by default too (100 pairs of 1241x376: detection
-    // 0.597 -> 0.585 ms, 12 of 752x480 with the learned skip 101 -> 95 us, one
-    // of 1920x1080 45 -> 42 us); with a chosen tuning its own order.
-    if (ctx->tune.tile_order == 1 || !ctx->tune_chosen) {
+    // changes no result.  The default tile goes so whatever the order (100 pairs
+    // of 1241x376: detection 0.597 -> 0.585 ms, 12 of 752x480 with the learned
+    // skip 101 -> 95 us, one of 1920x1080 45 -> 42 us).
+    if (ctx->tune.tile_order == 1 || !chosen) {
         std::vector<std::pair<int, int>> work(fast);
         for (int t = 0; t < fast; ++t) {
             const TileRec &R = trec[t];
@@ -795,7 +794,6 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
 
     ctx->keys = keys;
     ctx->plan_tune = ctx->tune;
-    ctx->plan_chosen = ctx->tune_chosen;
     ctx->plan_skip = ctx->skip_on;
     ctx->layouts = layouts;
     ctx->result_off = result_off;
@@ -1606,7 +1604,6 @@ jslam_status jslam_set_tuning(jslam_ctx *ctx, const jslam_tuning *t)
         return JSLAM_ERR_ARG;
     if (t->tile_order < 0 || t->tile_order > 1) return JSLAM_ERR_ARG;
     ctx->tune = *t;
-    ctx->tune_chosen = true;
     return JSLAM_OK;
 }
 
@@ -1634,18 +1631,14 @@ jslam_status jslam_autotune(jslam_ctx *ctx, const jslam_stereo_job *jobs, int32_
 {
     if (!ctx || !jobs) return JSLAM_ERR_ARG;
     if (ctx->status != JSLAM_OK) return ctx->status;
-    static const int tiles[][2] = { { 128, 64 }, { 128, 32 }, { 128, 128 }, { 64, 64 }, { 64, 128 } };
     const bool was_timing = ctx->timing;
+    const jslam_tuning before = ctx->tune;
     jslam_status st = jslam_enable_stage_timing(ctx, 1);
     if (st != JSLAM_OK) return st;
-    ctx->tune_chosen = true;
-    jslam_tuning best = ctx->tune;
-    best.nms_kernel = 0;
-    best.detect_ctas_per_sm = 0;
-    best.tile_order = 0;
+    jslam_tuning best{};
     // 1. the detection tile
     float best_ms = -1.0f;
-    for (const auto &tl : tiles) {
+    for (const auto &tl : kTuneTiles) {
         ctx->tune = best;
         ctx->tune.tile_w_px = tl[0];
         ctx->tune.tile_h_px = tl[1];
@@ -1685,8 +1678,8 @@ jslam_status jslam_autotune(jslam_ctx *ctx, const jslam_stereo_job *jobs, int32_
         if (st == JSLAM_OK) best.nms_kernel = nms_ms[1] < nms_ms[0] ? 1 : 0;
     }
     // 4. the tile order (a replan each), against the detection time of the
-    // pick so far
-    if (st == JSLAM_OK) {
+    // pick so far; the default tile has its own
+    if (st == JSLAM_OK && !default_tile(best.tile_w_px, best.tile_h_px)) {
         ctx->tune = best;
         ctx->tune.tile_order = 1;
         float ms;
@@ -1695,11 +1688,34 @@ jslam_status jslam_autotune(jslam_ctx *ctx, const jslam_stereo_job *jobs, int32_
             best.tile_order = 1;
         }
     }
-    ctx->tune = best;
+    // 5. the pick against the default once more, over more runs: the events
+    // resolve about 2 us, as much as the tiles of one small pair differ by
+    if (st == JSLAM_OK && (!default_tile(best.tile_w_px, best.tile_h_px) || best.detect_ctas_per_sm != 0)) {
+        float ms[2] = { -1.0f, -1.0f };
+        for (int v = 0; v < 2 && st == JSLAM_OK; ++v) {
+            ctx->tune = best;
+            if (v == 0) {
+                ctx->tune.tile_w_px = kDefaultTileW;
+                ctx->tune.tile_h_px = kDefaultTileH;
+                ctx->tune.detect_ctas_per_sm = ctx->tune.tile_order = 0;
+            }
+            st = time_stage(ctx, jobs, n, JSLAM_STAGE_DETECT, 12, &ms[v]);
+        }
+        best_ms = std::min(ms[0], ms[1]);
+        if (st == JSLAM_OK && ms[1] >= ms[0]) {
+            best.tile_w_px = kDefaultTileW;
+            best.tile_h_px = kDefaultTileH;
+            best.detect_ctas_per_sm = best.tile_order = 0;
+        }
+    }
+    // a failed tuning leaves the context as it was
+    ctx->tune = st == JSLAM_OK ? best : before;
+    ctx->timing = was_timing;
+    for (bool &d : ctx->stage_done) d = false;
+    if (st != JSLAM_OK) return st;
     ctx->tune_ms = best_ms;
-    if (st == JSLAM_OK) st = jslam_enable_stage_timing(ctx, was_timing ? 1 : 0);
-    if (st == JSLAM_OK && out) *out = best;
-    return st;
+    if (out) *out = best;
+    return JSLAM_OK;
 }
 
 jslam_status jslam_autotune_cached(jslam_ctx *ctx, const jslam_stereo_job *jobs, int32_t n, const char *cache_path,

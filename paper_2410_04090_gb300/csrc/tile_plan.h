@@ -21,6 +21,15 @@ constexpr int kMaxLevels = 8;
 constexpr int kFastMaxTile = 128, kFastThreads = 128, kFastCtasPerSm = 5;
 constexpr int kFastMaxCellsPerCta = 2048;  // cells x k per CTA
 
+// The default tile of a tuning stands for what an untuned context does: tile
+// heights that follow the batch, and the tiles in order of decreasing work.
+constexpr int kDefaultTileW = 128, kDefaultTileH = 64;
+constexpr bool default_tile(int w, int h) { return w == kDefaultTileW && h == kDefaultTileH; }
+// Tiles the autotuner times, the default first; 128 x 65 gives every batch the
+// tall tiles that the default gives large ones.
+constexpr int kTuneTiles[][2] = { { kDefaultTileW, kDefaultTileH }, { 128, 65 }, { 128, 32 },
+                                  { 128, 128 }, { 64, 64 }, { 64, 128 } };
+
 // Row stride of the bit-planes in 16-byte units for a tile of nch 32-pixel
 // chunks: chunks 0..nch (32 bytes each) and a 16-byte pad, an odd count, so
 // that the 128-bit loads of two neighbouring rows fall on the two halves of

@@ -1,0 +1,111 @@
+"""The default tuning: setting it is setting nothing, a failed tuning leaves it,
+and the autotuner times it before anything else."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from conftest import ROOT
+from paper_2410_04090_gb300 import scenes
+from parity_util import frontend_for, params_from
+
+CSRC = os.path.join(ROOT, "paper_2410_04090_gb300", "csrc")
+DRIVER = r"""
+#include "tile_plan.h"
+extern "C" int tune_tiles(int *out)
+{
+    int n = 0;
+    for (const auto &t : jslam::kTuneTiles) { out[n++] = t[0]; out[n++] = t[1]; }
+    return n / 2;
+}
+extern "C" int is_default(int w, int h) { return jslam::default_tile(w, h); }
+"""
+
+
+def test_the_tuner_starts_from_the_default(tmp_path):
+    (tmp_path / "driver.cpp").write_text(DRIVER)
+    so = str(tmp_path / "driver.so")
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(tmp_path / "driver.cpp"), "-o", so], check=True)
+    lib = C.CDLL(so)
+    out = (C.c_int * 64)()
+    tiles = [(out[2 * i], out[2 * i + 1]) for i in range(lib.tune_tiles(out))]
+    assert tiles[0] == (128, 64) and lib.is_default(128, 64)
+    assert not any(lib.is_default(*t) for t in tiles[1:]) and len(set(tiles)) == len(tiles)
+    for w, h in tiles:  # each is a tuning the library accepts
+        assert 32 <= w <= 128 and w % 4 == 0 and 8 <= h <= 128
+
+
+def _captured(J, oracle, pairs=1):
+    """A context with a captured graph: a replay is refused once its plan changes."""
+    import torch
+    p = params_from(oracle, levels=4, max_feats=400, fast_thresh_lo=7)
+    f = scenes.planes_pair(320, 240, 0, 3, 4)
+    img = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (f.left, f.right)]
+    torch.cuda.synchronize()
+    fe = frontend_for(J, p, max_width=320, max_height=240, max_pairs=pairs, stream=torch.cuda.Stream())
+    jobs = [J.Job(*img, levels=p.levels, max_feats=p.max_feats)] * pairs
+    fe.graph_capture(jobs)
+    return fe, jobs
+
+
+@pytest.mark.gpu
+def test_setting_the_defaults_is_setting_nothing(J, oracle):
+    fe, jobs = _captured(J, oracle)
+    fe.set_tuning(128, 64, 0, 0, 0)
+    fe.extract_batch(jobs)
+    fe.graph_launch()  # the plan is still the captured one
+    fe.sync()
+    fe.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("bad", ["batch too large", "image too large"])
+def test_a_failed_tuning_changes_nothing(J, oracle, bad):
+    import torch
+    fe, jobs = _captured(J, oracle)
+    if bad == "batch too large":
+        wrong = jobs * 2
+    else:
+        img = torch.zeros((480, 640), dtype=torch.uint8, device="cuda")
+        wrong = [J.Job(img, img, levels=4, max_feats=400)]
+    with pytest.raises(J.JslamError):
+        fe.autotune(wrong)
+    fe.extract_batch(jobs)
+    fe.graph_launch()
+    fe.sync()
+    with pytest.raises(J.JslamError) as e:  # stage timing is off, as before
+        fe.stage_times()
+    assert e.value.status == J.ERR_STATE
+    fe.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("width,height,levels", [(320, 240, 4), (640, 480, 8), (752, 480, 8), (1241, 376, 8)])
+def test_a_tuned_batch_is_not_slower(J, oracle, width, height, levels):
+    """Detection of the tuner's pick within the events' resolution (about 2 us
+    here) of the default's."""
+    import torch
+    p = params_from(oracle, levels=levels, max_feats=800, fast_thresh_lo=7)
+    f = scenes.planes_pair(width, height, 0, 3, 4)
+    img = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (f.left, f.right)]
+    torch.cuda.synchronize()
+    fe = frontend_for(J, p, max_width=width, max_height=height, max_pairs=1)
+    jobs = [J.Job(*img, levels=levels, max_feats=800)]
+
+    def detect_us():
+        fe.enable_stage_timing(True)
+        t = []
+        for _ in range(60):
+            fe.extract_batch(jobs)
+            fe.sync()
+            t.append(1e3 * fe.stage_times()["detect"])
+        fe.enable_stage_timing(False)
+        return float(np.median(t))
+
+    before = detect_us()
+    pick = fe.autotune(jobs)
+    tuned = detect_us()
+    assert tuned <= before + 2.5, (pick, before, tuned)
+    fe.close()
