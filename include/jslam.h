@@ -435,7 +435,8 @@ jslam_status jslam_autotune_cached(jslam_ctx *ctx, const jslam_stereo_job *jobs,
                                    jslam_tuning *out, int32_t *hit);
 
 /* Key of a batch in the tuning cache (host only, no device work): GPU name
- * and SM count, the configuration fields that shape the kernels' work
+ * and SM count, the revision of the library's launch shapes (picks stored for
+ * another one are not found), the configuration fields that shape the kernels' work
  * (P_min, P_max, k, q, border, rule, fallback threshold) and every pair's
  * size, depth, scale bits, threshold, cell, cap and memory kinds, written to
  * buf (len bytes) as a NUL-terminated string.  JSLAM_ERR_CAPACITY when it

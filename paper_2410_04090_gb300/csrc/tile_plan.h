@@ -46,6 +46,12 @@ inline void detect_box(int tw, int th, int *box_w, int *box_h)
     *box_h = th + 6;
 }
 
+// Part of the keys of the tuning cache: raised whenever the detection kernel's
+// CTAs or what a tuning's values mean change, so that picks made for others are
+// not applied (1: eight warps a CTA and exact tiles; 2: four warps, tiles by
+// cost; 3: the default tile stands for the untuned plan).
+constexpr int kTuneRevision = 3;
+
 // Cells per tile, horizontally and vertically, of each level of a pair.
 using LevelBlocks = std::array<std::pair<int, int>, kMaxLevels>;
 

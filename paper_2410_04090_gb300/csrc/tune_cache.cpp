@@ -14,7 +14,8 @@
 //       ...
 //     }
 //   }
-// Keys hold no quote or backslash (the key builder replaces them), so the
+// Keys hold the revision of the launch shapes, so picks of another one are not
+// found.  They hold no quote or backslash (the key builder replaces them), so the
 // parser needs no escapes.  A file that does not parse is treated as empty;
 // writes go to a temporary file renamed over the old one, so readers never
 // see a half-written file (two writers at once: the last rename wins).
@@ -28,6 +29,7 @@
 #include <unistd.h>
 
 #include "jslam.h"
+#include "tile_plan.h"
 
 namespace {
 
@@ -174,8 +176,9 @@ jslam_status jslam_tune_key(const char *gpu_name, int32_t sm_count, const jslam_
     std::string k = "gpu=";
     for (const char *c = gpu_name; *c; ++c) k += (*c == '"' || *c == '\\' || (unsigned char)*c < 32) ? '_' : *c;
     char tmp[256];
-    std::snprintf(tmp, sizeof tmp, "|sm=%d|p=%d,%d|k=%d|q=%d|b=%d|rule=%d|lo=%d", sm_count, cfg->p_min, cfg->p_max,
-                  cfg->k_per_cell, cfg->nms_q, cfg->border, cfg->pfa_rule, cfg->fast_thresh_lo);
+    std::snprintf(tmp, sizeof tmp, "|sm=%d|rev=%d|p=%d,%d|k=%d|q=%d|b=%d|rule=%d|lo=%d", sm_count,
+                  jslam::kTuneRevision, cfg->p_min, cfg->p_max, cfg->k_per_cell, cfg->nms_q, cfg->border, cfg->pfa_rule,
+                  cfg->fast_thresh_lo);
     k += tmp;
     k += "|jobs=";
     for (int p = 0; p < n; ++p) {
