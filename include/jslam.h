@@ -60,14 +60,23 @@ enum { JSLAM_MEM_DEVICE = 0, JSLAM_MEM_HOST = 1 };
  * (pitch >= width, and pitch x height below 4 GiB: the kernels address an
  * image with 32-bit offsets; larger spans are refused with JSLAM_ERR_ARG).
  * memory == JSLAM_MEM_DEVICE: `data` is device memory of the context's
- *   device and is read in place.
+ *   device and is read in place, in aligned units of 16 bytes: bytes in the
+ *   16-byte units that hold a row's first and last pixels are read too (and
+ *   ignored), never a unit without a pixel.
  * memory == JSLAM_MEM_HOST: `data` is host memory (pinned memory makes the
  *   copy asynchronous); the library copies it into its own device staging
- *   buffer on the context stream.  Host images of one call that lie back to
- *   back in host memory (image k + 1 starting at data_k + pitch_k x
- *   height_k, in the order left 0, right 0, left 1, ...) with pitch <= width
- *   rounded up to 128 are copied with a single transfer; keeping a step's
- *   frames in one pinned buffer therefore makes the upload one copy. */
+ *   buffer, after the work enqueued on the context stream before the call.
+ *   Host images of one call that lie back to back in host memory (image k + 1
+ *   starting at data_k + pitch_k x height_k, in the order left 0, right 0,
+ *   left 1, ...) with pitch <= width rounded up to 128 are copied with a
+ *   single transfer on the context stream; keeping a step's frames in one
+ *   pinned buffer therefore makes the upload one copy.  If all images of the
+ *   call are host images that lie so, of 8 MB or more together, they go up in
+ *   two to four transfers on a stream of the context's own, each beside the
+ *   pyramid of the ones before; the context stream waits for every transfer,
+ *   so work enqueued on it later, and jslam_sync(), come after the upload
+ *   all the same.  Under stream capture, with stage timing on and with the
+ *   cascaded pyramid the upload is one transfer. */
 typedef struct {
     int32_t width, height, pitch;
     int32_t memory;
@@ -376,13 +385,15 @@ enum {
 
 /* Turn per-stage timing on or off.  When on, every extraction and match
  * records a CUDA event on the context stream after each stage (a small
- * overhead per stage).  Per-stage times as the paper reports them for CRF,
+ * overhead per stage; no stage starts beside another, and host images go up
+ * before the first).  Per-stage times as the paper reports them for CRF,
  * FC and PFA (Sec. IV-B, IV-C). */
 jslam_status jslam_enable_stage_timing(jslam_ctx *ctx, int32_t enable);
 
 /* Device durations in milliseconds of each stage of the last extraction
  * (and match, if one followed it), measured between the recorded events
- * (the stage timings of Sec. IV-B, IV-C).  Valid after jslam_sync();
+ * (the stage timings of Sec. IV-B, IV-C); the upload of host images comes
+ * before the first of them.  Valid after jslam_sync();
  * JSLAM_ERR_STATE if timing was off. */
 jslam_status jslam_stage_times(jslam_ctx *ctx, float *ms /* JSLAM_NUM_STAGES entries */);
 

@@ -1029,8 +1029,9 @@ jslam_status jslam_extract_batch(jslam_ctx *ctx, const jslam_stereo_job *jobs, i
     // own, each part's pyramid waiting for its part only (25 pairs of 1241x376
     // with their results back: 531 us in one copy before the pyramid, 492 so).
     // Under capture it stays one copy: a captured batch is a part itself where
-    // uploads are to overlap.
-    bool in_parts = ctx->up_parts > 1 && fits_slot(image_of(0));
+    // uploads are to overlap; with stage timing too, so that the pyramid's time
+    // holds no waits for the upload.
+    bool in_parts = ctx->up_parts > 1 && !ctx->timing && fits_slot(image_of(0));
     for (int img = 1; img < n_img && in_parts; ++img) {
         const jslam_image &cur = image_of(img - 1), &nxt = image_of(img);
         in_parts = fits_slot(nxt) && nxt.data == cur.data + (size_t)cur.pitch * (size_t)cur.height;
