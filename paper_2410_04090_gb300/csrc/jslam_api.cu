@@ -59,6 +59,25 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
     return fn;
 }
 
+// Tensor map of boxes of box_w x box_h bytes of an image plane, written to `to`.
+bool encode_box(void *to, const uint8_t *plane, int W, int H, int pitch, int box_w, int box_h,
+                CUtensorMapL2promotion promote)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+    if (!encode) return false;
+    CUtensorMap map;  // encoded into an aligned object, then copied
+    const cuuint64_t dims[2] = { (cuuint64_t)W, (cuuint64_t)H };
+    const cuuint64_t strides[1] = { (cuuint64_t)pitch };
+    const cuuint32_t box[2] = { (cuuint32_t)box_w, (cuuint32_t)box_h };
+    const cuuint32_t estr[2] = { 1, 1 };
+    if (encode(&map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t *>(plane), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               promote, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+    std::memcpy(to, &map, sizeof(map));
+    return true;
+}
+
 constexpr size_t kLevelSlack = 256;  // bytes after each level buffer
 
 // Optional allocation-failure injection for host-side fault tests: the
@@ -337,10 +356,10 @@ int pyramid_mode_of(const uint32_t *tapx, int W, int src_W)
     return four <= 7 && stride <= kPyrMaxOne ? kPyrOne : two <= 7 && stride <= kPyrMaxTwo ? kPyrTwo : kPyrBytes;
 }
 
-// Build (or reuse) the plan of a batch and upload it.
 // The image after the last one of upload part `part` of a batch of n pairs.
 int upload_end(int n, int part, int parts) { return 2 * (int)((long long)n * (part + 1) / parts); }
 
+// Build (or reuse) the plan of a batch and upload it.
 jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
 {
     const jslam_config &cfg = ctx->cfg;
@@ -435,7 +454,8 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
     const size_t scratch_bytes = slot_words * 4 * 8 + seg_words * 4 * 2 + row_words * 4;
     if ((e = ctx->scratch.ensure(scratch_bytes, false, nullptr)) != cudaSuccess) return fail(ctx, e);
 
-    // Host tables: [images][levels][pairs][pyr base][fast base][seg level][taps/proj ...]
+    // Host tables: images, levels, pairs, segments, pyramid strips, detection
+    // tiles, level starts, tensor maps, taps and projections
     size_t off = 0;
     auto reserve = [&](size_t bytes) { size_t at = off; off = align_up(off + bytes, 256); return at; };
     const size_t o_images = reserve(sizeof(ImageDesc) * n_img);
@@ -573,37 +593,17 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
                 for (int y = 0; y < L.H; ++y) px[L.W + y] = project(y, sc, g.H[0]);
                 t_off += align_up((size_t)(L.W + L.H) * 2, 16);
 
-                // TMA map of the raw level (the box x is rounded down to 16
+                // TMA maps: detection boxes of the raw level, keypoint boxes of
+                // the raw and of the blurred one (their x is rounded down to 16
                 // bytes)
-                L.tmap = nullptr;
-                PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
-                if (encode) {
-                    CUtensorMap map;  // encoded into an aligned object, then copied into the plan
-                    const cuuint64_t dims[2] = { (cuuint64_t)L.W, (cuuint64_t)L.H };
-                    const cuuint64_t strides[1] = { (cuuint64_t)L.pitch };
-                    const cuuint32_t box[2] = { (cuuint32_t)L.box_w, (cuuint32_t)L.box_h };
-                    const cuuint32_t estr[2] = { 1, 1 };
-                    if (encode(&map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, L.raw_w, dims, strides, box, estr,
-                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS) {
-                        std::memcpy(host.data() + o_tmaps + sizeof(CUtensorMap) * li, &map, sizeof(CUtensorMap));
-                        L.tmap = reinterpret_cast<const CUtensorMap *>(dplan + o_tmaps) + li;
-                    }
-                }
-                // keypoint boxes of the raw and the blurred level
-                for (int q = 0; q < 2; ++q) {
-                    CUtensorMap map;
-                    const cuuint64_t dims[2] = { (cuuint64_t)L.W, (cuuint64_t)L.H };
-                    const cuuint64_t strides[1] = { (cuuint64_t)L.pitch };
-                    const cuuint32_t box[2] = { (cuuint32_t)kOrbBoxW, (cuuint32_t)(q ? kOrbBlurH : kOrbRawH) };
-                    const cuuint32_t estr[2] = { 1, 1 };
-                    if (!encode || encode(&map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, q ? L.blur : L.raw_w, dims, strides, box,
-                                          estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                          CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-                        return fail(ctx, cudaErrorNotSupported);
-                    std::memcpy(host.data() + o_omaps + sizeof(CUtensorMap) * (2 * li + q), &map, sizeof(CUtensorMap));
-                }
+                L.tmap = reinterpret_cast<const CUtensorMap *>(dplan + o_tmaps) + li;
+                char *const tm = host.data() + o_tmaps + sizeof(CUtensorMap) * li;
+                char *const om = host.data() + o_omaps + 2 * sizeof(CUtensorMap) * li;
+                if (!encode_box(tm, L.raw_w, L.W, L.H, L.pitch, L.box_w, L.box_h, CU_TENSOR_MAP_L2_PROMOTION_L2_128B) ||
+                    !encode_box(om, L.raw_w, L.W, L.H, L.pitch, kOrbBoxW, kOrbRawH, CU_TENSOR_MAP_L2_PROMOTION_NONE) ||
+                    !encode_box(om + sizeof(CUtensorMap), L.blur, L.W, L.H, L.pitch, kOrbBoxW, kOrbBlurH,
+                                CU_TENSOR_MAP_L2_PROMOTION_NONE))
+                    return fail(ctx, cudaErrorNotSupported);
                 L.slot_base = slot;
                 L.seg_base = seg;
                 for (int r = 0; r < L.cells_y; ++r) {
@@ -652,11 +652,11 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
             R.y0 = R.ccy0 * L.c;
             R.tw = std::min(R.ncx * L.c, L.W - R.x0);
             R.th = std::min(R.ncy * L.c, L.H - R.y0);
-            R.xs = L.tmap ? ((R.x0 - 4) & ~15) : R.x0 - 4;
+            R.xs = (R.x0 - 4) & ~15;
             R.ys = R.y0 - 3;
             R.delta = R.x0 - 4 - R.xs;
             R.c = L.c; R.cells_x = L.cells_x; R.W = L.W; R.H = L.H; R.cinv = L.cinv;
-            R.box_w = L.box_w; R.box_h = L.box_h; R.slot_base = L.slot_base; R.pitch = L.pitch;
+            R.box_w = L.box_w; R.box_h = L.box_h; R.slot_base = L.slot_base;
             R.eps_hi = I.eps_hi; R.eps_lo = I.eps_lo; R.W0 = I.W0;
             R.skip_c0 = I.skip_c0; R.skip_cells_x = I.skip_cells_x;
             // projection ranges, widened to 16-byte boundaries (inside the
@@ -683,7 +683,7 @@ jslam_status build_plan(jslam_ctx *ctx, const jslam_stereo_job *jobs, int n)
             R.ncx_div = recip_of(R.ncx);
             R.all_open = R.x0 + R.c > cfg.border && R.y0 + R.c > cfg.border &&
                          R.x0 + (R.ncx - 1) * R.c < R.W - cfg.border && R.y0 + (R.ncy - 1) * R.c < R.H - cfg.border;
-            R.raw = L.raw; R.tmap = L.tmap; R.map = I.map; R.skip = I.skip;
+            R.tmap = L.tmap; R.map = I.map; R.skip = I.skip;
         }
     }
     // Tile order 1: the persistent detection CTAs take the records in order;

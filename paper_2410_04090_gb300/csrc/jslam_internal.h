@@ -90,7 +90,7 @@ struct LevelDesc {
     int32_t c, cells_x, cells_y;
     int32_t bx, by;          // cells per detection tile
     int32_t cinv;            // ceil(2^16 / c): exact division by c for values < 128
-    const CUtensorMap *tmap; // TMA map of the raw level (nullptr: tiles loaded with plain loads)
+    const CUtensorMap *tmap; // TMA map of the raw level
     int32_t box_w, box_h;    // detection tile box: bytes per row (multiple of 16) and rows
     int32_t slot_base;       // first candidate slot of the level
     int32_t seg_base;        // first segment (cell row) of the level
@@ -154,7 +154,6 @@ struct Inputs {
     int32_t pitch[kMaxImages];
 };
 
-// Everything the kernels of one extraction need.
 // One detection tile, prepared on the host: the
 // tile's place in its level, the level's and image's scalars, and the
 // 16-byte-aligned ranges of the level's s0 projection tables that cover the
@@ -163,7 +162,7 @@ struct Inputs {
 constexpr int kPrjBytes = 288;  // staged projection bytes per axis: 2 x 128 + alignment slack, rounded to 16
 struct __align__(16) TileRec {
     int32_t ccx0, ccy0, ncx, ncy, x0, y0, tw, th, xs, ys, delta;
-    int32_t c, cells_x, W, H, cinv, box_w, box_h, slot_base, pitch;
+    int32_t c, cells_x, W, H, cinv, box_w, box_h, slot_base;
     int32_t eps_hi, eps_lo, W0, skip_c0, skip_cells_x;
     int32_t prj_bytes_x, prj_bytes_y;  // bulk copy sizes (multiples of 16)
     int32_t prj_off_x, prj_off_y;      // element offset of x0 / y0 in the staged copies
@@ -173,9 +172,7 @@ struct __align__(16) TileRec {
     uint32_t nch_inv, row_inv;         // ceil(2^16 / nch), ceil(2^16 / (nch + 1))
     uint32_t cdiv, ncx_div;            // reciprocals of c and ncx (see div_recip)
     int32_t all_open;                  // every cell has evaluated pixels
-    int32_t pad[1];
-    const uint8_t *raw;
-    const CUtensorMap *tmap;           // nullptr: the box is loaded with plain loads
+    const CUtensorMap *tmap;
     const uint16_t *prj_src_x, *prj_src_y;
     uint32_t *map;
     const uint8_t *skip;
@@ -202,6 +199,7 @@ struct __align__(16) PyrRec {
 // Rank of a slot that is no survivor (SlotInfo's w): no corner, suppressed.
 constexpr int kSlotEmpty = -2, kSlotSuppressed = -1;
 
+// Everything the kernels of one extraction need.
 struct Batch {
     const ImageDesc *images;
     const LevelDesc *levels;

@@ -397,19 +397,18 @@ __device__ __forceinline__ void fetch_rec(const Batch &b, int t, TileRec *dst, u
                  "r"((uint32_t)sizeof(TileRec)), "r"(smem_u32(bar)) : "memory");
 }
 
-// The tile box (TMA, levels with a tensor map) and the tile's projection
-// ranges (bulk copies) of record R, all completing on `bar`.
+// The tile box (TMA) and the tile's projection ranges (bulk copies) of record
+// R, all completing on `bar`.
 __device__ __forceinline__ void issue_rec_tile(const TileRec &R, uint8_t *buf, uint8_t *prj, uint64_t *bar)
 {
-    const uint32_t box = R.tmap ? (uint32_t)(R.box_w * R.box_h) : 0u;
+    const uint32_t box = (uint32_t)(R.box_w * R.box_h);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
                  "r"(box + (uint32_t)(R.prj_bytes_x + R.prj_bytes_y)) : "memory");
-    if (R.tmap)
-        asm volatile(
-            "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-            ::"r"(smem_u32(buf)), "l"(reinterpret_cast<uint64_t>(R.tmap)), "r"(R.xs), "r"(R.ys), "r"(smem_u32(bar))
-            : "memory");
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(smem_u32(buf)), "l"(reinterpret_cast<uint64_t>(R.tmap)), "r"(R.xs), "r"(R.ys), "r"(smem_u32(bar))
+        : "memory");
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_u32(prj)), "l"(reinterpret_cast<uint64_t>(R.prj_src_x)), "r"((uint32_t)R.prj_bytes_x),
                  "r"(smem_u32(bar)) : "memory");
@@ -529,8 +528,7 @@ __global__ void __launch_bounds__(kFastThreads, kFastCtasPerSm) k_fast_bits(cons
             s_more[cur] = t1 < tiles;
         }
         uint8_t *const tb = cur ? buf1 : buf0;
-        // the box and the projections (every tile waits: the projections
-        // come on the same barrier whether or not the box does)
+        // the box and the projections
         if (!wait_tile(&bars[cur], (phases >> cur) & 1u)) {
             if (threadIdx.x == 0) {
                 atomicOr(b.err, kErrTimeout);
@@ -549,21 +547,6 @@ __global__ void __launch_bounds__(kFastThreads, kFastCtasPerSm) k_fast_bits(cons
         // image with none takes the exact path: no per-cell flags, no extra
         // barrier)
         const bool tskip = kSkip && R.skip != nullptr && b.skip_any[R.image] != 0;
-        if (!R.tmap) {
-            // levels whose tiles cannot start on a word boundary: plain loads
-            // (box rows of box_w bytes, delta = 0)
-            const int wpr = rowb >> 2;
-            uint32_t *tw32 = reinterpret_cast<uint32_t *>(tb);
-            for (int i = threadIdx.x; i < R.box_h * wpr; i += kFastThreads) {
-                const int r = i / wpr, wi = i - r * wpr;
-                const uint8_t *row = R.raw + (size_t)min(max(R.ys + r, 0), Hh - 1) * R.pitch;
-                const int gx = R.xs + 4 * wi;
-                uint32_t v = 0;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) v |= (uint32_t)row[min(max(gx + q, 0), W - 1)] << (8 * q);
-                tw32[i] = v;
-            }
-        }
         // cell states and cleared selections.  State: 0 no corner yet, 1
         // primary-threshold corner, 2 skipped by the learned proposal (its
         // centre projects into a skipped s0 cell), 3 no pixel inside the
@@ -590,9 +573,9 @@ __global__ void __launch_bounds__(kFastThreads, kFastCtasPerSm) k_fast_bits(cons
         for (int i = threadIdx.x; i < (cells * k + 3) >> 2; i += kFastThreads)
             reinterpret_cast<uint4 *>(sel)[i] = make_uint4(0u, 0u, 0u, 0u);
         if (my_skipped) atomicAdd(&s_skipped[cur], my_skipped);
-        // a box loaded with plain loads, the cell states and, in skip mode,
-        // the skipped count are complete before the planes
-        if (!R.tmap || tskip) __syncthreads();
+        // in skip mode the cell states and the skipped count are complete
+        // before the planes
+        if (tskip) __syncthreads();
         all_skipped = tskip && s_skipped[cur] == cells;
 
         // bit-planes of the box rows [r0, r1 + 6) that the evaluated rows
