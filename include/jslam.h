@@ -401,7 +401,9 @@ jslam_status jslam_stage_times(jslam_ctx *ctx, float *ms /* JSLAM_NUM_STAGES ent
  * whole culling cells, and every kernel variant computes the same outputs.
  * The default tile, 128 x 64, stands for tile heights that follow the batch
  * and tiles in order of decreasing work, whatever tile_order says; setting the
- * defaults is the same as setting nothing, and the way back from a tuning. */
+ * defaults is the same as setting nothing, and the way back from a tuning.
+ * Those heights suit a batch alone on the GPU; contexts that run beside each
+ * other do better with tall tiles (128 x 65, order 1). */
 typedef struct {
     int32_t tile_w_px;           /* detection tile width, at most: 32..128, multiple of 4 (default 128) */
     int32_t tile_h_px;           /* detection tile height, about (up to half as much again): 8..128 (default 64) */
@@ -423,14 +425,13 @@ typedef struct {
 jslam_status jslam_set_tuning(jslam_ctx *ctx, const jslam_tuning *t);
 
 /* Tune the launch shapes on the batch `jobs` (n pairs, as for
- * jslam_extract_batch), timing the stages with the stage events: the
+ * jslam_extract_batch), timing extractions enqueued back to back: the
  * detection tile among six shapes, the default first, then the number of
  * persistent detection CTAs per SM, then (when every segment fits a warp) the
- * NMS kernel, then the tile order of a tile that is not the default, then the
- * pick for detection against the default once more.  Keeps
+ * NMS kernel, then the tile order of a tile that is not the default.  Keeps
  * the fastest for the context and returns it in *out (may be NULL); a call
  * that fails leaves tuning and stage timing as they were.  Runs the
- * batch several times; results are unaffected.  No counterpart in the paper
+ * batch some hundred times; results are unaffected.  No counterpart in the paper
  * (an autotuner in place of the fixed thread allocation of Sec. II-C-1). */
 jslam_status jslam_autotune(jslam_ctx *ctx, const jslam_stereo_job *jobs, int32_t n, jslam_tuning *out);
 
@@ -462,7 +463,7 @@ jslam_status jslam_tune_key(const char *gpu_name, int32_t sm_count, const jslam_
 jslam_status jslam_tune_cache_get(const char *path, const char *key, jslam_tuning *out, int32_t *found);
 
 /* Add or replace the entry of `key` in the tuning cache file (host only),
- * with the tuned stage time for reference; the file is rewritten through a
+ * with the time of a tuned call for reference; the file is rewritten through a
  * temporary file and a rename.  JSLAM_ERR_ARG for an invalid tuning, a key
  * holding a quote or backslash, or a file that cannot be written.  No
  * counterpart in the paper. */

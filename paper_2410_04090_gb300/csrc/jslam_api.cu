@@ -265,7 +265,7 @@ struct jslam_ctx {
     // generation of the plan: bumped whenever build_plan rebuilds the tables
     // or buffers, which invalidates a graph captured on an earlier plan
     uint64_t plan_gen = 0;
-    float tune_ms = 0.0f;  // detection stage time of the last autotuned pick
+    float tune_ms = 0.0f;  // time of a call with the last autotuned pick
 };
 
 namespace {
@@ -1610,18 +1610,26 @@ jslam_status jslam_set_tuning(jslam_ctx *ctx, const jslam_tuning *t)
 
 namespace {
 
-// Median-free minimum of a stage's time over `reps` runs of the batch (the
-// first run of a new tuning also rebuilds the plan and is not counted).
-jslam_status time_stage(jslam_ctx *ctx, const jslam_stereo_job *jobs, int32_t n, int stage, int reps, float *best)
+// Device time of one extraction of the batch among others, back to back: the
+// least of some rounds of calls (the first round of a new tuning also rebuilds
+// the plan and is not counted).  Whole calls, since a stage by itself says
+// little: its launch may start while the one before still runs, or not, by how
+// many tiles there are (one pair of 752x480: tiles of 128 x 65 take 2 us longer
+// than the default's in the detection stage, and the call 52 us, not 59).
+jslam_status time_calls(jslam_ctx *ctx, const jslam_stereo_job *jobs, int32_t n, float *best)
 {
+    constexpr int kRounds = 5, kCalls = 6;
     *best = -1.0f;
-    for (int rep = 0; rep <= reps; ++rep) {
-        jslam_status st = jslam_extract_batch(ctx, jobs, n);
+    for (int round = 0; round <= kRounds; ++round) {
+        cudaError_t e = cudaEventRecord(ctx->events[0], ctx->stream);
+        jslam_status st = fail(ctx, e);
+        for (int i = 0; st == JSLAM_OK && i < kCalls; ++i) st = jslam_extract_batch(ctx, jobs, n);
+        if (st == JSLAM_OK) st = fail(ctx, cudaEventRecord(ctx->events[1], ctx->stream));
         if (st == JSLAM_OK) st = jslam_sync(ctx);
-        float ms[JSLAM_NUM_STAGES];
-        if (st == JSLAM_OK) st = jslam_stage_times(ctx, ms);
+        float ms = 0.0f;
+        if (st == JSLAM_OK) st = fail(ctx, cudaEventElapsedTime(&ms, ctx->events[0], ctx->events[1]));
         if (st != JSLAM_OK) return st;
-        if (rep > 0 && (*best < 0 || ms[stage] < *best)) *best = ms[stage];
+        if (round > 0 && (*best < 0.0f || ms < *best * kCalls)) *best = ms / kCalls;
     }
     return JSLAM_OK;
 }
@@ -1634,81 +1642,40 @@ jslam_status jslam_autotune(jslam_ctx *ctx, const jslam_stereo_job *jobs, int32_
     if (ctx->status != JSLAM_OK) return ctx->status;
     const bool was_timing = ctx->timing;
     const jslam_tuning before = ctx->tune;
-    jslam_status st = jslam_enable_stage_timing(ctx, 1);
+    jslam_status st = jslam_enable_stage_timing(ctx, 1);  // creates the events
     if (st != JSLAM_OK) return st;
+    ctx->timing = false;
     jslam_tuning best{};
-    // 1. the detection tile
     float best_ms = -1.0f;
-    for (const auto &tl : kTuneTiles) {
-        ctx->tune = best;
-        ctx->tune.tile_w_px = tl[0];
-        ctx->tune.tile_h_px = tl[1];
+    // the batch with tuning t, kept if it is faster by more than runs of one
+    // tuning differ (about 1 %)
+    const auto attempt = [&](const jslam_tuning &t) {
+        ctx->tune = t;
         float ms;
-        if ((st = time_stage(ctx, jobs, n, JSLAM_STAGE_DETECT, 3, &ms)) != JSLAM_OK) break;
-        if (best_ms < 0 || ms < best_ms) {
+        if (st != JSLAM_OK || (st = time_calls(ctx, jobs, n, &ms)) != JSLAM_OK) return;
+        if (best_ms < 0.0f || ms < 0.99f * best_ms) {
             best_ms = ms;
-            best.tile_w_px = tl[0];
-            best.tile_h_px = tl[1];
+            best = t;
         }
-    }
+    };
+    // 1. the detection tile: the default, then fixed ones, taken by decreasing work
+    for (const auto &tl : kTuneTiles) attempt({ tl[0], tl[1], 0, 0, default_tile(tl[0], tl[1]) ? 0 : 1 });
     // 2. fewer persistent detection CTAs per SM than fit (one less, then two)
     int fit = 0;
     if (st == JSLAM_OK) {
         ctx->tune = best;
         if ((st = jslam_extract_batch(ctx, jobs, n)) == JSLAM_OK) st = jslam_sync(ctx);
-        if (st == JSLAM_OK) {
-            const cudaError_t e = detect_ctas_that_fit(ctx->batch, &fit);
-            if (e != cudaSuccess) st = fail(ctx, e);
-        }
+        if (st == JSLAM_OK) st = fail(ctx, detect_ctas_that_fit(ctx->batch, &fit));
     }
-    for (int c = fit - 1; st == JSLAM_OK && c >= 1 && c >= fit - 2; --c) {
-        ctx->tune = best;
-        ctx->tune.detect_ctas_per_sm = c;
-        float ms;
-        if ((st = time_stage(ctx, jobs, n, JSLAM_STAGE_DETECT, 3, &ms)) != JSLAM_OK) break;
-        if (ms < best_ms) { best_ms = ms; best.detect_ctas_per_sm = c; }
-    }
+    const jslam_tuning tile = best;
+    for (int c = fit - 1; st == JSLAM_OK && c >= 1 && c >= fit - 2; --c)
+        attempt({ tile.tile_w_px, tile.tile_h_px, 0, c, tile.tile_order });
     // 3. the NMS kernel, where the warp-per-segment variant applies
-    if (st == JSLAM_OK && ctx->batch.max_segment <= 96) {
-        float nms_ms[2] = { -1.0f, -1.0f };
-        for (int v = 0; v < 2 && st == JSLAM_OK; ++v) {
-            ctx->tune = best;
-            ctx->tune.nms_kernel = v;
-            st = time_stage(ctx, jobs, n, JSLAM_STAGE_PFA_NMS, 3, &nms_ms[v]);
-        }
-        if (st == JSLAM_OK) best.nms_kernel = nms_ms[1] < nms_ms[0] ? 1 : 0;
-    }
-    // 4. the tile order (a replan each), against the detection time of the
-    // pick so far; the default tile has its own
-    if (st == JSLAM_OK && !default_tile(best.tile_w_px, best.tile_h_px)) {
-        ctx->tune = best;
-        ctx->tune.tile_order = 1;
-        float ms;
-        if ((st = time_stage(ctx, jobs, n, JSLAM_STAGE_DETECT, 3, &ms)) == JSLAM_OK && ms < best_ms) {
-            best_ms = ms;
-            best.tile_order = 1;
-        }
-    }
-    // 5. the pick against the default once more, over more runs: the events
-    // resolve about 2 us, as much as the tiles of one small pair differ by
-    if (st == JSLAM_OK && (!default_tile(best.tile_w_px, best.tile_h_px) || best.detect_ctas_per_sm != 0)) {
-        float ms[2] = { -1.0f, -1.0f };
-        for (int v = 0; v < 2 && st == JSLAM_OK; ++v) {
-            ctx->tune = best;
-            if (v == 0) {
-                ctx->tune.tile_w_px = kDefaultTileW;
-                ctx->tune.tile_h_px = kDefaultTileH;
-                ctx->tune.detect_ctas_per_sm = ctx->tune.tile_order = 0;
-            }
-            st = time_stage(ctx, jobs, n, JSLAM_STAGE_DETECT, 12, &ms[v]);
-        }
-        best_ms = std::min(ms[0], ms[1]);
-        if (st == JSLAM_OK && ms[1] >= ms[0]) {
-            best.tile_w_px = kDefaultTileW;
-            best.tile_h_px = kDefaultTileH;
-            best.detect_ctas_per_sm = best.tile_order = 0;
-        }
-    }
+    if (st == JSLAM_OK && ctx->batch.max_segment <= 96)
+        attempt({ best.tile_w_px, best.tile_h_px, 1, best.detect_ctas_per_sm, best.tile_order });
+    // 4. a fixed tile in plan order
+    if (st == JSLAM_OK && !default_tile(best.tile_w_px, best.tile_h_px))
+        attempt({ best.tile_w_px, best.tile_h_px, best.nms_kernel, best.detect_ctas_per_sm, 0 });
     // a failed tuning leaves the context as it was
     ctx->tune = st == JSLAM_OK ? best : before;
     ctx->timing = was_timing;

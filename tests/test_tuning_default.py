@@ -82,30 +82,36 @@ def test_a_failed_tuning_changes_nothing(J, oracle, bad):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("width,height,levels", [(320, 240, 4), (640, 480, 8), (752, 480, 8), (1241, 376, 8)])
-def test_a_tuned_batch_is_not_slower(J, oracle, width, height, levels):
-    """Detection of the tuner's pick within the events' resolution (about 2 us
-    here) of the default's."""
+@pytest.mark.parametrize("width,height,levels,pairs", [(320, 240, 4, 1), (640, 480, 8, 1), (752, 480, 8, 1),
+                                                       (1241, 376, 8, 1), (640, 480, 1, 12)])
+def test_a_tuned_batch_is_not_slower(J, oracle, width, height, levels, pairs):
+    """Calls back to back with the tuner's pick take no longer than untuned
+    ones, but for 3 %: rounds of 40 calls on one context differ by 1 to 2."""
     import torch
     p = params_from(oracle, levels=levels, max_feats=800, fast_thresh_lo=7)
     f = scenes.planes_pair(width, height, 0, 3, 4)
     img = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (f.left, f.right)]
     torch.cuda.synchronize()
-    fe = frontend_for(J, p, max_width=width, max_height=height, max_pairs=1)
-    jobs = [J.Job(*img, levels=levels, max_feats=800)]
+    stream = torch.cuda.Stream()
+    plain, tuned = [frontend_for(J, p, max_width=width, max_height=height, max_pairs=pairs, stream=stream) for _ in range(2)]
+    jobs = [J.Job(*img, levels=levels, max_feats=800)] * pairs
+    pick = tuned.autotune(jobs)
 
-    def detect_us():
-        fe.enable_stage_timing(True)
-        t = []
-        for _ in range(60):
-            fe.extract_batch(jobs)
-            fe.sync()
-            t.append(1e3 * fe.stage_times()["detect"])
-        fe.enable_stage_timing(False)
-        return float(np.median(t))
+    def call_us(fe):
+        batch = fe.prepare_batch(jobs)
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        fe.extract_batch(batch)
+        fe.sync()
+        e0.record(stream)
+        for _ in range(40):
+            fe.extract_batch(batch)
+        e1.record(stream)
+        fe.sync()
+        e1.synchronize()
+        return 1e3 * e0.elapsed_time(e1) / 40
 
-    before = detect_us()
-    pick = fe.autotune(jobs)
-    tuned = detect_us()
-    assert tuned <= before + 2.5, (pick, before, tuned)
-    fe.close()
+    rounds = [(call_us(plain), call_us(tuned)) for _ in range(7)]
+    a, b = (float(np.median(r)) for r in zip(*rounds))
+    assert b <= 1.03 * a, (pick, a, b)
+    plain.close()
+    tuned.close()
