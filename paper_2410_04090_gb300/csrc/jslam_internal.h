@@ -298,7 +298,8 @@ int skipnet_smem_bytes();
 // 320x240 76 / 69 / 66, of 1241x376 with refinement and tracking 126 / 115 /
 // 105, of 1920x1080 143 / 142 / 142; 100 of 1241x376 1251 / 1258 / 1348, 16
 // streams of four sizes 375 / 368 / 415, 24 pairs of 647x363 343 / 338 / 381, 16
-// of 800x602 on a cascaded pyramid 390 / 373 / 502.
+// of 800x602 on a cascaded pyramid 390 / 373 / 502 (before detection of the last
+// two became faster; they take 239 and 325 now).
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

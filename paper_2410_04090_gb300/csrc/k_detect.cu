@@ -443,11 +443,11 @@ __device__ __forceinline__ void drain_bits(uint64_t *bars, bool more, int cur, i
 // write this one's slots (what the next tile's first phase overwrites -- the
 // planes, the other set -- was last read before the barrier that ended this
 // tile's passes, and what thread 0 refills, before the next one's first).
-// What bounds it: the ALU pipe (LOP3 and shifts, half rate: 60 % busy) and the
+// What bounds it: the ALU pipe (LOP3 and shifts, half rate: 69 % busy) and the
 // barriers and dependent steps between.  Four warps a CTA, five CTAs an SM (96
 // registers): with eight warps and three CTAs a barrier stopped more of the
 // SM.  For 100 pairs of 1241x376 the kernel executed 1750 instructions per
-// 1024 pixels and took 0.965 ms; now 1430 and 0.585 ms (threads and barriers
+// 1024 pixels and took 0.965 ms; now 1420 and 0.577 ms (threads and barriers
 // 0.965 -> 0.82, run test and registers -> 0.765, host-made tile numbers,
 // reciprocals and whole-word clears -> 0.729, blocks of cells that fill the
 // warps -> 0.692, tiles from a counter -> 0.596, largest first -> 0.585).

@@ -73,7 +73,8 @@ __device__ __forceinline__ void orb_box(const CUtensorMap *map, const uint8_t *t
 // moments -> sector -> pattern -> patch, 32 warps an SM).  Reading disk and
 // patch with plain loads touches a line per row, 75 of the 170 load
 // wavefronts a keypoint took, and those bounded it: 400 000 keypoints 0.260 ms
-// with one warp each and 563 instructions a keypoint; 0.205 ms now, with 328.
+// with one warp each and 563 instructions a keypoint; 0.211 ms now, with 345
+// (0.205 and 328 without the row index, which the finalisation wrote then).
 // A warp takes keypoints i, i + stride, ... of its image.
 __global__ void __launch_bounds__(32 * kOrbWarps) k_orient_desc(const __grid_constant__ Batch b)
 {
@@ -278,7 +279,7 @@ cudaError_t launch_orient_desc(const Batch &b, cudaStream_t stream)
 // most, of which a good part lies outside the search range.  What bounds it:
 // the chain of gathers from L2 (keypoint -> row index -> X -> descriptor);
 // eight CTAs an SM hide most of it.  200 000 left keypoints: 0.121 ms with a
-// warp each, 0.072 now (0.078 with six CTAs an SM).
+// warp each, 0.068 now (six CTAs an SM cost 8 % more).
 __global__ void __launch_bounds__(256, 8) k_match(const __grid_constant__ Batch b)
 {
     const PairDesc &P = b.pairs[blockIdx.y];

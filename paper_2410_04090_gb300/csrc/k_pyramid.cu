@@ -29,9 +29,9 @@
 // strip is 30 lanes x 4 columns wide; a strip computes six rows more than it
 // writes, three above and three below (see pyramid_strip_rows for how tall).
 //
-// What bounds it: instruction issue (76 % of the slots, 110 instructions per
-// strip row; DRAM at 10 %, a pixel of the pyramid being two bytes written).
-// For 100 pairs of 1241x376 with 8 levels it takes 0.337 ms; a CTA per
+// What bounds it: instruction issue (77 % of the slots, 110 instructions per
+// strip row; DRAM at 31 %, a pixel of the pyramid being two bytes written).
+// For 100 pairs of 1241x376 with 8 levels it takes 0.333 ms; a CTA per
 // 128 x 32 tile, with byte gathers and three shared-memory stages between
 // barriers, executed 72 instructions per pixel and took 0.740 ms.  One pair
 // (10 rows a strip): 16.2 us, before 19.6.
