@@ -670,10 +670,11 @@ __global__ void __launch_bounds__(kFastThreads, kFastCtasPerSm) k_fast_bits(cons
                     uint32_t valid = border_bits(px0, plo, phi);
                     if (listed && valid) {
                         const uint8_t *strow = has_hi + div_small(py, cinv) * ncx;
-                        if (pass == 1)  // only cells without a corner (and not skipped)
-                            valid &= cell_bits(strow, px0, tw, c, cinv, [](uint8_t st) { return st == 0; });
-                        else            // not in a skipped cell
-                            valid &= cell_bits(strow, px0, tw, c, cinv, [](uint8_t st) { return st != 2; });
+                        // pass 1: only cells without a corner (and not skipped); pass 0: not in a
+                        // skipped cell.  One copy of the loop for both spills less in the skip mode
+                        // (12 pairs of 752x480 213.0 -> 211.4 us).
+                        valid &= cell_bits(strow, px0, tw, c, cinv,
+                                           [=](uint8_t st) { return pass == 1 ? st == 0 : st != 2; });
                     }
                     if (valid) bits = bs_corners<kAny>(planes, ru, py, m, sb, eps_mask, b.prm.p_min, b.prm.p_max) & valid;
                 }
